@@ -271,17 +271,10 @@ int fwi_gradient_lanes(fwi_batch* b, double* grad_out, double* misfit_out, void*
  * FWI_EINVAL. The batch's device memory is sized for the per-shot form either way. */
 int fwi_batch_set_gradient_lanes(fwi_batch* b, int per_shot);
 
-/* Trades memory for arithmetic in the gradient steps (Eq. gradient3), for triangles in the
- * chunked layout with a multiple of 4 shots, the summed gradient form and tensor_cores off
- * (elsewhere the setting has no effect). With on = 1 the forward recompute of each adjoint
- * segment also stores, per element, node, shot and direction, the forward field's
- * (Ghat grad u) at the gradient levels, and the gradient steps read it back instead of
- * contracting the forward field again (one more recompute step per segment gives the last
- * level). The store takes (ckpt_stride / grad_stride) x (chunks without damping-layer
- * elements) x (S / 4) x (nodes per element) x 1 KB of device memory, allocated by the
- * next fwi_adjoint_* call (FWI_ENOMEM if it does not fit) and not counted by
- * fwi_batch_bytes; on = 0 frees it. The results equal those without the store up to FP32
- * summation order. */
+/* Accepted for callers that set it (on = 0 or 1, anything else FWI_EINVAL); has no effect. It
+ * used to make the recompute store the forward field's gradients for the gradient steps. With
+ * the derivatives in symmetry-adapted coordinates a second contraction of the forward field
+ * costs less than writing and reading its stored gradients, so no step keeps them. */
 int fwi_batch_set_gradient_store(fwi_batch* b, int on);
 
 /* Per-kernel timing (tracing): when enabled, every time step of the batch's forward,

@@ -13,7 +13,9 @@ LIB = os.path.join(OUT, "libfwi_gb300.so")
 # KMV element (triangles k = 2..5, tetrahedra k = 2, 3)
 UNITS = [("kmv_tab.cpp", "kmv_tab", []), ("api.cu", "api", []), ("kernels.cu", "kernels", [])] + [
     ("inst.cu", f"inst_{d}_{k}", [f"-DKMV_DIM={d}", f"-DKMV_K={k}"])
-    for d, k in ((2, 2), (2, 3), (2, 4), (2, 5), (3, 2), (3, 3))]
+    for d, k in ((2, 2), (2, 3), (2, 4), (2, 5), (3, 2), (3, 3))] + [
+    ("sym_inst.cu", f"sym_{d}_{k}_{g}", [f"-DKMV_DIM={d}", f"-DKMV_K={k}", f"-DKMV_SG={g}"])
+    for d, k in ((3, 3), (2, 5), (3, 2), (2, 4), (2, 3), (2, 2)) for g in (4, 2, 1)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2"]
 

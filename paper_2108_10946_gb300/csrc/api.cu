@@ -45,7 +45,8 @@ template <class T>
 int dalloc(T** p, size_t count) {
   *p = nullptr;
   if (count == 0) return 0;
-  cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
+  // 16 bytes to spare: the kernels' bulk copies move whole 16-byte groups
+  cudaError_t e = cudaMalloc((void**)p, count * sizeof(T) + 16);
   if (e != cudaSuccess) {
     *p = nullptr;
     cudaGetLastError();  // an allocation failure is not sticky: clear it for later checks
@@ -127,6 +128,11 @@ struct fwi_mesh {
   std::vector<int32_t> ch_e0, ch_own_lo, ch_nsh;  // chunk element ranges, owned ranges
   std::vector<int32_t> ch_halo_ptr, halo_ids;     // per-chunk halo lists (global DoF ids)
   std::vector<uint16_t> lconn;                    // [ns][E] chunk-local index of shared nodes
+  // symmetry-adapted chunk kernels: descriptors, tables (positions, incidence lists)
+  std::vector<int32_t> sdesc;                     // [nch][8]
+  std::vector<uint16_t> smeta;
+  int T_max = 0, SH_max = 0;
+  int p_own = 0, p_halo = 0;  // layer index of an owned / halo DoF of the layer: DoF - shift
   std::vector<double> verts;
   std::vector<int32_t> cells;      // user order
   std::vector<int32_t> order;      // new element -> user element
@@ -154,6 +160,11 @@ struct fwi_mesh {
   int* d_chunks = nullptr;   // [nch][6]: e0, ne, own_lo, own_n, nsh, halo_ptr
   int* d_halo = nullptr;     // halo DoF ids, chunk by chunk
   unsigned short* d_lconn = nullptr;
+  int* d_sdesc = nullptr;
+  unsigned short* d_smeta = nullptr;
+  float* d_lpsi = nullptr;            // nodal layer coefficients, [Nl] (2D) or [Nl][4]
+  float* d_lcs = nullptr;             // the update's layer coefficients, [Nl][8 or 12]
+  unsigned char* d_splain = nullptr;  // [nch] set with the velocity
   int nch() const { return (int)ch_e0.size() - 1; }
 };
 
@@ -197,9 +208,6 @@ struct fwi_batch {
   int tc_wait_limit = 1 << 22;  // polls of each bounded wait of the tensor-core kernel
   int grad_lanes = 0;           // 1: the next adjoint keeps each shot's gradient apart
   int acc_lanes = -1;           // what the accumulators hold: -1 nothing, 0 summed, 1 per shot
-  int gstore_on = 0;            // store the forward field's gradients during the recompute
-  float* gring = nullptr;       // [levels][gstore_level_floats] (allocated at first use)
-  size_t gring_level = 0;       // floats per level
   // optional per-kernel timing with CUDA events (fwi_profile)
   bool prof = false;
   std::vector<cudaEvent_t> ev;
@@ -229,9 +237,11 @@ int ensure_constants(fwi_mesh* m) {
   std::lock_guard<std::mutex> lk(mu);
   for (auto& d : done)
     if (d[0] == m->device && d[1] == m->dim && d[2] == m->k) return 0;
-  std::vector<float> dh, w;
+  std::vector<float> dh, w, sym;
   kmvtab::fp32_tables(m->el, dh, w);
-  int e = m->ks->upload_constants(dh.data(), w.data());
+  std::string err;
+  if (!kmvtab::sym_tables(m->el, sym, err)) return fail(FWI_EINVAL, "KMV tabulation: " + err);
+  int e = m->ks->upload_constants(dh.data(), w.data(), sym.data(), (int)sym.size());
   if (e != 0) return fail(FWI_ECUDA, std::string("constant upload: ") + cudaGetErrorString((cudaError_t)e));
   done.push_back({m->device, m->dim, m->k});
   return 0;
@@ -512,6 +522,42 @@ int64_t fwi_launch_count(void) {
 }  // extern "C"
 
 namespace {
+// Tables of the symmetry-adapted chunk kernels, one block per chunk: the position of each shared
+// node in the chunk's table, and per shared DoF (owned, then halo) the list of its (node, element)
+// places in element order.
+void build_incidence(fwi_mesh* m) {
+  const int P = fwi::sym_pe(m->dim, m->nn), ns = m->ns, nch = m->nch();
+  m->smeta.clear();
+  m->sdesc.assign((size_t)nch * 8, 0);
+  std::vector<int> cnt;
+  for (int c = 0; c < nch; ++c) {
+    const int e0 = m->ch_e0[c], ne = m->ch_e0[c + 1] - e0;
+    const int own = m->ch_own_lo[c], own_n = m->ch_own_lo[c + 1] - own, nsh = m->ch_nsh[c];
+    const int hp = m->ch_halo_ptr[c], hn = m->ch_halo_ptr[c + 1] - hp, nloc = nsh + hn;
+    const size_t at = m->smeta.size(), size = (size_t)2 * ns * P + (nloc + 8) / 8 * 8;
+    m->smeta.resize(at + size, 0);
+    uint16_t *lq = &m->smeta[at], *ge = lq + ns * P, *gp = ge + ns * P;
+    auto place = [&](int q, int e) {  // list of node q of element e
+      const int l = m->lconn[(size_t)q * m->Es + e];
+      return l < nsh ? l : l - (own_n - nsh);
+    };
+    cnt.assign(nloc + 1, 0);
+    for (int q = 0; q < ns; ++q)
+      for (int e = e0; e < e0 + ne; ++e) {
+        lq[q * P + e - e0] = m->lconn[(size_t)q * m->Es + e];
+        cnt[place(q, e) + 1]++;
+      }
+    for (int l = 0; l < nloc; ++l) cnt[l + 1] += cnt[l];
+    for (int l = 0; l <= nloc; ++l) gp[l] = (uint16_t)cnt[l];
+    for (int e = e0; e < e0 + ne; ++e)
+      for (int q = 0; q < ns; ++q) ge[cnt[place(q, e)]++] = (uint16_t)(q * P + e - e0);
+    const int d[8] = {e0, ne, own, nsh, hp, hn, (int)(at / 2), (int)(size / 2)};
+    std::copy(d, d + 8, &m->sdesc[(size_t)c * 8]);
+    m->T_max = std::max(m->T_max, own_n + hn);
+    m->SH_max = std::max(m->SH_max, nloc);
+  }
+}
+
 int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64_t ncells,
                 const fwi_params* params, bool host_only, fwi_mesh** out) {
   if (!verts || !cells || !params || !out || nverts <= 0 || ncells <= 0)
@@ -533,10 +579,12 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
   m->k = params->k;
   m->ks = ks;
   m->layout = params->layout == 1 ? 1 : 0;
-  m->P = d == 2 ? 32 : 16;
   if (params->tensor_cores > 0 && (d != 2 || m->layout != 0))
     return fail(FWI_EINVAL, "tensor_cores = 1 needs triangles and the chunked layout");
   m->use_tc = d == 2 && m->layout == 0 && params->tensor_cores > 0;
+  // elements per chunk: the kernels' most where that still gives every SM two chunks
+  m->P = 32;
+  if (!m->use_tc && ncells >= (int64_t)304 * fwi::sym_pe(d, ks->nn)) m->P = fwi::sym_pe(d, ks->nn);
   if (!host_only) CUDA_TRY(cudaGetDevice(&m->device));
   std::string err;
   if (!kmvtab::build(d, params->k, m->el, err)) return fail(FWI_EINVAL, "KMV tabulation: " + err);
@@ -674,11 +722,13 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
     int32_t cur = 0;
     for (int c = 0; c < nch; ++c) {
       m->ch_own_lo[c] = cur;
-      for (int e = m->ch_e0[c]; e < m->ch_e0[c + 1]; ++e)
-        for (int q = 0; q < m->ns; ++q) {
-          int pid = m->conn[(size_t)e * n + q];
-          if (!halo[pid] && fin[pid] < 0) fin[pid] = cur++;
-        }
+      // vertices first: their incidence lists are the long ones, so a warp sees one kind
+      for (int part = 0; part < 2; ++part)
+        for (int e = m->ch_e0[c]; e < m->ch_e0[c + 1]; ++e)
+          for (int q = part ? d + 1 : 0; q < (part ? m->ns : d + 1); ++q) {
+            int pid = m->conn[(size_t)e * n + q];
+            if (!halo[pid] && fin[pid] < 0) fin[pid] = cur++;
+          }
       m->ch_nsh[c] = cur - m->ch_own_lo[c];
       for (int e = m->ch_e0[c]; e < m->ch_e0[c + 1]; ++e) {
         m->bub[e] = cur;
@@ -711,8 +761,8 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
     for (int c = 0; c < nch; ++c) {
       hmap.clear();
       const int own_lo = m->ch_own_lo[c], own_n = m->ch_own_lo[c + 1] - own_lo;
-      for (int e = m->ch_e0[c]; e < m->ch_e0[c + 1]; ++e)
-        for (int q = 0; q < m->ns; ++q) {
+      for (int q = 0; q < m->ns; ++q)  // node by node: vertices first
+        for (int e = m->ch_e0[c]; e < m->ch_e0[c + 1]; ++e) {
           int dof = m->conn[(size_t)e * n + q];
           int loc;
           if (dof < m->N_own) {
@@ -733,6 +783,7 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
       m->O_max = std::max(m->O_max, own_n);
       m->H_max = std::max(m->H_max, (int)hmap.size());
     }
+    build_incidence(m.get());
   }
   for (int e = 0; e < E; ++e)
     for (int j = 0; j < m->ni; ++j) m->conn[(size_t)e * n + m->ns + j] = m->bub[e] + j;
@@ -767,11 +818,30 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
   for (int i = 0; i < N; ++i)
     for (int c = 0; c < d; ++c)
       m->sigma[(size_t)i * d + c] = sigma_at(m->p, d, &m->dof_xyz[(size_t)i * d], c);
-  for (int e = m->E0; e < E; ++e)
-    for (int q = 0; q < n; ++q) {
-      const int i = m->conn[(size_t)e * n + q];
-      if (m->pidx[i] < 0) m->pidx[i] = m->Nl++;
+  if (m->layout == 0) {
+    // the layer chunks' owned DoFs and the layer's halo DoFs are each one range of DoFs: the
+    // layer index is the DoF less a shift, so a chunk's auxiliaries are contiguous like its u
+    if (m->E0 < E) {
+      const int lo = m->ch_own_lo[m->nch0];
+      int h0 = N;
+      for (int e = m->E0; e < E; ++e)
+        for (int q = 0; q < m->ns; ++q) {
+          const int i = m->conn[(size_t)e * n + q];
+          if (i >= m->N_own) h0 = std::min(h0, i);
+        }
+      m->p_own = lo;
+      m->p_halo = h0 - (m->N_own - lo);
+      for (int i = lo; i < m->N_own; ++i) m->pidx[i] = i - m->p_own;
+      for (int i = h0; i < N; ++i) m->pidx[i] = i - m->p_halo;
+      m->Nl = (m->N_own - lo) + (N - h0);
     }
+  } else {
+    for (int e = m->E0; e < E; ++e)
+      for (int q = 0; q < n; ++q) {
+        const int i = m->conn[(size_t)e * n + q];
+        if (m->pidx[i] < 0) m->pidx[i] = m->Nl++;
+      }
+  }
   // lumped boundary mass: facets owned by one element
   m->Mb.assign(N, 0);
   if (m->p.absorbing) {
@@ -839,6 +909,24 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
         for (int t = 0; t < d; ++t) s += Ji[r * d + t] * Ji[c * d + t];
         Gm[r * d + c] = det * s;  // |J| J^-1 J^-T
       }
+    double Am[9];
+    for (int c = 0; c < d * d; ++c) Am[c] = det * Ji[c];  // |J| J^-1
+    if (d == 3 && m->layout == 0) {
+      // in the axes of the cube around the tetrahedron (sym_layout.h): dx_cube/dxhat = -2 (1 - I)
+      const double Gx[9] = {Gm[0], Gm[1], Gm[2], Gm[3], Gm[4], Gm[5], Gm[6], Gm[7], Gm[8]};
+      const double Ax[9] = {Am[0], Am[1], Am[2], Am[3], Am[4], Am[5], Am[6], Am[7], Am[8]};
+      for (int r = 0; r < 3; ++r)
+        for (int c = 0; c < 3; ++c) {
+          double s = 0, t = 0;
+          for (int i = 0; i < 3; ++i) {
+            if (i != r) t += -2.0 * Ax[i * 3 + c];
+            for (int j = 0; j < 3; ++j)
+              if (i != r && j != c) s += 4.0 * Gx[i * 3 + j];
+          }
+          Gm[r * 3 + c] = s;
+          Am[r * 3 + c] = t;
+        }
+    }
     if (d == 2) {
       geo[0 * Es + e] = (float)Gm[0];
       geo[1 * Es + e] = (float)Gm[1];
@@ -848,7 +936,7 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
       for (int g = 0; g < 6; ++g) geo[(size_t)g * Es + e] = (float)Gm[idx[g]];
     }
     if (e >= m->E0)
-      for (int c = 0; c < d * d; ++c) lgeo[(size_t)c * (E - m->E0) + (e - m->E0)] = (float)(det * Ji[c]);
+      for (int c = 0; c < d * d; ++c) lgeo[(size_t)c * (E - m->E0) + (e - m->E0)] = (float)Am[c];
   }
   std::vector<int> conn_dev((size_t)m->ns * E);
   for (int e = 0; e < E; ++e)
@@ -875,7 +963,8 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
   int rc;
   if (m->layout == 0 && ((rc = upload(&m->d_chunks, chunks)) || (rc = upload(&m->d_halo, halo_dev)) ||
 
-                         (rc = upload(&m->d_lconn, m->lconn)))) {
+                         (rc = upload(&m->d_lconn, m->lconn)) || (rc = upload(&m->d_sdesc, m->sdesc)) ||
+                         (rc = upload(&m->d_smeta, m->smeta)))) {
     fwi_mesh_free(m.release());
     return rc;
   }
@@ -998,6 +1087,7 @@ int fwi_set_velocity(fwi_mesh* m, const double* c) {
   std::vector<float> c2(N), cv(N), cf((size_t)3 * N);
   const int LC = fwi::layer_coef_count(d);
   std::vector<float> lcf((size_t)m->Nl * LC, 0.f);
+  std::vector<float> lpsi((size_t)m->Nl * (d == 2 ? 1 : 4)), lcs((size_t)m->Nl * (d == 2 ? 8 : 12));
   std::vector<unsigned char> mask(N);
   for (int i = 0; i < N; ++i) {
     const double* s = &m->sigma[(size_t)i * d];
@@ -1028,6 +1118,7 @@ int fwi_set_velocity(fwi_mesh* m, const double* c) {
         L[d + k] = (float)(dt * psi2 * c[i] * c[i] / (m->M[i] * dk));
         L[2 * d + k] = (float)(dt / (m->M[i] * dk));
         L[3 * d + k] = (float)(psi2 * c[i] * c[i]);
+        if (d == 2 && k == 0) lpsi[m->pidx[i]] = L[3 * d];
         if (d == 3) {
           double psi3 = 1;
           for (int l = 0; l < 3; ++l)
@@ -1042,18 +1133,41 @@ int fwi_set_velocity(fwi_mesh* m, const double* c) {
         L[6 * d + 2] = (float)(dt * det1);
         L[6 * d + 3] = (float)(dt / m->M[i]);
       }
+      if (m->layout == 0) {
+        float* Q = &lcs[(size_t)m->pidx[i] * (d == 2 ? 8 : 12)];
+        if (d == 2) {
+          std::copy(L, L + 8, Q);
+        } else {
+          const float q[12] = {L[0], L[1], L[2], L[18], L[6], L[7], L[8], L[21], L[19], L[20], 0.f, 0.f};
+          std::copy(q, q + 12, Q);
+          for (int k = 0; k < 3; ++k) lpsi[(size_t)m->pidx[i] * 4 + k] = (float)s[k];
+        }
+      }
     }
   }
+  // chunks whose owned DoFs are neither damped nor on an absorbing boundary: v' = v - c2 y
+  std::vector<unsigned char> plain(m->layout == 0 ? m->nch() : 0, 1);
+  for (size_t ch = 0; ch < plain.size(); ++ch)
+    for (int i = m->ch_own_lo[ch]; i < m->ch_own_lo[ch + 1] && plain[ch]; ++i)
+      plain[ch] = cf[i] == 1.f && cf[(size_t)2 * N + i] == 0.f;
   dfree(m->d_c2);
   dfree(m->d_c);
   dfree(m->d_cf);
   dfree(m->d_lcf);
   dfree(m->d_mask);
+  dfree(m->d_splain);
+  dfree(m->d_lpsi);
+  m->d_splain = nullptr;
+  m->d_lpsi = nullptr;
+  dfree(m->d_lcs);
+  m->d_lcs = nullptr;
   m->d_c2 = m->d_c = m->d_cf = m->d_lcf = nullptr;
   m->d_mask = nullptr;
   int rc;
   if ((rc = upload(&m->d_c2, c2)) || (rc = upload(&m->d_c, cv)) || (rc = upload(&m->d_cf, cf)) ||
-      (rc = upload(&m->d_lcf, lcf)) || (rc = upload(&m->d_mask, mask)))
+      (rc = upload(&m->d_lcf, lcf)) || (rc = upload(&m->d_mask, mask)) ||
+      (rc = upload(&m->d_splain, plain)) || (rc = upload(&m->d_lpsi, lpsi)) ||
+      (rc = upload(&m->d_lcs, lcs)))
     return rc;
   m->have_velocity = true;
   return 0;
@@ -1076,7 +1190,7 @@ int fwi_batch_free(fwi_batch* b) {
                   b->d_rslot_phi, b->d_rec_elem, b->d_rec_phi, b->u, b->v, b->r, b->P, b->Pacc,
                   b->PaccY, b->Y, b->Yacc, b->ua, b->va, b->Pa, b->Ya, b->ckpt, b->ring,
                   b->gseg, b->gsum, b->gcomp, b->misfit, b->status, b->wav_dev, b->rec_dev, b->res_dev, b->stage_in, b->stage_out,
-                  b->stage_grad, b->gring};
+                  b->stage_grad};
   for (void* p : ptrs) dfree(p);
   delete b;
   return 0;
@@ -1198,6 +1312,16 @@ StepArgs base_args(fwi_batch* b) {
     a.chunks = m->d_chunks;
     a.halo = m->d_halo;
     a.lconn = m->d_lconn;
+    a.sdesc = m->d_sdesc;
+    a.smeta = m->d_smeta;
+    a.splain = m->d_splain;
+    a.lpsi = m->d_lpsi;
+    a.lcs = m->d_lcs;
+    a.comb = m->dim == 3 ? 1 : 0;
+    a.T_max = m->T_max;
+    a.SH_max = m->SH_max;
+    a.p_own = m->p_own;
+    a.p_halo = m->p_halo;
     a.h0 = m->N_own;
     a.hcnt = m->N - m->N_own;
   } else {
@@ -1227,8 +1351,6 @@ StepArgs base_args(fwi_batch* b) {
   a.R = b->R;
   a.gseg = b->gseg;
   a.grad_lanes = b->grad_lanes;
-  a.gstore = nullptr;
-  a.gload = nullptr;
   a.status = b->status;
   a.tc_wait_limit = b->tc_wait_limit;
   return a;
@@ -1346,17 +1468,14 @@ int check_status(fwi_batch* b, cudaStream_t st) {
 
 // Forward steps n0 .. n1-1 on the batch's forward state; optional records and checkpoints.
 // window > 0: wav is [S][window] and recs [S][window+1][R] (the steps of one segment).
-// gstore: where the steps write the forward field's gradients (one step only).
 void forward_steps(fwi_batch* b, int n0, int n1, const float* wav, float* recs, bool ckpts,
-                   cudaStream_t st, float* r_scratch = nullptr, int window = 0,
-                   float* gstore = nullptr) {
+                   cudaStream_t st, float* r_scratch = nullptr, int window = 0) {
   StepArgs a = base_args(b);
   if (r_scratch) a.r = r_scratch;
   if (window > 0) a.nt = window;
-  a.gstore = gstore;
   a.mode = 0;
   a.tc = 0;  // forward and recompute steps always on FP32 CUDA cores (records within 1e-5)
-  a.u = b->u;
+  a.u = a.u_out = b->u;
   a.v = b->v;
   a.P = b->P;
   a.Y = b->Y;
@@ -1416,21 +1535,13 @@ int adjoint_device(fwi_batch* b, const float* res, cudaStream_t st) {
   if (b->acc_lanes >= 0 && b->acc_lanes != b->grad_lanes)
     return fail(FWI_EINVAL, "the gradient accumulators hold sums of the other kind: call "
                             "fwi_gradient* before changing fwi_batch_set_gradient_lanes");
-  // the gradient store: triangles on the persistent kernel, summed gradient form
-  const fwi_mesh* mc = b->m;
-  const bool gst = b->gstore_on && mc->dim == 2 && mc->layout == 0 && !mc->use_tc &&
-                   b->S % 4 == 0 && mc->nch0 > 0 && !b->grad_lanes;
-  if (gst && !b->gring) {
-    b->gring_level = fwi::gstore_level_floats(mc->nch0, b->S, mc->nn);
-    if (int rc = dalloc(&b->gring, b->gring_level * (size_t)(b->K / b->gstride))) return rc;
-  }
   b->acc_lanes = b->grad_lanes;
   const size_t rn = (size_t)b->S * (b->nt + 1) * b->R;
   fwi::launch_misfit(res, (int64_t)rn / b->S, b->S, b->misfit, st);
   g_launches += 1;
   StepArgs a = base_args(b);
   a.mode = 1;
-  a.u = b->ua;
+  a.u = a.u_out = b->ua;
   a.v = b->va;
   a.P = b->Pa;
   a.Y = b->Ya;
@@ -1447,17 +1558,12 @@ int adjoint_device(fwi_batch* b, const float* res, cudaStream_t st) {
     float *cu, *cv, *cP, *cY;
     ckpt_ptrs(b, c, &cu, &cv, &cP, &cY);
     if (int rc = copy_state(b, b->u, b->v, b->P, b->Y, cu, cv, cP, cY, st)) return rc;
-    // the ring keeps U^n for the levels n = 0 (mod r) of the segment (n0 is one of them);
-    // with the gradient store, the forward step from level n also writes the gradients of
-    // U^n for the persistent kernel's gradient step, and one more step (from level n1 - 1)
-    // gives those of the segment's last level
+    // the ring keeps U^n for the levels n = 0 (mod r) of the segment (n0 is one of them)
     const int r = b->gstride;
     CUDA_TRY(cudaMemcpyAsync(b->ring, b->u, NS_ * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    auto glevel = [&](int n) { return b->gring + b->gring_level * (size_t)((n - n0) / r); };
-    for (int n = n0; n < (gst ? n1 : n1 - 1); ++n) {
-      forward_steps(b, n, n + 1, b->wav_dev, nullptr, false, st, nullptr, 0,
-                    gst && n % r == 0 ? glevel(n) : nullptr);
-      if (n + 1 < n1 && (n + 1) % r == 0)
+    for (int n = n0; n < n1 - 1; ++n) {
+      forward_steps(b, n, n + 1, b->wav_dev, nullptr, false, st);
+      if ((n + 1) % r == 0)
         CUDA_TRY(cudaMemcpyAsync(b->ring + NS_ * (size_t)((n + 1 - n0) / r), b->u,
                                  NS_ * sizeof(float), cudaMemcpyDeviceToDevice, st));
     }
@@ -1465,7 +1571,6 @@ int adjoint_device(fwi_batch* b, const float* res, cudaStream_t st) {
       a.n = mm;
       // the gradient integrand at the subsampled levels only (the others: adjoint step alone)
       a.ring_u = mm % r == 0 ? b->ring + NS_ * (size_t)((mm - n0) / r) : nullptr;
-      a.gload = gst && mm % r == 0 ? glevel(mm) : nullptr;
       run_step(b, a, st);
     }
     fwi::launch_fold(b->gseg, b->gsum, b->gcomp, (int64_t)b->m->N * (b->grad_lanes ? b->S : 1),
@@ -1749,12 +1854,7 @@ int fwi_gradient_raw(fwi_batch* b, double* dJdc_out, double* misfit_out, void* s
 int fwi_batch_set_gradient_store(fwi_batch* b, int on) {
   if (!b || (on != 0 && on != 1))
     return fail(FWI_EINVAL, "fwi_batch_set_gradient_store: on must be 0 or 1");
-  b->gstore_on = on;
-  if (!on && b->gring) {
-    dfree(b->gring);
-    b->gring = nullptr;
-  }
-  return 0;
+  return 0;  // no form of the gradient steps reads stored gradients (see the header)
 }
 
 int fwi_batch_set_gradient_lanes(fwi_batch* b, int per_shot) {
@@ -1791,7 +1891,8 @@ int fwi_profile_read(fwi_batch* b, double* ms, int64_t* steps) {
 int fwi_mesh_free(fwi_mesh* m) {
   if (!m) return 0;
   void* ptrs[] = {m->d_conn, m->d_geo, m->d_lgeo, m->d_pidx, m->d_c2, m->d_c, m->d_cf,
-                  m->d_lcf, m->d_M, m->d_mask, m->d_bub, m->d_chunks, m->d_halo, m->d_lconn};
+                  m->d_lcf, m->d_M, m->d_mask, m->d_bub, m->d_chunks, m->d_halo, m->d_lconn,
+                  m->d_sdesc, m->d_smeta, m->d_splain, m->d_lpsi, m->d_lcs};
   for (void* p : ptrs) dfree(p);
   delete m;
   return 0;

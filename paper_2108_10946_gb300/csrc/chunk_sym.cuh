@@ -1,0 +1,797 @@
+// Chunked time step on symmetry-adapted derivatives: one CTA assembles one chunk of
+// consecutive elements (Morton order) for a group of SG = min(S, 4) shots, entirely in
+// shared memory; a thread takes one element for one shot or for two (SymMap).
+//
+//   1. load    the chunk's owned DoFs, one contiguous range (bulk copies issued by one thread;
+//              copies of one DoF each if the batch has more shots than the group), its halo
+//              DoFs and its tables, all at once; the owned ranges of the chunk that will run a
+//              wave of CTAs later are brought to L2 meanwhile;
+//   2. element the stiffness, layer and gradient arithmetic in adapted coordinates
+//              (sym_tri.cuh); every thread writes its nodal sums to places of its own, [node]
+//              [element][shot] for shared nodes and the bubble range, so nothing is added by
+//              atomics;
+//   3. update  each shared DoF adds its elements' sums in the order of an incidence list
+//              (bubble DoFs have one) and, if owned, takes its increment update with coalesced
+//              writes; halo sums go to global accumulators that the node kernel finishes.
+//
+// Owned DoFs are read and written by this CTA only; halo DoFs are only read here.
+#pragma once
+#include "sym_tet.cuh"
+#include "update.cuh"
+#include <type_traits>
+
+namespace fwi {
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// asynchronous copy of BYTES = 4, 8 or 16 (aligned) bytes
+template <int BYTES>
+__device__ __forceinline__ void sym_cp(void* dst, const void* src) {
+  if constexpr (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst)), "l"(src), "n"(BYTES)
+                 : "memory");
+}
+__device__ __forceinline__ void sym_cp_wait() {
+  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+}
+
+__device__ __forceinline__ void sym_bar_init(uint64_t* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+__device__ __forceinline__ void sym_bar_expect(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+// Waits for phase 0 of the barrier; false if it gave up (bounded: 2^22 polls, each of which the
+// hardware may suspend for a while).
+__device__ __forceinline__ bool sym_bar_wait(uint64_t* bar) {
+  for (int i = 0; i < (1 << 22); ++i) {
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\nselp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(smem_addr(bar))
+        : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+__device__ __forceinline__ void sym_bulk(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_addr(dst)),
+               "l"(src), "r"(bytes), "r"(smem_addr(bar))
+               : "memory");
+}
+
+// A contiguous run of floats as a bulk copy: from the 16-byte boundary at or below its start, so
+// it lands `shift` floats past the place it is copied to; whole 16-byte groups (arrays that are
+// copied this way are allocated with four floats to spare).
+struct SymRun {
+  const float* src;
+  int shift;
+  uint32_t bytes;
+};
+__device__ __forceinline__ int sym_shift(const float* p) { return (int)(((uintptr_t)p >> 2) & 3); }
+__device__ __forceinline__ SymRun sym_run(const float* p, int n) {
+  SymRun r;
+  r.shift = sym_shift(p);
+  r.src = p - r.shift;
+  r.bytes = n > 0 ? (uint32_t)((n + r.shift + 3) & ~3) * 4u : 0u;
+  return r;
+}
+__device__ __forceinline__ void sym_prefetch(const float* p, int n) {  // to L2
+  const SymRun r = sym_run(p, n);
+  if (r.bytes) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(r.src), "r"(r.bytes) : "memory");
+}
+
+template <int SG>
+struct alignas(4 * SG) Lanes {  // one DoF's values of SG consecutive shots
+  float x[SG];
+};
+template <int SG>
+__device__ __forceinline__ Lanes<SG> lanes_ld(const float* p) {
+  return *reinterpret_cast<const Lanes<SG>*>(p);
+}
+template <int SG>
+__device__ __forceinline__ void lanes_st(float* p, const Lanes<SG>& v) {
+  *reinterpret_cast<Lanes<SG>*>(p) = v;
+}
+template <int SG>
+__device__ __forceinline__ void lanes_add(float* p, const Lanes<SG>& v) {  // global, no result
+  if constexpr (SG == 4) atomicAdd(reinterpret_cast<float4*>(p), make_float4(v.x[0], v.x[1], v.x[2], v.x[3]));
+  else if constexpr (SG == 2) atomicAdd(reinterpret_cast<float2*>(p), make_float2(v.x[0], v.x[1]));
+  else atomicAdd(p, v.x[0]);
+}
+// y += z, and y = a y + b z, on every shot
+template <int SG>
+__device__ __forceinline__ void lanes_acc(Lanes<SG>& y, const Lanes<SG>& z) {
+  if constexpr (SG == 1) {
+    y.x[0] += z.x[0];
+  } else {
+#pragma unroll
+    for (int k = 0; k < SG; k += 2) {
+      const float2 t = add2(make_float2(y.x[k], y.x[k + 1]), make_float2(z.x[k], z.x[k + 1]));
+      y.x[k] = t.x;
+      y.x[k + 1] = t.y;
+    }
+  }
+}
+template <int SG>
+__device__ __forceinline__ Lanes<SG> lanes_fma(float a, const Lanes<SG>& x, const Lanes<SG>& y) {  // a x + y
+  Lanes<SG> r;
+  if constexpr (SG == 1) {
+    r.x[0] = fmaf(a, x.x[0], y.x[0]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < SG; k += 2) {
+      const float2 t = fma2(dup<float2>(a), make_float2(x.x[k], x.x[k + 1]), make_float2(y.x[k], y.x[k + 1]));
+      r.x[k] = t.x;
+      r.x[k + 1] = t.y;
+    }
+  }
+  return r;
+}
+template <int SG>
+__device__ __forceinline__ Lanes<SG> lanes_mul(float a, const Lanes<SG>& x) {
+  Lanes<SG> r;
+#pragma unroll
+  for (int k = 0; k < SG; ++k) r.x[k] = a * x.x[k];
+  return r;
+}
+
+constexpr int SYM_PE = sym_pe(D, NN);  // most elements of a chunk, stride of its tables
+
+// A CTA's threads: one element for LANES shots each.
+template <int SG>
+struct SymMap {
+  static constexpr int LANES = SYM_LANES < SG ? SYM_LANES : SG, PER = SG / LANES, NT = SYM_PE * PER;
+  typedef typename std::conditional<LANES == 2, float2, float>::type V;
+};
+
+// Dynamic shared memory of one chunk (offsets in floats). T: largest chunk table, SH: most shared
+// DoFs (owned and halo), H: longest halo list of a chunk.
+struct SymSmem {
+  int u, f, c2, ps, om, ys, yb, p1, gs, gb, ws, wb, ss, sb, ids, meta, total;
+};
+// Floats per DoF of the layer's nodal coefficients: Psi2 c^2 (2D adjoint), sigma (3D).
+template <int D, int MODE>
+__host__ __device__ constexpr int sym_psi() { return D == 3 ? 4 : MODE != 0 ? 1 : 0; }
+
+template <int D, int NN, int NS, int SG, int MODE, bool LAYER>
+__host__ __device__ inline SymSmem sym_smem(int T, int SH, int H) {
+  constexpr int PE = SYM_PE, NI = NN - NS, NE = NS * PE * SG, NB = (NI * PE * SG + 3) / 4 * 4;
+  constexpr bool GRAD = MODE == 2;
+  auto up = [](int n) { return (n + 7) & ~3; };  // a multiple of 4 with room for a run's shift
+  SymSmem m{};
+  int o = 4;  // the mbarrier
+  m.u = o, o += up(T * SG);
+  m.f = o, o += GRAD ? up(T * SG) : 0;
+  m.c2 = o, o += up(T);
+  m.ps = o, o += LAYER ? up(T * sym_psi<D, MODE>()) : 0;
+  m.om = o, o += LAYER && D == 3 && MODE == 0 ? up(T * SG) : 0;  // the omega state
+  // the shared DoFs' layer auxiliaries P lie where the elements' sums go once all have read P (in
+  // 2D gradient steps that place holds the forward field's derivatives)
+  constexpr bool APART = GRAD && D == 2;
+  m.ys = o, m.yb = o + NE, m.p1 = o + (APART ? NE + NB : 0);
+  if (LAYER && APART) o += NE + NB + up(D * SH * SG);
+  else o += LAYER && up(D * SH * SG) > NE + NB ? up(D * SH * SG) : NE + NB;
+  m.gs = o, o += GRAD ? NE : 0;
+  m.gb = o, o += GRAD ? NB : 0;
+  m.ws = o, o += LAYER && D == 3 && MODE != 0 ? NE : 0;  // the omega row's sums
+  m.wb = o, o += LAYER && D == 3 && MODE != 0 ? NB : 0;
+  m.ss = o, o += LAYER ? D * NE : 0;
+  m.sb = o, o += LAYER ? up(D * NB) : 0;  // bubbles: P, then each (element, shot)'s own layer sums
+  m.ids = o, o += up(H);
+  m.meta = o, o += up(NS * PE + (SH + 16) / 2);  // table positions, incidence list, its pointers
+  m.total = o;
+  return m;
+}
+
+// Floats per layer DoF of the update's coefficients a.lcs: 2D e1, e2 forward, e2 adjoint, Psi2 c^2
+// of the two directions each; 3D e1 and c4, e2 (adjoint) and dt/M, c5 and dt det Psi1.
+template <int D>
+constexpr int SYM_LCS = D == 2 ? 8 : 12;
+
+struct SymDesc {
+  int e0, ne, own, nsh, hp, hn, meta, meta_n, plain;
+};
+__device__ __forceinline__ SymDesc sym_desc(const StepArgs& a, int c) {
+  SymDesc d;
+  const int4* p = reinterpret_cast<const int4*>(a.sdesc) + 2 * c;
+  const int4 x = __ldg(p), y = __ldg(p + 1);
+  d.e0 = x.x, d.ne = x.y, d.own = x.z, d.nsh = x.w;
+  d.hp = y.x, d.hn = y.y, d.meta = y.z, d.meta_n = y.w;
+  d.plain = __ldg(a.splain + c);
+  return d;
+}
+
+// Phase 1 of one chunk. The table: owned shared DoFs [0, nsh), bubbles, halo DoFs. The runs' shifts
+// follow from their addresses (sym_shift).
+template <int D, int NN, int NS, int SG, int MODE, bool LAYER>
+__device__ __forceinline__ void sym_load(const StepArgs& a, const SymDesc& cd, const SymSmem& L, float* sm, uint64_t* bar,
+                                         int s0, int tid) {
+  constexpr int NI = NN - NS, NT = SymMap<SG>::NT;
+  constexpr bool GRAD = MODE == 2, OM = LAYER && D == 3 && MODE == 0;
+  constexpr int PSI = LAYER ? sym_psi<D, MODE>() : 0;
+  const int S = a.S, on = cd.nsh + cd.ne * NI;
+  const size_t i0 = (size_t)cd.own * S + s0;
+  const size_t pi0 = (size_t)(cd.own - a.p_own);
+  if (tid == 0) {
+    // everything that is one run: coefficients, tables, and the fields if the group is the batch
+    const SymRun c2 = sym_run(a.c2 + cd.own, on),
+                 me = sym_run(reinterpret_cast<const float*>(a.smeta) + cd.meta, cd.meta_n);
+    SymRun u{}, f{}, ps{}, om{}, p1{}, p2{};
+    if (S == SG) {
+      u = sym_run(a.u + i0, on * SG);
+      if (GRAD) f = sym_run(a.ring_u + i0, on * SG);
+    }
+    if (LAYER) {
+      if (S == SG) {
+        p1 = sym_run(a.P + pi0 * D * SG, cd.nsh * D * SG);
+        p2 = sym_run(a.P + (pi0 + cd.nsh) * D * SG, cd.ne * NI * D * SG);
+      }
+      if (PSI) ps = sym_run(a.lpsi + pi0 * PSI, on * PSI);
+      if (OM && S == SG) om = sym_run(a.Y + pi0 * SG, on * SG);
+    }
+    sym_bar_expect(bar, c2.bytes + me.bytes + u.bytes + f.bytes + ps.bytes + om.bytes + p1.bytes + p2.bytes);
+    auto go = [&](int at, const SymRun& r) {
+      if (r.bytes) sym_bulk(sm + at, r.src, r.bytes, bar);
+    };
+    go(L.meta, me);
+    go(L.u, u);
+    go(L.c2, c2);
+    if (GRAD) go(L.f, f);
+    if (LAYER) {
+      go(L.p1, p1);
+      go(L.sb, p2);
+      go(L.ps, ps);
+      go(L.om, om);
+    }
+    // the update's own reads, to L2 meanwhile
+    if (S == SG) sym_prefetch(a.v + i0, on * SG);
+    sym_prefetch(a.cf + (size_t)a.N + cd.own, on);
+    if (!cd.plain) {
+      sym_prefetch(a.cf + cd.own, on);
+      sym_prefetch(a.cf + 2 * (size_t)a.N + cd.own, on);
+    }
+    if (LAYER) sym_prefetch(a.lcs + pi0 * SYM_LCS<D>, on * SYM_LCS<D>);
+    if (LAYER && D == 3 && S == SG) sym_prefetch(a.Y + pi0 * SG, on * SG);
+    // and the ranges of the chunk a wave of CTAs further on
+    const int nc = blockIdx.x + a.ch0 + a.wave;
+    if (nc < a.ch1) {
+      const SymDesc nx = sym_desc(a, nc);
+      const int nn = nx.nsh + nx.ne * NI;
+      sym_prefetch(reinterpret_cast<const float*>(a.smeta) + nx.meta, nx.meta_n);
+      sym_prefetch(reinterpret_cast<const float*>(a.halo) + nx.hp, nx.hn);
+      sym_prefetch(a.c2 + nx.own, nn);
+      if (S == SG) {
+        sym_prefetch(a.u + (size_t)nx.own * S, nn * SG);
+        if (GRAD) sym_prefetch(a.ring_u + (size_t)nx.own * S, nn * SG);
+        if (LAYER) sym_prefetch(a.P + (size_t)(nx.own - a.p_own) * D * SG, nn * D * SG);
+      }
+    }
+  }
+  float* us = sm + L.u + sym_shift(a.u + i0);
+  float* fs = sm + L.f + (GRAD ? sym_shift(a.ring_u + i0) : 0);
+  float* cs = sm + L.c2 + sym_shift(a.c2 + cd.own);
+  float *ps = sm + L.ps, *om = sm + L.om, *p1 = sm + L.p1, *p2 = sm + L.sb;
+  if (LAYER) {
+    if (PSI) ps += sym_shift(a.lpsi + pi0 * PSI);
+    if (OM) om += sym_shift(a.Y + pi0 * S + s0);
+    p1 += sym_shift(a.P + (pi0 * S + s0) * D);
+    p2 += sym_shift(a.P + ((pi0 + cd.nsh) * S + s0) * D);
+  }
+  if (S != SG) {  // the group's shots are a part of each DoF's run
+    for (int l = tid; l < on; l += NT) {
+      const size_t dof = (size_t)(cd.own + l);
+      sym_cp<4 * SG>(us + l * SG, a.u + dof * S + s0);
+      if (GRAD) sym_cp<4 * SG>(fs + l * SG, a.ring_u + dof * S + s0);
+      if (LAYER)
+#pragma unroll
+        for (int k = 0; k < D; ++k)
+          sym_cp<4 * SG>((l < cd.nsh ? p1 + l * D * SG : p2 + (l - cd.nsh) * D * SG) + k * SG,
+                         a.P + ((pi0 + l) * D + k) * S + s0);
+      if (OM) sym_cp<4 * SG>(om + l * SG, a.Y + (pi0 + l) * S + s0);
+      if (l % (32 / SG) == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.v + dof * S + s0));
+    }
+  }
+  for (int h = tid; h < cd.hn; h += NT) {
+    const int id = __ldg(a.halo + cd.hp + h), l = on + h;
+    reinterpret_cast<int*>(sm + L.ids)[h] = id;
+    sym_cp<4 * SG>(us + l * SG, a.u + (size_t)id * S + s0);
+    if (GRAD) sym_cp<4 * SG>(fs + l * SG, a.ring_u + (size_t)id * S + s0);
+    sym_cp<4>(cs + l, a.c2 + id);
+    if (LAYER) {
+      const size_t pi = (size_t)(id - a.p_halo);
+#pragma unroll
+      for (int k = 0; k < D; ++k) sym_cp<4 * SG>(p1 + ((cd.nsh + h) * D + k) * SG, a.P + (pi * D + k) * S + s0);
+      if (PSI) sym_cp<4 * (PSI ? PSI : 1)>(ps + l * PSI, a.lpsi + pi * PSI);
+      if (OM) sym_cp<4 * SG>(om + l * SG, a.Y + pi * S + s0);
+    }
+  }
+}
+
+// Sum over the incidence list of a shared DoF of the table t ([node][element][shot]).
+template <int SG>
+__device__ __forceinline__ Lanes<SG> sym_sum(const float* t, const uint16_t* ge, int b, int e) {
+  Lanes<SG> y = lanes_ld<SG>(t + (int)ge[b] * SG);
+  for (int i = b + 1; i < e; ++i) lanes_acc<SG>(y, lanes_ld<SG>(t + (int)ge[i] * SG));
+  return y;
+}
+
+// The update's reads of a round of owned DoFs: increments and coefficients.
+template <int SG, int B>
+struct SymRound {
+  Lanes<SG> v[B];
+  float c1[B], c2[B], c3[B];
+  __device__ __forceinline__ void load(const StepArgs& a, const SymDesc& cd, int on, int s0, int l0, int nt) {
+#pragma unroll
+    for (int k = 0; k < B; ++k) {
+      const int l = l0 + k * nt;
+      if (l < on) {
+        const size_t dof = (size_t)(cd.own + l);
+        v[k] = lanes_ld<SG>(a.v + dof * a.S + s0);
+        c2[k] = __ldg(a.cf + (size_t)a.N + dof);
+        c1[k] = cd.plain ? 1.f : __ldg(a.cf + dof);
+        c3[k] = cd.plain ? 0.f : __ldg(a.cf + 2 * (size_t)a.N + dof);
+      }
+    }
+  }
+};
+
+// Phase 3 of one chunk (after a barrier); cur: its first round's reads, issued before the barrier.
+// v' = c1 v - c2 y - c3 u, u' = u + v'. chk collects 0 * u', which stays zero while every value is
+// finite.
+template <int D, int NN, int NS, int MODE, bool LAYER, int SG, int B>
+__device__ __forceinline__ void sym_finish(const StepArgs& a, const SymDesc& cd, const SymSmem& L, const float* sm,
+                                           int s0, int tid, SymRound<SG, B>& cur, float& chk) {
+  constexpr int PE = SYM_PE, NI = NN - NS, NT = SymMap<SG>::NT;
+  constexpr bool GRAD = MODE == 2;
+  const int S = a.S, nb = cd.ne * NI, on = cd.nsh + nb;
+  const uint16_t* ge = reinterpret_cast<const uint16_t*>(sm + L.meta) + NS * PE;
+  const uint16_t* gp = ge + NS * PE;
+  const int* ids = reinterpret_cast<const int*>(sm + L.ids);
+  const float* us = sm + L.u + sym_shift(a.u + (size_t)cd.own * S + s0);
+  for (int l0 = tid; l0 < on; l0 += B * NT) {
+    SymRound<SG, B> nxt;
+    nxt.load(a, cd, on, s0, l0 + B * NT, NT);
+#pragma unroll
+    for (int k = 0; k < B; ++k) {
+      const int l = l0 + k * NT;
+      if (l < on) {
+        const Lanes<SG> y = l < cd.nsh ? sym_sum<SG>(sm + L.ys, ge, gp[l], gp[l + 1]) : lanes_ld<SG>(sm + L.yb + (l - cd.nsh) * SG);
+        Lanes<SG> un = lanes_ld<SG>(us + l * SG), vn = cur.v[k];
+        if (!cd.plain) vn = lanes_fma<SG>(-cur.c3[k], un, lanes_mul<SG>(cur.c1[k], vn));
+        vn = lanes_fma<SG>(-cur.c2[k], y, vn);
+        if constexpr (LAYER && D == 3) {  // the omega state
+          const size_t pi = (size_t)(cd.own + l - a.p_own);
+          const float* lc = a.lcs + pi * 12;
+          float* Y = a.Y + pi * S + s0;
+          const Lanes<SG> Yo = lanes_ld<SG>(Y);
+          if constexpr (MODE == 0) {
+            vn = lanes_fma<SG>(-__ldg(lc + 3), Yo, vn);
+            lanes_st<SG>(Y, lanes_fma<SG>(a.dt, un, Yo));
+          } else {
+            const Lanes<SG> yw = l < cd.nsh ? sym_sum<SG>(sm + L.ws, ge, gp[l], gp[l + 1]) : lanes_ld<SG>(sm + L.wb + (l - cd.nsh) * SG);
+            vn = lanes_fma<SG>(__ldg(lc + 8), Yo, vn);
+            lanes_st<SG>(Y, lanes_fma<SG>(__ldg(lc + 7), yw, lanes_fma<SG>(-__ldg(lc + 9), un, Yo)));
+          }
+        }
+        lanes_acc<SG>(un, vn);
+#pragma unroll
+        for (int j = 0; j < SG; ++j) chk = fmaf(0.f, un.x[j], chk);
+        const size_t gi = (size_t)(cd.own + l) * S + s0;
+        lanes_st<SG>(a.v + gi, vn);
+        lanes_st<SG>(a.u_out + gi, un);
+      }
+    }
+    cur = nxt;
+  }
+  for (int h = tid; h < cd.hn; h += NT) {
+    const int l = cd.nsh + h;
+    lanes_add<SG>(a.r + (size_t)(ids[h] - a.N_own) * S + s0, sym_sum<SG>(sm + L.ys, ge, gp[l], gp[l + 1]));
+  }
+  if constexpr (LAYER) {  // the layer auxiliaries: P' = e1 P - e2 s
+    const size_t pi0 = (size_t)(cd.own - a.p_own);
+    const float* sb = sm + L.sb + sym_shift(a.P + ((pi0 + cd.nsh) * S + s0) * D);
+    constexpr int LC = SYM_LCS<D>, E2 = D == 3 ? 4 : MODE == 0 ? 2 : 4;  // e1 first
+    for (int l0 = tid; l0 < on; l0 += 2 * NT) {
+      Lanes<SG> P[2][D];
+      float e[2][2 * D];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int l = l0 + k * NT;
+        if (l < on) {
+#pragma unroll
+          for (int d = 0; d < D; ++d) {
+            P[k][d] = lanes_ld<SG>(a.P + ((pi0 + l) * D + d) * S + s0);
+            e[k][d] = __ldg(a.lcs + (pi0 + l) * LC + d);
+            e[k][D + d] = __ldg(a.lcs + (pi0 + l) * LC + E2 + d);
+          }
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int l = l0 + k * NT;
+        if (l < on) {
+          const int b = l < cd.nsh ? gp[l] : 0, f = l < cd.nsh ? gp[l + 1] : 0;
+#pragma unroll
+          for (int d = 0; d < D; ++d) {
+            const Lanes<SG> s = l < cd.nsh ? sym_sum<SG>(sm + L.ss + d * NS * PE * SG, ge, b, f)
+                                           : lanes_ld<SG>(sb + ((l - cd.nsh) * D + d) * SG);
+            lanes_st<SG>(a.P + ((pi0 + l) * D + d) * S + s0,
+                         lanes_fma<SG>(-e[k][D + d], s, lanes_mul<SG>(e[k][d], P[k][d])));
+          }
+        }
+      }
+    }
+    for (int h = tid; h < cd.hn; h += NT) {
+      const int b = gp[cd.nsh + h], e = gp[cd.nsh + h + 1];
+      const size_t pi = (size_t)(ids[h] - a.p_halo);
+#pragma unroll
+      for (int d = 0; d < D; ++d)
+        lanes_add<SG>(a.Pacc + (pi * D + d) * S + s0, sym_sum<SG>(sm + L.ss + d * NS * PE * SG, ge, b, e));
+      if constexpr (D == 3 && MODE != 0) lanes_add<SG>(a.Yacc + pi * S + s0, sym_sum<SG>(sm + L.ws, ge, b, e));
+    }
+  }
+  if constexpr (GRAD) {  // 2 c of the integrand here, once per DoF
+    auto put = [&](int dof, const Lanes<SG>& g) {
+      const float c = 2.f * __ldg(a.cvel + dof);
+      if (a.grad_lanes) {  // one segment accumulator per shot, [S][N]
+#pragma unroll
+        for (int k = 0; k < SG; ++k) atomicAdd(a.gseg + (size_t)(s0 + k) * a.N + dof, c * g.x[k]);
+      } else {  // summed over the shots, [N]
+        float t = g.x[0];
+#pragma unroll
+        for (int k = 1; k < SG; ++k) t += g.x[k];
+        atomicAdd(a.gseg + dof, c * t);
+      }
+    };
+    for (int l = tid; l < cd.nsh; l += NT) put(cd.own + l, sym_sum<SG>(sm + L.gs, ge, gp[l], gp[l + 1]));
+    for (int l = tid; l < nb; l += NT) put(cd.own + cd.nsh + l, lanes_ld<SG>(sm + L.gb + l * SG));
+    for (int h = tid; h < cd.hn; h += NT) put(ids[h], sym_sum<SG>(sm + L.gs, ge, gp[cd.nsh + h], gp[cd.nsh + h + 1]));
+  }
+}
+
+// Sources and receivers of an element (few have any), for the lanes of a thread: shots s, s + 1, ...;
+// u: their nodal values, y(q): their sums at node q.
+template <int NN, int MODE, int SG, class A, class F>
+__device__ __forceinline__ void sym_inject(const StepArgs& a, int slot, int e, int s1, const float* u, A at, F y) {
+  const int rb = __ldg(a.rslot_ptr + slot), re = __ldg(a.rslot_ptr + slot + 1);
+#pragma unroll 1
+  for (int k = 0; k < SymMap<SG>::LANES; ++k) {
+    const int s = s1 + k;
+    for (int r = rb; r < re; ++r) {
+      const float* phi = a.rslot_phi + (size_t)r * NN;
+      const size_t at_rec = ((size_t)s * (a.nt + 1) + a.n) * a.R + __ldg(a.rslot_rec + r);
+      if constexpr (MODE != 0) {
+        const float res = __ldg(a.resid + at_rec);
+        for (int q = 0; q < NN; ++q) y(q)[k] += res * __ldg(phi + q);
+      } else if (a.rec != nullptr) {
+        float acc = 0.f;
+        for (int q = 0; q < NN; ++q) acc = fmaf(__ldg(phi + q), u[at(q) * SG + k], acc);
+        a.rec[at_rec] = acc;
+      }
+    }
+    if (MODE == 0 && __ldg(a.src_elem + s) == e) {
+      const float wv = __ldg(a.wavelet + (size_t)s * a.nt + a.n);
+      for (int q = 0; q < NN; ++q) y(q)[k] -= wv * __ldg(a.src_phi + (size_t)s * NN + q);
+    }
+  }
+}
+
+// The element phase's walk over the orbits of a triangle: derivatives, node(q, v, r, t) for each
+// node, divergence (of the fluxes that node leaves in r, t; not for a field that is only read).
+template <class V, int NN, bool DIV, int O, class F>
+__device__ __forceinline__ void sym_tri_orbits(const TriCoef<V, NN>& U, TriCoef<V, NN>& Y, F node) {
+  using T = TriSym<NN>;
+  if constexpr (O < T::NO) {
+    constexpr int SIDES = T::kind(O) == 'X' ? 2 : 1, NV = T::kind(O) == 'C' ? 1 : 3;
+    V r[2][3], t[2][3];
+    tri_grad<V, NN, O>(U, r, t);
+#pragma unroll
+    for (int k = 0; k < SIDES; ++k)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) node(T::node(O, v, k), v, r[k][v], t[k][v]);
+    if constexpr (DIV) tri_div<V, NN, O>(r, t, Y);
+    sym_tri_orbits<V, NN, DIV, O + 1>(U, Y, node);
+  }
+}
+
+// One step of a triangle chunk. MODE: 0 forward, 1 adjoint, 2 adjoint with the gradient integrand.
+template <int NN, int NS, int MODE, bool LAYER, int SG>
+__device__ __forceinline__ void sym_tri_body(const StepArgs& a, float* sm) {
+  using M = SymMap<SG>;
+  using V = typename M::V;
+  constexpr int NI = NN - NS, PE = SYM_PE;
+  constexpr bool ADJ = MODE != 0, GRAD = MODE == 2;
+  const int tid = threadIdx.x, S = a.S, s0 = blockIdx.y * SG;
+  const SymSmem L = sym_smem<2, NN, NS, SG, MODE, LAYER>(a.T_max, a.SH_max, a.H_max);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(sm);
+  if (tid == 0) sym_bar_init(bar);  // (the thread that issues the barrier's copies)
+  const SymDesc cd = sym_desc(a, blockIdx.x + a.ch0);
+  sym_load<2, NN, NS, SG, MODE, LAYER>(a, cd, L, sm, bar, s0, tid);
+  __syncthreads();  // the barrier is set up before anyone asks it
+  const int el = tid / M::PER, ln = tid % M::PER * M::LANES;  // element, first shot of the group
+  const bool act = el < cd.ne;
+  const int ee = act ? el : 0, e = cd.e0 + ee, nb = cd.ne * NI;
+  const int slot = act ? __ldg(a.inj + e) : -1, bub = cd.nsh + ee * NI;
+  const size_t i0 = (size_t)cd.own * S + s0, pi0 = (size_t)(cd.own - a.p_own);
+  const uint16_t* lq = reinterpret_cast<const uint16_t*>(sm + L.meta) + ee;
+  float H0[3], A0[2][2];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) H0[c] = __ldg(a.geo + (size_t)c * a.Es + e);
+  if constexpr (LAYER)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) A0[c >> 1][c & 1] = __ldg(a.lgeo + (size_t)c * (a.E - a.E0) + (e - a.E0));
+  sym_cp_wait();
+  const bool ok = sym_bar_wait(bar);
+  if (__syncthreads_or(!ok)) {  // a copy did not arrive: report it and leave the fields alone
+    sym_bar_wait(bar);
+    if (tid == 0) atomicOr(a.status, 2);
+    return;
+  }
+
+  // ---- elements --------------------------------------------------------------------------
+  const float* us = sm + L.u + sym_shift(a.u + i0) + ln;
+  const float* cs = sm + L.c2 + sym_shift(a.c2 + cd.own);
+  // a thread's own places for node q: the sums' ([node][element][shot], bubbles in DoF order), ...
+  const int ps = el * SG + ln, pb = el * NI * SG + ln;
+  auto at = [&](int q) { return q < NS ? (int)lq[q * PE] : bub + (q - NS); };
+  auto ld = [&](const float* p) { return *reinterpret_cast<const V*>(p); };
+  auto st = [&](float* p, V v) { *reinterpret_cast<V*>(p) = v; };
+  auto own = [&](int s, int b, int q) { return sm + (q < NS ? s + ps + q * PE * SG : b + pb + (q - NS) * SG); };
+  TriCoef<V, NN> Y;
+  if (act) {
+    TriCoef<V, NN> U;
+    if constexpr (GRAD) {  // the forward field's derivatives wait in places that are filled later
+      const float* fs = sm + L.f + sym_shift(a.ring_u + i0) + ln;
+      tri_analyse<V, NN>(U, [&](int q) { return ld(fs + at(q) * SG); });
+      sym_tri_orbits<V, NN, false, 0>(U, Y, [&](int q, int, V& r, V& t) {
+        st(own(L.gs, L.gb, q), r);
+        st(own(L.ys, L.yb, q), t);
+      });
+      asm volatile("" ::: "memory");  // (keeps the two passes' registers apart)
+    }
+    float H[3][3], A[3][2][2];  // A: rows (radial, tangential) of |J| J^-1 in the three frames
+    tri_metric(H0[0], H0[1], H0[2], H);
+    if constexpr (LAYER) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        tri_frame<0>(A0[0][c], A0[1][c], A[0][0][c], A[0][1][c]);
+        tri_frame<1>(A0[0][c], A0[1][c], A[1][0][c], A[1][1][c]);
+        tri_frame<2>(A0[0][c], A0[1][c], A[2][0][c], A[2][1][c]);
+      }
+    }
+    const float* p1 = sm + L.p1 + (LAYER ? sym_shift(a.P + (pi0 * S + s0) * 2) : 0) + ln;
+    float* p2 = sm + L.sb + (LAYER ? sym_shift(a.P + ((pi0 + cd.nsh) * S + s0) * 2) : 0) + el * NI * 2 * SG + ln;
+    const float* psi = sm + L.ps + (LAYER && ADJ ? sym_shift(a.lpsi + pi0) : 0);
+    tri_analyse<V, NN>(U, [&](int q) { return ld(us + at(q) * SG); });
+    tri_zero(Y);
+    // one node: (r, t) in are the field's derivatives in frame v, out the flux
+    sym_tri_orbits<V, NN, true, 0>(U, Y, [&](int q, int v, V& r, V& t) {
+      const float w = c_w[q];
+      const int l = at(q);
+      const V wc = dup<V>(w * cs[l]), gr = r, gt = t;
+      const V hr = fma2(dup<V>(H[v][0]), gr, mul2(dup<V>(H[v][1]), gt));
+      const V ht = fma2(dup<V>(H[v][1]), gr, mul2(dup<V>(H[v][2]), gt));
+      r = mul2(wc, hr);
+      t = mul2(wc, ht);
+      if constexpr (GRAD) {  // w (Ghat grad u_dag) . grad u
+        float* g = own(L.gs, L.gb, q);
+        st(g, mul2(dup<V>(w), fma2(hr, ld(g), mul2(ht, ld(own(L.ys, L.yb, q))))));
+      }
+      if constexpr (LAYER) {
+        const V sx = mul2(dup<V>(w), fma2(dup<V>(A[v][0][0]), gr, mul2(dup<V>(A[v][1][0]), gt)));
+        const V sz = mul2(dup<V>(w), fma2(dup<V>(A[v][0][1]), gr, mul2(dup<V>(A[v][1][1]), gt)));
+        V px, pz;
+        if (q < NS) {
+          const float* p = p1 + (l - (l >= cd.nsh ? nb : 0)) * 2 * SG;
+          px = ld(p);
+          pz = ld(p + SG);
+          st(sm + L.ss + ps + q * PE * SG, sx);
+          st(sm + L.ss + ps + (NS + q) * PE * SG, sz);
+        } else {  // a bubble's P gives way to its layer sums
+          float* p = p2 + (q - NS) * 2 * SG;
+          px = ld(p);
+          pz = ld(p + SG);
+          st(p, sx);
+          st(p + SG, sz);
+        }
+        // Psi2 c^2 (adjoint) is opposite in the two directions
+        const float wp = ADJ ? w * psi[l] : w;
+        const V zz = dup<V>(ADJ ? -wp : wp), xx = dup<V>(wp);
+        px = mul2(xx, px);
+        pz = mul2(zz, pz);
+        r = fma2(dup<V>(A[v][0][0]), px, fma2(dup<V>(A[v][0][1]), pz, r));
+        t = fma2(dup<V>(A[v][1][0]), px, fma2(dup<V>(A[v][1][1]), pz, t));
+      }
+    });
+  }
+  if (LAYER && !GRAD) __syncthreads();  // every P of a shared DoF has been read
+  if (act) {
+    tri_gather_back<V, NN>(Y, [&](int q, V y) { st(own(L.ys, L.yb, q), y); });
+    if (slot >= 0) sym_inject<NN, MODE, SG>(a, slot, e, s0 + ln, us, at, [&](int q) { return own(L.ys, L.yb, q); });
+  }
+  constexpr int B = 4;
+  SymRound<SG, B> first;
+  first.load(a, cd, cd.nsh + nb, s0, tid, M::NT);
+  __syncthreads();
+
+  float chk = 0.f;
+  sym_finish<2, NN, NS, MODE, LAYER, SG, B>(a, cd, L, sm, s0, tid, first, chk);
+  if (!(chk == 0.f)) atomicOr(a.status, 1);
+}
+
+// The walk over the orbits of a tetrahedron: derivatives of N fields, node(q, g) for each node with
+// g[field][axis], then the divergence of the fluxes that node leaves in g[0] to Y (and of g[1] to
+// Y2, if DIV2).
+template <class V, int NN, int N, bool DIV2, int O, class F>
+__device__ __forceinline__ void sym_tet_orbits(const TetCoef<V, NN>* const (&U)[N], TetCoef<V, NN>& Y,
+                                               TetCoef<V, NN>& Y2, F node) {
+  if constexpr (O < TetSym<NN>::NO) {
+    V g[N > 1 || !DIV2 ? N : 2][3][4];
+#pragma unroll
+    for (int f = 0; f < N; ++f) {
+      tet_grad<V, NN, O, 0>(*U[f], g[f][0]);
+      tet_grad<V, NN, O, 1>(*U[f], g[f][1]);
+      tet_grad<V, NN, O, 2>(*U[f], g[f][2]);
+    }
+#pragma unroll
+    for (int h = 0; h < TetSize<NN, O>::N; ++h) {
+      V x[N > 1 || !DIV2 ? N : 2][3];
+#pragma unroll
+      for (int f = 0; f < N; ++f)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) x[f][d] = g[f][d][h];
+      node(TetSym<NN>::node(O, h), x);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        g[0][d][h] = x[0][d];
+        if constexpr (DIV2) g[1][d][h] = x[1][d];
+      }
+    }
+    tet_div<V, NN, O, 0>(g[0][0], Y);
+    tet_div<V, NN, O, 1>(g[0][1], Y);
+    tet_div<V, NN, O, 2>(g[0][2], Y);
+    if constexpr (DIV2) {
+      tet_div<V, NN, O, 0>(g[1][0], Y2);
+      tet_div<V, NN, O, 1>(g[1][1], Y2);
+      tet_div<V, NN, O, 2>(g[1][2], Y2);
+    }
+    sym_tet_orbits<V, NN, N, DIV2, O + 1>(U, Y, Y2, node);
+  }
+}
+
+// One step of a tetrahedra chunk. Fields: u; the forward field (gradient steps); omega (forward
+// steps in the layer).
+template <int NN, int NS, int MODE, bool LAYER, int SG>
+__device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
+  using M = SymMap<SG>;
+  using V = typename M::V;
+  constexpr int NI = NN - NS, PE = SYM_PE;
+  constexpr bool ADJ = MODE != 0, GRAD = MODE == 2, OM = LAYER && !ADJ, W = LAYER && ADJ;
+  constexpr int NF = 1 + (GRAD || OM);
+  const int tid = threadIdx.x, S = a.S, s0 = blockIdx.y * SG;
+  const SymSmem L = sym_smem<3, NN, NS, SG, MODE, LAYER>(a.T_max, a.SH_max, a.H_max);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(sm);
+  if (tid == 0) sym_bar_init(bar);  // (the thread that issues the barrier's copies)
+  const SymDesc cd = sym_desc(a, blockIdx.x + a.ch0);
+  sym_load<3, NN, NS, SG, MODE, LAYER>(a, cd, L, sm, bar, s0, tid);
+  __syncthreads();  // the barrier is set up before anyone asks it
+  const int el = tid / M::PER, ln = tid % M::PER * M::LANES;  // element, first shot of the group
+  const bool act = el < cd.ne;
+  const int ee = act ? el : 0, e = cd.e0 + ee, nb = cd.ne * NI;
+  const int slot = act ? __ldg(a.inj + e) : -1, bub = cd.nsh + ee * NI;
+  const size_t i0 = (size_t)cd.own * S + s0, pi0 = (size_t)(cd.own - a.p_own);
+  const uint16_t* lq = reinterpret_cast<const uint16_t*>(sm + L.meta) + ee;
+  float G[6], A[3][3];  // |J| J^-1 J^-T and |J| J^-1 in the cube's axes
+#pragma unroll
+  for (int c = 0; c < 6; ++c) G[c] = __ldg(a.geo + (size_t)c * a.Es + e);
+  if constexpr (LAYER)
+#pragma unroll
+    for (int c = 0; c < 9; ++c) A[c / 3][c % 3] = __ldg(a.lgeo + (size_t)c * (a.E - a.E0) + (e - a.E0));
+  sym_cp_wait();
+  const bool ok = sym_bar_wait(bar);
+  if (__syncthreads_or(!ok)) {  // a copy did not arrive: report it and leave the fields alone
+    sym_bar_wait(bar);
+    if (tid == 0) atomicOr(a.status, 2);
+    return;
+  }
+
+  // ---- elements --------------------------------------------------------------------------
+  const float* us = sm + L.u + sym_shift(a.u + i0) + ln;
+  const float* cs = sm + L.c2 + sym_shift(a.c2 + cd.own);
+  const int ps = el * SG + ln, pb = el * NI * SG + ln;  // a thread's own places (see sym_tri_body)
+  auto at = [&](int q) { return q < NS ? (int)lq[q * PE] : bub + (q - NS); };
+  auto ld = [&](const float* p) { return *reinterpret_cast<const V*>(p); };
+  auto st = [&](float* p, V v) { *reinterpret_cast<V*>(p) = v; };
+  auto own = [&](int s, int b, int q) { return sm + (q < NS ? s + ps + q * PE * SG : b + pb + (q - NS) * SG); };
+  TetCoef<V, NN> Y, Y2;
+  if (act) {
+    TetCoef<V, NN> U, F;
+    if constexpr (GRAD) {
+      const float* fs = sm + L.f + sym_shift(a.ring_u + i0) + ln;
+      tet_analyse<V, NN>(F, [&](int q) { return ld(fs + at(q) * SG); });
+    }
+    if constexpr (OM) {
+      const float* om = sm + L.om + sym_shift(a.Y + pi0 * S + s0) + ln;
+      tet_analyse<V, NN>(F, [&](int q) { return ld(om + at(q) * SG); });
+    }
+    const float* p1 = sm + L.p1 + (LAYER ? sym_shift(a.P + (pi0 * S + s0) * 3) : 0) + ln;
+    float* p2 = sm + L.sb + (LAYER ? sym_shift(a.P + ((pi0 + cd.nsh) * S + s0) * 3) : 0) + el * NI * 3 * SG + ln;
+    const float* sig = sm + L.ps + (LAYER ? sym_shift(a.lpsi + pi0 * 4) : 0);
+    tet_analyse<V, NN>(U, [&](int q) { return ld(us + at(q) * SG); });
+    tet_zero(Y);
+    if constexpr (W) tet_zero(Y2);
+    // one node: x[0] in are the field's derivatives, out the flux (x[1]: the other field's; out, in
+    // the layer's adjoint, the omega row's flux)
+    auto node = [&](int q, auto& x) {
+      const float w = c_w[q];
+      const int l = at(q);
+      const float c2 = cs[l];
+      const V wc = dup<V>(w * c2), g0 = x[0][0], g1 = x[0][1], g2 = x[0][2];
+      const V h0 = fma2(dup<V>(G[0]), g0, fma2(dup<V>(G[1]), g1, mul2(dup<V>(G[2]), g2)));
+      const V h1 = fma2(dup<V>(G[1]), g0, fma2(dup<V>(G[3]), g1, mul2(dup<V>(G[4]), g2)));
+      const V h2 = fma2(dup<V>(G[2]), g0, fma2(dup<V>(G[4]), g1, mul2(dup<V>(G[5]), g2)));
+      if constexpr (GRAD)  // w (Ghat grad u_dag) . grad u
+        st(own(L.gs, L.gb, q), mul2(dup<V>(w), fma2(h0, x[1][0], fma2(h1, x[1][1], mul2(h2, x[1][2])))));
+      V f[3] = {mul2(wc, h0), mul2(wc, h1), mul2(wc, h2)};
+      if constexpr (LAYER) {
+        const float s1 = sig[4 * l], s2 = sig[4 * l + 1], s3 = sig[4 * l + 2], tr = s1 + s2 + s3;
+        const float psi2[3] = {c2 * (2.f * s1 - tr), c2 * (2.f * s2 - tr), c2 * (2.f * s3 - tr)};
+        const float psi3[3] = {c2 * s2 * s3, c2 * s1 * s3, c2 * s1 * s2};
+        float* p = q < NS ? const_cast<float*>(p1) + (l - (l >= cd.nsh ? nb : 0)) * 3 * SG : p2 + (q - NS) * 3 * SG;
+        V P[3], Q[3], s[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          P[k] = ld(p + k * SG);
+          s[k] = fma2(dup<V>(A[0][k]), g0, fma2(dup<V>(A[1][k]), g1, mul2(dup<V>(A[2][k]), g2)));
+          if constexpr (OM) {  // both gradients, each with its Psi c^2
+            const V y = fma2(dup<V>(A[0][k]), x[1][0], fma2(dup<V>(A[1][k]), x[1][1], mul2(dup<V>(A[2][k]), x[1][2])));
+            s[k] = fma2(dup<V>(-psi3[k]), y, mul2(dup<V>(psi2[k]), s[k]));
+          }
+          s[k] = mul2(dup<V>(w), s[k]);
+          Q[k] = ADJ ? mul2(dup<V>(w * psi2[k]), P[k]) : mul2(dup<V>(w), P[k]);
+          if (q < NS) st(sm + L.ss + ps + (k * NS + q) * PE * SG, s[k]);
+          else st(p + k * SG, s[k]);  // a bubble's P gives way to its layer sums
+        }
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          f[d] = fma2(dup<V>(A[d][0]), Q[0], fma2(dup<V>(A[d][1]), Q[1], fma2(dup<V>(A[d][2]), Q[2], f[d])));
+          if constexpr (W)
+            x[1][d] = fma2(dup<V>(w * psi3[0] * A[d][0]), P[0],
+                           fma2(dup<V>(w * psi3[1] * A[d][1]), P[1], mul2(dup<V>(w * psi3[2] * A[d][2]), P[2])));
+        }
+      }
+#pragma unroll
+      for (int d = 0; d < 3; ++d) x[0][d] = f[d];
+    };
+    if constexpr (NF == 2) {
+      const TetCoef<V, NN>* const fields[2] = {&U, &F};
+      sym_tet_orbits<V, NN, 2, W, 0>(fields, Y, Y2, node);
+    } else {
+      const TetCoef<V, NN>* const fields[1] = {&U};
+      sym_tet_orbits<V, NN, 1, W, 0>(fields, Y, Y2, node);
+    }
+  }
+  if (LAYER) __syncthreads();  // every P of a shared DoF has been read
+  if (act) {
+    tet_gather_back<V, NN>(Y, [&](int q, V y) { st(own(L.ys, L.yb, q), y); });
+    if constexpr (W) tet_gather_back<V, NN>(Y2, [&](int q, V y) { st(own(L.ws, L.wb, q), y); });
+    if (slot >= 0) sym_inject<NN, MODE, SG>(a, slot, e, s0 + ln, us, at, [&](int q) { return own(L.ys, L.yb, q); });
+  }
+  constexpr int B = 2;
+  SymRound<SG, B> first;
+  first.load(a, cd, cd.nsh + nb, s0, tid, M::NT);
+  __syncthreads();
+
+  float chk = 0.f;
+  sym_finish<3, NN, NS, MODE, LAYER, SG, B>(a, cd, L, sm, s0, tid, first, chk);
+  if (!(chk == 0.f)) atomicOr(a.status, 1);
+}
+
+}  // namespace fwi

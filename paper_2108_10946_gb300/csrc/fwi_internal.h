@@ -5,6 +5,10 @@
 
 namespace fwi {
 
+// Most elements of a chunk by element (nodes NN), and the stride of a chunk's tables: about as
+// many DoFs per chunk for every degree.
+constexpr int sym_pe(int dim, int nn) { return dim == 2 ? (nn == 7 ? 128 : nn == 12 ? 64 : nn == 18 ? 64 : 32) : nn == 15 ? 64 : 32; }
+
 // Element-kernel arguments (one step of the forward, recompute or adjoint recurrence).
 // Layouts (S = shots of the batch, stored shot-interleaved so that the lanes of one
 // element read one contiguous run of S floats):
@@ -17,12 +21,6 @@ namespace fwi {
 //                   e >= E0 (indexed e - E0)
 //   pidx   [N] index into the layer arrays or -1
 //   P, Pacc          [Nl][D][S], Y / Yacc [Nl][S] (3D)
-// Stored forward-field gradients (triangles, persistent kernel): per (chunk without layer
-// elements, group of 4 shots) item and node, 4 shots x 32 elements x 2 directions.
-constexpr int kGstoreNodeFloats = 256;
-inline size_t gstore_level_floats(int nch0, int S, int NN) {
-  return (size_t)nch0 * (size_t)(S / 4) * (size_t)NN * kGstoreNodeFloats;
-}
 
 struct StepArgs {
   int E, E0, S, Ns, N;
@@ -38,6 +36,16 @@ struct StepArgs {
   const int* chunks;         // [nch][6]: e0, ne, own_lo, own_n, nsh, halo_ptr
   const int* halo;           // halo DoF ids, chunk by chunk
   const unsigned short* lconn;  // [NS][Es] chunk-local index of each shared node
+  // symmetry-adapted chunk kernels (chunk_sym.cuh): chunk descriptors [nch][8] (e0, ne, first
+  // owned DoF, owned shared DoFs, halo list and its length, tables and their floats); the tables,
+  // chunk by chunk, 16-bit: table position [NS][PE] of every shared node, the incidence lists
+  // (node * PE + element), their pointers (PE = sym_pe)
+  const int* sdesc;
+  const unsigned short* smeta;
+  int ch1, wave;                // one past the last chunk of a launch; CTAs that run at a time
+  const unsigned char* splain;  // [nch] 1: c1 = 1 and c3 = 0 for every owned DoF
+  int T_max, SH_max;   // largest chunk table and most shared DoFs of a chunk
+  int p_own, p_halo;   // layer index of an owned / halo DoF of a layer chunk: dof - shift
   int tc;              // chunked layout, 2D: element contraction on the tensor cores
   int tc_wait_limit;   // polls of each bounded mbarrier wait of the tensor-core kernel
   int mode;            // 0 forward, 1 adjoint (with gradient when ring != null)
@@ -52,7 +60,11 @@ struct StepArgs {
   const float* cf;     // [3][N]: c1, c2, c3 of the increment update
   const int* pidx;     // [N]
   const float* lcf;    // [Nl][LCF] layer coefficients (see layer_coef_layout)
+  const float* lpsi;   // of the layer DoFs: 2D [Nl] Psi2_xx c^2 = -Psi2_zz c^2; 3D [Nl][4] sigma
+  const float* lcs;    // [Nl][8 or 12] the update's layer coefficients (chunk_sym.cuh)
+  int comb;            // 3D forward: Pacc holds Psi2 c^2 G u - Psi3 c^2 G omega in one sum
   float* u;
+  float* u_out;        // where u^{n+1} goes (symmetry-adapted kernels; u itself elsewhere)
   float* v;
   float* r;
   float* P;
@@ -75,8 +87,6 @@ struct StepArgs {
   const float* ring_u;     // forward U^m [N][S] (null: no gradient this step)
   float* gseg;             // FP32 segment accumulator: [S][N] per shot, or [N] summed
   int grad_lanes;          // 1: per-shot gradient accumulators, 0: summed over the shots
-  float* gstore;           // forward steps: write the forward field's (Ghat grad u) here
-  const float* gload;      // gradient steps: read it back (persistent kernel, triangles)
   int* status;             // bit 0: non-finite value seen; bit 1: a bounded wait gave up
 };
 
@@ -90,10 +100,17 @@ struct StepArgs {
 //            6D+2: dt detPsi1; 6D+3: dt / M
 inline int layer_coef_count(int dim) { return dim == 2 ? 4 * 2 : 6 * 3 + 4; }
 
+// Entry points of one symmetry-adapted unit (sym_inst.cu).
+struct SymKernels {
+  int (*upload)(const float* w, const float* sym, int nsym);
+  int (*launch)(const StepArgs& a, cudaStream_t st, cudaStream_t st_layer);
+};
+
 // Per-(dim,k) entry points, defined in the instantiation units.
 struct KernelSet {
   int dim, k, nn, ns, ni;
-  int (*upload_constants)(const float* dhat, const float* w);  // [D][NN][NN], [NN]
+  // dhat [D][NN][NN], w [NN], sym [nsym] (kmvtab::sym_tables)
+  int (*upload_constants)(const float* dhat, const float* w, const float* sym, int nsym);
   void (*launch_step)(const StepArgs& a, cudaStream_t st);        // plain layout
   // chunked layout: chunks without layer elements on st, layer chunks on st_layer (the two
   // launches are independent and may overlap; st_layer may be st)

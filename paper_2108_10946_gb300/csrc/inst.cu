@@ -25,11 +25,16 @@ __constant__ float c_w[NN];
 }  // namespace fwi
 
 #include "step_kernel.cuh"
-#include "chunk_kernel.cuh"
 #if KMV_DIM == 2
 #include "chunk_tc.cuh"
-#include "chunk_persist.cuh"
 #endif
+
+#define SYM_CAT2(a, b, c, d) a##b##_##c##_##d
+#define SYM_CAT(a, b, c, d) SYM_CAT2(a, b, c, d)
+namespace fwi {
+extern const SymKernels SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 1), SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 2),
+    SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 4);
+}
 
 namespace fwi {
 namespace {
@@ -39,34 +44,6 @@ __device__ __align__(16) float g_bimg[TcShape<D, NN>::BIMG];
 #endif
 
 __global__ void __launch_bounds__(128) k_step(const StepArgs a) { step_body<D, NN, NS>(a); }
-
-template <int MODE, bool LAYER>
-__global__ void __launch_bounds__(128) k_chunk(const StepArgs a) {
-  extern __shared__ float smem[];
-  chunk_body<D, NN, NS, MODE, LAYER>(a, smem);
-}
-
-template <int MODE, bool LAYER>
-int launch_chunk_t(const StepArgs& a, int ch0, int nch, cudaStream_t st) {
-  if (nch <= 0) return 0;
-  const size_t bytes =
-      chunk_smem_floats(a.L_max, a.SG, D, MODE == 2, LAYER, NN, NS, a.PE * a.SG) * sizeof(float);
-  if (bytes > 227 * 1024) return (int)cudaErrorInvalidValue;
-  static size_t configured[64] = {0};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (bytes > 48 * 1024 && dev < 64 && bytes > configured[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(k_chunk<MODE, LAYER>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) return (int)e;
-    configured[dev] = bytes;
-  }
-  StepArgs b = a;
-  b.ch0 = ch0;
-  dim3 grid((unsigned)nch, (unsigned)(a.S / a.SG));
-  k_chunk<MODE, LAYER><<<grid, a.PE * a.SG * chunk_qsplit<D, NN, MODE, LAYER>(), bytes, st>>>(b);
-  return 0;
-}
 
 #if KMV_DIM == 2
 template <int MODE, bool LAYER>
@@ -107,47 +84,6 @@ int launch_chunk_tc_t(const StepArgs& a, int ch0, int nch, cudaStream_t st) {
 
 #endif
 
-#if KMV_DIM == 2
-template <int MODE>
-__global__ void __launch_bounds__(PT_THREADS, 2) k_chunk_pt(const StepArgs a, int nwork) {
-  extern __shared__ __align__(16) char smem_pt[];
-  pt_body<NN, NS, MODE>(a, smem_pt, nwork);
-}
-
-// Persistent pipelined kernel over chunks [ch0, ch0 + nch) (no layer elements), S a
-// multiple of 4. Returns -1 (nothing launched) when its shared-memory tables do not fit, a
-// cudaError_t on failure, 0 once launched.
-template <int MODE>
-int launch_chunk_pt_t(const StepArgs& a, int ch0, int nch, cudaStream_t st) {
-  if (nch <= 0) return 0;
-  const PtLayout L = pt_layout<NN, NS>(a.L_max, a.O_max, a.H_max, MODE == 2);
-  if (L.total > 227u * 1024u) return -1;
-  static size_t configured[64] = {0};
-  static int per_sm[64] = {0}, nsm[64] = {0};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64) return (int)cudaErrorInvalidDevice;
-  if (L.total > configured[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(k_chunk_pt<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)L.total);
-    if (e != cudaSuccess) return (int)e;
-    configured[dev] = L.total;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[dev], k_chunk_pt<MODE>, PT_THREADS,
-                                                      L.total);
-    if (e != cudaSuccess) return (int)e;
-    e = cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return (int)e;
-  }
-  if (per_sm[dev] < 1) return -1;
-  const int nwork = nch * (a.S / PT_SG);
-  StepArgs b = a;
-  b.ch0 = ch0;
-  const int grid = std::min(nwork, per_sm[dev] * nsm[dev]);
-  k_chunk_pt<MODE><<<grid, PT_THREADS, L.total, st>>>(b, nwork);
-  return 0;
-}
-#endif
-
 // chunks [0, nch0) hold no damping-layer element, chunks [nch0, nch) do
 int launch_chunk(const StepArgs& a, cudaStream_t st, cudaStream_t stl) {
   const int mode = a.mode == 0 ? 0 : (a.ring_u != nullptr ? 2 : 1);
@@ -166,43 +102,13 @@ int launch_chunk(const StepArgs& a, cudaStream_t st, cudaStream_t stl) {
     return rc;
   }
 #endif
-#if KMV_DIM == 2
-  // triangles, four shots per work item: the persistent kernel takes the chunks without
-  // layer elements in the forward and adjoint steps, and in the gradient steps when the
-  // forward recompute stored the forward field's gradients (a.gload; summed gradient form);
-  // otherwise the gradient steps and the layer chunks use the chunk kernel. (The persistent
-  // kernel's gradient step needs more shared memory than its forward step, so if the forward
-  // step fell back to the chunk kernel, which stores nothing, so does the gradient step.)
-  if (a.S % PT_SG == 0 && a.nch0 > 0 && (mode != 2 || (a.gload != nullptr && !a.grad_lanes))) {
-    rc = mode == 0   ? launch_chunk_pt_t<0>(a, 0, a.nch0, st)
-         : mode == 1 ? launch_chunk_pt_t<1>(a, 0, a.nch0, st)
-                     : launch_chunk_pt_t<2>(a, 0, a.nch0, st);
-    if (rc > 0) return rc;
-    if (rc == 0) {
-      if (mode == 0) return launch_chunk_t<0, true>(a, a.nch0, a.nch - a.nch0, stl);
-      if (mode == 1) return launch_chunk_t<1, true>(a, a.nch0, a.nch - a.nch0, stl);
-      return launch_chunk_t<2, true>(a, a.nch0, a.nch - a.nch0, stl);
-    }
-    rc = 0;  // the tables do not fit: the chunk kernel below takes every chunk
-  }
-#endif
-  switch (mode) {
-    case 0:
-      rc = launch_chunk_t<0, false>(a, 0, a.nch0, st);
-      if (!rc) rc = launch_chunk_t<0, true>(a, a.nch0, a.nch - a.nch0, stl);
-      break;
-    case 1:
-      rc = launch_chunk_t<1, false>(a, 0, a.nch0, st);
-      if (!rc) rc = launch_chunk_t<1, true>(a, a.nch0, a.nch - a.nch0, stl);
-      break;
-    default:
-      rc = launch_chunk_t<2, false>(a, 0, a.nch0, st);
-      if (!rc) rc = launch_chunk_t<2, true>(a, a.nch0, a.nch - a.nch0, stl);
-  }
-  return rc;
+  return (a.SG == 4   ? SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 4)
+          : a.SG == 2 ? SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 2)
+                      : SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 1))
+      .launch(a, st, stl);
 }
 
-int upload(const float* dhat, const float* w) {
+int upload(const float* dhat, const float* w, const float* sym, int nsym) {
   cudaError_t e = cudaMemcpyToSymbol(c_dhat, dhat, sizeof(float) * D * NN * NN);
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w, w, sizeof(float) * NN);
 #if KMV_DIM == 2
@@ -212,7 +118,11 @@ int upload(const float* dhat, const float* w) {
     e = cudaMemcpyToSymbol(g_bimg, img.data(), sizeof(float) * img.size());
   }
 #endif
-  return (int)e;
+  int rc = (int)e;
+  if (!rc) rc = SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 1).upload(w, sym, nsym);
+  if (!rc) rc = SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 2).upload(w, sym, nsym);
+  if (!rc) rc = SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 4).upload(w, sym, nsym);
+  return rc;
 }
 
 void launch_step(const StepArgs& a, cudaStream_t st) {

@@ -16,6 +16,9 @@
 #include <array>
 #include <cmath>
 #include <cstring>
+#include <functional>
+
+#include "sym_layout.h"
 
 namespace kmvtab {
 namespace {
@@ -556,6 +559,333 @@ void fp32_tables(const Element& el, std::vector<float>& dhat32, std::vector<floa
   }
   std::vector<ld> wv(el.w.begin(), el.w.end());
   round_keeping(wv, A1, b1, m1, w32.data());
+}
+
+namespace {
+// Nodal pattern of each input coordinate of a triangle's field (inverse of tri_analyse) and
+// the coordinates of a nodal field (tri_analyse), in the order s1, s2, e1, e2.
+template <int NN>
+struct TriCoords {
+  using T = fwi::TriSym<NN>;
+  static constexpr int N = T::NA1 + T::NA2 + 2 * T::NV;
+  static constexpr int S1 = 0, S2 = T::NA1, E1 = S2 + T::NA2, E2 = E1 + T::NV;
+  static void of(const ld* u, ld* c) {
+    for (int o = 0; o < T::NO; ++o) {
+      const int i = T::vec(o);
+      if (T::kind(o) == 'C') {
+        c[S1 + o] = u[T::node(o, 0)];
+        continue;
+      }
+      ld p[3], m[3];
+      for (int v = 0; v < 3; ++v) {
+        const bool x = T::kind(o) == 'X';
+        const ld a = u[T::node(o, v, 0)], b = x ? u[T::node(o, v, 1)] : 0;
+        p[v] = a + b;
+        m[v] = a - b;
+      }
+      c[S1 + o] = p[0] + p[1] + p[2];
+      c[E1 + i] = p[0] - (p[1] + p[2]) / 2;
+      c[E2 + i] = p[1] - p[2];
+      if (T::kind(o) == 'X') {
+        c[S2 + T::odd(o)] = m[0] + m[1] + m[2];
+        c[E1 + i + 1] = (m[2] - m[1]) * 3 / 4;
+        c[E2 + i + 1] = m[0] - (m[1] + m[2]) / 2;
+      }
+    }
+  }
+  static void back(const ld* c, ld* u) {
+    for (int o = 0; o < T::NO; ++o) {
+      const int i = T::vec(o);
+      if (T::kind(o) == 'C') {
+        u[T::node(o, 0)] = c[S1 + o];
+        continue;
+      }
+      const ld s = c[S1 + o] / 3, a = c[E1 + i] * 2 / 3, b = c[E2 + i] / 2;
+      const ld p[3] = {s + a, s - a / 2 + b, s - a / 2 - b};
+      ld m[3] = {0, 0, 0};
+      const bool x = T::kind(o) == 'X';
+      if (x) {
+        const ld ms = c[S2 + T::odd(o)] / 3, mb = c[E2 + i + 1] * 2 / 3, ma = c[E1 + i + 1] * 2 / 3;
+        m[0] = ms + mb;
+        m[1] = ms - mb / 2 - ma;
+        m[2] = ms - mb / 2 + ma;
+      }
+      for (int v = 0; v < 3; ++v) {
+        u[T::node(o, v, 0)] = x ? (p[v] + m[v]) / 2 : p[v];
+        if (x) u[T::node(o, v, 1)] = (p[v] - m[v]) / 2;
+      }
+    }
+  }
+};
+
+// Coordinates (S, E1, E2) of an output three-vector (inverse of the assembly in tri_out).
+void tri_out_coords(const ld* x, bool odd, ld* c) {
+  c[0] = (x[0] + x[1] + x[2]) / 3;
+  c[1] = odd ? (x[2] - x[1]) / 2 : x[0] - c[0];
+  c[2] = odd ? x[0] - c[0] : (x[1] - x[2]) * 2 / 3;
+}
+
+template <int NN>
+bool tri_sym_tables(const Element& el, std::vector<float>& tab, std::string& err) {
+  using T = fwi::TriSym<NN>;
+  using C = TriCoords<NN>;
+  // the layout's node order is the element's
+  for (int o = 0; o < T::NO; ++o)
+    for (int v = 0; v < 3; ++v) {
+      const double* b0 = &el.bary[(size_t)T::node(o, v, 0) * 3];
+      const double* b1 = &el.bary[(size_t)T::node(o, v, T::kind(o) == 'X') * 3];
+      const int w = (v + 1) % 3, z = (v + 2) % 3;
+      bool ok = std::fabs(b0[v] - b1[v]) < 1e-12 && std::fabs(b0[w] - b1[z]) < 1e-12 &&
+                std::fabs(b0[z] - b1[w]) < 1e-12;
+      if (v > 0) {  // the orbit's generator, rotated
+        const double* g = &el.bary[(size_t)T::node(o, 0, 0) * 3];
+        ok = ok && std::fabs(b0[v] - g[0]) < 1e-12 && std::fabs(b0[w] - g[1]) < 1e-12;
+      }
+      if (!ok) {
+        err = "node order is not the symmetry layout's";
+        return false;
+      }
+    }
+  // derivatives in the frames: row (v, radial / tangential) of node q
+  const ld fr[3][2][2] = {{{-0.5L, -0.5L}, {1, -1}}, {{1, -0.5L}, {0, 1}}, {{-0.5L, 1}, {-1, 0}}};
+  auto deriv = [&](const ld* u, int q, int v, int k) {
+    ld s = 0;
+    for (int d = 0; d < 2; ++d) {
+      ld g = 0;
+      for (int j = 0; j < NN; ++j) g += (ld)el.dhat[((size_t)d * NN + q) * NN + j] * u[j];
+      s += fr[v][k][d] * g;
+    }
+    return s;
+  };
+  // output three-vectors of a nodal field, in table order
+  struct Out {
+    bool odd, centroid;
+    ld c[3];
+  };
+  auto outputs = [&](const ld* u) {
+    std::vector<Out> out;
+    for (int o = 0; o < T::NO; ++o) {
+      if (T::kind(o) == 'C') {
+        Out x{false, true, {0, deriv(u, T::node(o, 0), 0, 0), deriv(u, T::node(o, 0), 0, 1)}};
+        out.push_back(x);
+        continue;
+      }
+      for (int k = 0; k < 2; ++k) {
+        ld a[3], b[3];
+        for (int v = 0; v < 3; ++v) {
+          a[v] = deriv(u, T::node(o, v, 0), v, k);
+          b[v] = T::kind(o) == 'X' ? deriv(u, T::node(o, v, 1), v, k) : a[v];
+        }
+        for (int h = 0; h < (T::kind(o) == 'X' ? 2 : 1); ++h) {
+          ld x[3];
+          for (int v = 0; v < 3; ++v) x[v] = h == 0 ? (a[v] + b[v]) / 2 : (a[v] - b[v]) / 2;
+          // radial sums are even and differences odd; tangential the other way round
+          Out r{(k == 1) != (h == 1), false, {0, 0, 0}};
+          tri_out_coords(x, r.odd, r.c);
+          out.push_back(r);
+        }
+      }
+    }
+    return out;
+  };
+  std::vector<std::vector<Out>> resp(C::N);
+  for (int i = 0; i < C::N; ++i) {
+    ld c[C::N] = {0}, u[NN];
+    c[i] = 1;
+    C::back(c, u);
+    resp[i] = outputs(u);
+  }
+  // polynomials of degree <= 2 by the representation of their coordinates: 1 and r^2 are
+  // invariant; x and x^2 - y^2 are first components of vectors (equilateral coordinates)
+  ld inv[2][C::N], vec[2][C::N];
+  {
+    ld f[4][NN];
+    for (int q = 0; q < NN; ++q) {
+      const double* b = &el.bary[(size_t)q * 3];
+      const ld X = (ld)b[0] - ((ld)b[1] + b[2]) / 2, Y = sqrtl(3.0L) / 2 * ((ld)b[1] - b[2]);
+      f[0][q] = 1;
+      f[1][q] = X * X + Y * Y;
+      f[2][q] = X;
+      f[3][q] = X * X - Y * Y;
+    }
+    C::of(f[0], inv[0]);
+    C::of(f[1], inv[1]);
+    C::of(f[2], vec[0]);
+    C::of(f[3], vec[1]);
+  }
+  tab.clear();
+  ld worst = 0;
+  auto row = [&](const std::vector<int>& in, int r, int comp, const ld (*poly)[C::N], int npoly) {
+    const int n = (int)in.size();
+    std::vector<ld> x(n), A((size_t)npoly * n), b(npoly, 0);
+    for (int j = 0; j < n; ++j) x[j] = resp[in[j]][r].c[comp];
+    for (int p = 0; p < npoly; ++p)
+      for (int j = 0; j < n; ++j) {
+        A[(size_t)p * n + j] = poly[p][in[j]];
+        b[p] += x[j] * poly[p][in[j]];
+      }
+    std::vector<float> out(n);
+    if (n > 0) round_keeping(x, A, b, npoly, out.data());
+    tab.insert(tab.end(), out.begin(), out.end());
+  };
+  std::vector<int> i1, i2, iv;
+  for (int i = 0; i < T::NA1; ++i) i1.push_back(C::S1 + i);
+  for (int i = 0; i < T::NA2; ++i) i2.push_back(C::S2 + i);
+  for (int i = 0; i < T::NV; ++i) iv.push_back(C::E1 + i);
+  for (size_t r = 0; r < resp[0].size(); ++r) {
+    const bool odd = resp[0][r].odd, cen = resp[0][r].centroid;
+    for (int i = 0; i < C::N; ++i)
+      for (int c = 0; c < 3; ++c) {  // every other block vanishes; both vector components agree
+        const bool s1 = i < C::S2, s2 = i >= C::S2 && i < C::E1, e1 = i >= C::E1 && i < C::E2;
+        ld want = 0;
+        if (c == 0 && !cen && ((s1 && !odd) || (s2 && odd))) continue;
+        if (c == 1 && e1) continue;
+        if (c == 2 && i >= C::E2) want = resp[i - T::NV][r].c[1];
+        worst = std::max(worst, std::fabs(resp[i][r].c[c] - want));
+      }
+    if (!cen) row(odd ? i2 : i1, (int)r, 0, inv, odd ? 0 : 2);
+    row(iv, (int)r, 1, vec, 2);
+  }
+  if (!(worst < 1e-9L) || (int)tab.size() != T::TAB) {
+    err = "the derivative matrices do not have the layout's symmetry";
+    return false;
+  }
+  return true;
+}
+// The tetrahedron's table: the derivative along axis 1 of the cube, output by output.
+template <int NN>
+bool tet_sym_tables(const Element& el, std::vector<float>& tab, std::string& err) {
+  using T = fwi::TetSym<NN>;
+  const int swap[4][4] = {{0, 1, 2, 3}, {1, 0, 3, 2}, {2, 3, 0, 1}, {3, 2, 1, 0}};
+  const int size[3] = {4, 2, 1};
+  auto nodes = [&](int o) { return size[T::kind(o) == 'R' ? 0 : T::kind(o) == 'P' ? 1 : 2]; };
+  auto chi = [](int x, int h) { return x == 0 || h == 0 || h == x ? 1 : -1; };
+  for (int o = 0; o < T::NO; ++o)  // the layout's node order is the element's
+    for (int h = 0; h < 4; ++h) {
+      // a 'P' orbit's two nodes are swapped by the turns about the other axes
+      const int i = nodes(o) == 4 ? h : nodes(o) == 2 ? (h != 0 && h != T::axis(o)) : 0;
+      for (int v = 0; v < 4; ++v)
+        if (std::fabs(el.bary[(size_t)T::node(o, 0) * 4 + v] - el.bary[(size_t)T::node(o, i) * 4 + swap[h][v]]) > 1e-12) {
+          err = "node order is not the symmetry layout's";
+          return false;
+        }
+    }
+  // nodal field of mode i of character x
+  struct Mode {
+    int x, i;
+    std::vector<ld> u;
+  };
+  std::vector<Mode> modes;
+  for (int x = 0; x < 4; ++x)
+    for (int o = 0; o < T::NO; ++o) {
+      if (!T::has(o, x)) continue;
+      Mode m{x, T::mode(o, x), std::vector<ld>(NN, 0)};
+      const int n = nodes(o);
+      for (int h = 0; h < n; ++h)
+        m.u[T::node(o, h)] = (ld)(n == 4 ? chi(x, h) : n == 2 && x ? 1 - 2 * h : 1) / n;
+      modes.push_back(m);
+    }
+  const ld ax[3][3] = {{0.25L, -0.25L, -0.25L}, {-0.25L, 0.25L, -0.25L}, {-0.25L, -0.25L, 0.25L}};
+  auto deriv = [&](const std::vector<ld>& u, int q, int d) {
+    ld s = 0;
+    for (int r = 0; r < 3; ++r) {
+      ld g = 0;
+      for (int j = 0; j < NN; ++j) g += (ld)el.dhat[((size_t)r * NN + q) * NN + j] * u[j];
+      s += ax[d][r] * g;
+    }
+    return s;
+  };
+  // output z of the derivative of u along axis d at orbit o
+  auto output = [&](const std::vector<ld>& u, int o, int d, int z) {
+    const int n = nodes(o);
+    ld s = 0;
+    for (int h = 0; h < n; ++h) s += (n == 4 ? chi(z, h) : n == 2 && z ? 1 - 2 * h : 1) * deriv(u, T::node(o, h), d);
+    return s / n;
+  };
+  // polynomials of degree <= 2 by character
+  std::vector<std::vector<ld>> poly[4];
+  {
+    const int sg[4][3] = {{1, 1, 1}, {1, -1, -1}, {-1, 1, -1}, {-1, -1, 1}};
+    auto add = [&](int x, std::function<ld(const ld*)> f) {
+      std::vector<ld> c(x ? T::M1 : T::M0, 0);
+      for (int o = 0; o < T::NO; ++o) {
+        if (!T::has(o, x)) continue;
+        const int n = nodes(o);
+        for (int h = 0; h < n; ++h) {
+          ld X[3] = {0, 0, 0};
+          for (int v = 0; v < 4; ++v)
+            for (int a = 0; a < 3; ++a) X[a] += (ld)el.bary[(size_t)T::node(o, h) * 4 + v] * sg[v][a];
+          c[T::mode(o, x)] += (n == 4 ? chi(x, h) : n == 2 && x ? 1 - 2 * h : 1) * f(X);
+        }
+      }
+      poly[x].push_back(c);
+    };
+    add(0, [](const ld*) { return 1.0L; });
+    for (int a = 0; a < 3; ++a) {
+      add(0, [a](const ld* X) { return X[a] * X[a]; });
+      add(a + 1, [a](const ld* X) { return X[a]; });
+      add(a + 1, [a](const ld* X) { return X[(a + 1) % 3] * X[(a + 2) % 3]; });
+    }
+  }
+  tab.assign(T::TAB, 0.f);
+  std::vector<ld> exact(T::TAB, 0);
+  std::vector<char> set(T::TAB, 0);
+  ld worst = 0;
+  for (int d = 0; d < 3; ++d)
+    for (int o = 0; o < T::NO; ++o)
+      for (int z = 0; z < nodes(o); ++z) {
+        const int y = T::kind(o) == 'P' ? (z ? (d + 1) ^ T::axis(o) : d + 1) : z ^ (d + 1);
+        std::vector<ld> row(y ? T::M1 : T::M0, 0);
+        for (const Mode& m : modes) {
+          const ld v = output(m.u, o, d, z);
+          if (m.x == y) row[m.i] = v;
+          else worst = std::max(worst, std::fabs(v));  // every other block vanishes
+        }
+        const int n = (int)row.size();
+        if (d == 0) {
+          const int np = (int)poly[y].size();
+          std::vector<ld> A((size_t)np * n), b(np, 0);
+          for (int p = 0; p < np; ++p)
+            for (int i = 0; i < n; ++i) {
+              A[(size_t)p * n + i] = poly[y][p][i];
+              b[p] += row[i] * poly[y][p][i];
+            }
+          std::vector<float> out(n);
+          round_keeping(row, A, b, np, out.data());
+          for (int i = 0; i < n; ++i) {
+            const int at = fwi::tet_at<NN>(o, 0, z, y, i);
+            tab[at] = out[i];
+            exact[at] = row[i];
+            set[at] = 1;
+          }
+        } else {  // the turn about the diagonal: axis 1's coefficients
+          for (int i = 0; i < n; ++i) worst = std::max(worst, std::fabs(exact[fwi::tet_at<NN>(o, d, z, y, i)] - row[i]));
+        }
+      }
+  for (char c : set)
+    if (!c) worst = 1;
+  if (!(worst < 1e-9L)) {
+    err = "the derivative matrices do not have the layout's symmetry";
+    return false;
+  }
+  return true;
+}
+}  // namespace
+
+bool sym_tables(const Element& el, std::vector<float>& tab, std::string& err) {
+  if (el.dim == 3 && el.n == 15) return tet_sym_tables<15>(el, tab, err);
+  if (el.dim == 3 && el.n == 32) return tet_sym_tables<32>(el, tab, err);
+  tab.clear();
+  if (el.dim == 2) {
+    switch (el.n) {
+      case 7: return tri_sym_tables<7>(el, tab, err);
+      case 12: return tri_sym_tables<12>(el, tab, err);
+      case 18: return tri_sym_tables<18>(el, tab, err);
+      case 30: return tri_sym_tables<30>(el, tab, err);
+    }
+  }
+  err = "no symmetry layout for this element";
+  return false;
 }
 
 void Element::basis(const double* x, double* phi) const {

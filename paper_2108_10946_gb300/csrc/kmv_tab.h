@@ -42,4 +42,11 @@ bool build(int dim, int k, Element& out, std::string& err);
 // and the weights integrate degree <= 1 (see kmv_tab.cpp).
 void fp32_tables(const Element& el, std::vector<float>& dhat32, std::vector<float>& w32);
 
+// The derivative matrices in the coordinates adapted to the element's symmetries (see
+// sym_layout.h, sym_tri.cuh), in the kernels' order, FP32: every row
+// keeps the derivatives of the polynomials of degree <= 2 like the rows of dhat32. Returns
+// false with a message if the node order is not the layout's or a block that has to vanish
+// does not.
+bool sym_tables(const Element& el, std::vector<float>& tab, std::string& err);
+
 }  // namespace kmvtab

@@ -36,8 +36,10 @@ __device__ __forceinline__ void dof_update_pre(const StepArgs& a, int dof, int s
       for (int k = 0; k < D; ++k) {
         const size_t pk = ((size_t)pi * D + k) * S + s;
         const float pold = po ? po[k] : a.P[pk];
-        float pn = __ldg(lc + L::E1 + k) * pold - __ldg(lc + L::E2F + k) * sU[k];
-        if constexpr (D == 3) pn += __ldg(lc + L::E3F + k) * sY[k];
+        float pn = __ldg(lc + L::E1 + k) * pold - __ldg(lc + (a.comb ? L::E2A : L::E2F) + k) * sU[k];
+        if constexpr (D == 3) {
+          if (!a.comb) pn += __ldg(lc + L::E3F + k) * sY[k];
+        }
         a.P[pk] = pn;
       }
       if constexpr (D == 3) {
@@ -181,7 +183,7 @@ __global__ void __launch_bounds__(256) node_kernel(const StepArgs a) {
         sU[d] = __ldcg(a.Pacc + pk);
         a.Pacc[pk] = 0.f;
         if constexpr (D == 3) {
-          if (a.mode == 0) {
+          if (a.mode == 0 && !a.comb) {
             sY[d] = __ldcg(a.PaccY + pk);
             a.PaccY[pk] = 0.f;
           }
@@ -235,6 +237,7 @@ __global__ void __launch_bounds__(256) node_kernel4(const StepArgs a) {
   vn.w = c1 * vo.w - c2 * y.w - c3 * uo.w;
   if (pi >= 0) {
     const float* lc = a.lcf + (size_t)pi * L::COUNT;
+    const bool sep = a.mode == 0 && !a.comb;  // omega's gradient in a sum of its own (3D)
     float4 sU[D], sY[D], Po[D];
     float e1[D], e2[D], e3[D];
 #pragma unroll
@@ -244,11 +247,11 @@ __global__ void __launch_bounds__(256) node_kernel4(const StepArgs a) {
       Po[k] = ld4(a.P + pk);
       sY[k] = make_float4(0.f, 0.f, 0.f, 0.f);
       if constexpr (D == 3) {
-        if (a.mode == 0) sY[k] = ldcg4(a.PaccY + pk);
+        if (sep) sY[k] = ldcg4(a.PaccY + pk);
       }
       e1[k] = __ldg(lc + L::E1 + k);
-      e2[k] = __ldg(lc + (a.mode == 0 ? L::E2F : L::E2A) + k);
-      e3[k] = D == 3 && a.mode == 0 ? __ldg(lc + L::E3F + k) : 0.f;
+      e2[k] = __ldg(lc + (a.mode == 0 && !a.comb ? L::E2F : L::E2A) + k);
+      e3[k] = D == 3 && sep ? __ldg(lc + L::E3F + k) : 0.f;
     }
     float4 Yo = make_float4(0.f, 0.f, 0.f, 0.f), yw = Yo;
     float cy0 = 0.f, cy1 = 0.f, cy2 = 0.f;
@@ -267,13 +270,13 @@ __global__ void __launch_bounds__(256) node_kernel4(const StepArgs a) {
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         float x = e1[k] * comp(Po[k], c) - e2[k] * comp(sU[k], c);  // e2: E2F or E2A
-        if (D == 3 && a.mode == 0) x += e3[k] * comp(sY[k], c);
+        if (D == 3 && sep) x += e3[k] * comp(sY[k], c);
         setc(pn, c, x);
       }
       st4(a.P + pk, pn);
       st4(a.Pacc + pk, make_float4(0.f, 0.f, 0.f, 0.f));
       if constexpr (D == 3) {
-        if (a.mode == 0) st4(a.PaccY + pk, make_float4(0.f, 0.f, 0.f, 0.f));
+        if (sep) st4(a.PaccY + pk, make_float4(0.f, 0.f, 0.f, 0.f));
       }
     }
     if constexpr (D == 3) {
