@@ -20,6 +20,7 @@
 #include "../../include/fwi.h"
 #include "fwi_internal.h"
 #include "kmv_tab.h"
+#include "sym_layout.h"
 
 using fwi::StepArgs;
 
@@ -537,14 +538,15 @@ void build_incidence(fwi_mesh* m) {
     const size_t at = m->smeta.size(), size = (size_t)2 * ns * P + (nloc + 8) / 8 * 8;
     m->smeta.resize(at + size, 0);
     uint16_t *lq = &m->smeta[at], *ge = lq + ns * P, *gp = ge + ns * P;
-    auto place = [&](int q, int e) {  // list of node q of element e
-      const int l = m->lconn[(size_t)q * m->Es + e];
+    auto node = [&](int j) { return fwi::sym_slot_node(m->dim, m->nn, j); };
+    auto place = [&](int j, int e) {  // list of the node at slot j of element e
+      const int l = m->lconn[(size_t)node(j) * m->Es + e];
       return l < nsh ? l : l - (own_n - nsh);
     };
     cnt.assign(nloc + 1, 0);
     for (int q = 0; q < ns; ++q)
       for (int e = e0; e < e0 + ne; ++e) {
-        lq[q * P + e - e0] = m->lconn[(size_t)q * m->Es + e];
+        lq[q * P + e - e0] = m->lconn[(size_t)node(q) * m->Es + e];
         cnt[place(q, e) + 1]++;
       }
     for (int l = 0; l < nloc; ++l) cnt[l + 1] += cnt[l];

@@ -666,6 +666,59 @@ __device__ __forceinline__ void sym_tet_orbits(const TetCoef<V, NN>* const (&U)[
   }
 }
 
+// The same walk rolled (KMV3: all orbits are alike; node slots 4 o + h). The unrolled code of the
+// layer kernels, some 7,000 instructions, does not fit the instruction caches.
+template <class V, int N, bool DIV2, class F>
+__device__ __forceinline__ void sym_tet_roll(const TetCoef<V, 32>* const (&U)[N], TetCoef<V, 32>& Y, TetCoef<V, 32>& Y2,
+                                             F node) {
+  constexpr int NG = N > 1 || !DIV2 ? N : 2;
+#pragma unroll 1
+  for (int o = 0; o < 8; ++o) {
+    const float* t = c_sym + o * 96;  // [axis][output][mode] of this orbit
+    V g[NG][3][4];
+#pragma unroll
+    for (int f = 0; f < N; ++f)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          V s = mul2(dup<V>(t[(d * 4 + z) * 8]), U[f]->at(z ^ (d + 1), 0));
+#pragma unroll
+          for (int i = 1; i < 8; ++i) s = fma2(dup<V>(t[(d * 4 + z) * 8 + i]), U[f]->at(z ^ (d + 1), i), s);
+          g[f][d][z] = s;
+        }
+        tet_butterfly(g[f][d]);
+      }
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      V x[NG][3];
+#pragma unroll
+      for (int f = 0; f < N; ++f)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) x[f][d] = g[f][d][h];
+      node(4 * o + h, x);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        g[0][d][h] = x[0][d];
+        if constexpr (DIV2) g[1][d][h] = x[1][d];
+      }
+    }
+#pragma unroll
+    for (int f = 0; f < 1 + DIV2; ++f) {
+      TetCoef<V, 32>& y = f == 0 ? Y : Y2;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        tet_butterfly(g[f][d]);
+#pragma unroll
+        for (int z = 0; z < 4; ++z)
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            y.at(z ^ (d + 1), i) = fma2(dup<V>(t[(d * 4 + z) * 8 + i]), g[f][d][z], y.at(z ^ (d + 1), i));
+      }
+    }
+  }
+}
+
 // One step of a tetrahedra chunk. Fields: u; the forward field (gradient steps); omega (forward
 // steps in the layer).
 template <int NN, int NS, int MODE, bool LAYER, int SG>
@@ -706,25 +759,35 @@ __device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
   const float* us = sm + L.u + sym_shift(a.u + i0) + ln;
   const float* cs = sm + L.c2 + sym_shift(a.c2 + cd.own);
   const int ps = el * SG + ln, pb = el * NI * SG + ln;  // a thread's own places (see sym_tri_body)
-  auto at = [&](int q) { return q < NS ? (int)lq[q * PE] : bub + (q - NS); };
+  // q: a node's slot (sym_slot_node: the local node, at KMV3 orbit by orbit)
+  constexpr bool ROLL = NN == 32;
+  auto bi = [](int q) { return ROLL ? NN - 1 - q : q - NS; };  // a bubble's place in its element
+  auto at = [&](int q) { return q < NS ? (int)lq[q * PE] : bub + bi(q); };
   auto ld = [&](const float* p) { return *reinterpret_cast<const V*>(p); };
   auto st = [&](float* p, V v) { *reinterpret_cast<V*>(p) = v; };
-  auto own = [&](int s, int b, int q) { return sm + (q < NS ? s + ps + q * PE * SG : b + pb + (q - NS) * SG); };
+  auto own = [&](int s, int b, int q) { return sm + (q < NS ? s + ps + q * PE * SG : b + pb + bi(q) * SG); };
+  auto slot_of = [](int q) {  // (q and the loop are compile-time once unrolled)
+    int j = 0;
+#pragma unroll
+    for (int i = 0; i < NN; ++i)
+      if (sym_slot_node(3, NN, i) == q) j = i;
+    return j;
+  };
   TetCoef<V, NN> Y, Y2;
   if (act) {
     TetCoef<V, NN> U, F;
     if constexpr (GRAD) {
       const float* fs = sm + L.f + sym_shift(a.ring_u + i0) + ln;
-      tet_analyse<V, NN>(F, [&](int q) { return ld(fs + at(q) * SG); });
+      tet_analyse<V, NN>(F, [&](int q) { return ld(fs + at(slot_of(q)) * SG); });
     }
     if constexpr (OM) {
       const float* om = sm + L.om + sym_shift(a.Y + pi0 * S + s0) + ln;
-      tet_analyse<V, NN>(F, [&](int q) { return ld(om + at(q) * SG); });
+      tet_analyse<V, NN>(F, [&](int q) { return ld(om + at(slot_of(q)) * SG); });
     }
     const float* p1 = sm + L.p1 + (LAYER ? sym_shift(a.P + (pi0 * S + s0) * 3) : 0) + ln;
     float* p2 = sm + L.sb + (LAYER ? sym_shift(a.P + ((pi0 + cd.nsh) * S + s0) * 3) : 0) + el * NI * 3 * SG + ln;
     const float* sig = sm + L.ps + (LAYER ? sym_shift(a.lpsi + pi0 * 4) : 0);
-    tet_analyse<V, NN>(U, [&](int q) { return ld(us + at(q) * SG); });
+    tet_analyse<V, NN>(U, [&](int q) { return ld(us + at(slot_of(q)) * SG); });
     tet_zero(Y);
     if constexpr (W) tet_zero(Y2);
     // one node: x[0] in are the field's derivatives, out the flux (x[1]: the other field's; out, in
@@ -744,7 +807,7 @@ __device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
         const float s1 = sig[4 * l], s2 = sig[4 * l + 1], s3 = sig[4 * l + 2], tr = s1 + s2 + s3;
         const float psi2[3] = {c2 * (2.f * s1 - tr), c2 * (2.f * s2 - tr), c2 * (2.f * s3 - tr)};
         const float psi3[3] = {c2 * s2 * s3, c2 * s1 * s3, c2 * s1 * s2};
-        float* p = q < NS ? const_cast<float*>(p1) + (l - (l >= cd.nsh ? nb : 0)) * 3 * SG : p2 + (q - NS) * 3 * SG;
+        float* p = q < NS ? const_cast<float*>(p1) + (l - (l >= cd.nsh ? nb : 0)) * 3 * SG : p2 + bi(q) * 3 * SG;
         V P[3], Q[3], s[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -772,17 +835,22 @@ __device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
     };
     if constexpr (NF == 2) {
       const TetCoef<V, NN>* const fields[2] = {&U, &F};
-      sym_tet_orbits<V, NN, 2, W, 0>(fields, Y, Y2, node);
+      if constexpr (ROLL) sym_tet_roll<V, 2, W>(fields, Y, Y2, node);
+      else sym_tet_orbits<V, NN, 2, W, 0>(fields, Y, Y2, node);
     } else {
       const TetCoef<V, NN>* const fields[1] = {&U};
-      sym_tet_orbits<V, NN, 1, W, 0>(fields, Y, Y2, node);
+      if constexpr (ROLL) sym_tet_roll<V, 1, W>(fields, Y, Y2, node);
+      else sym_tet_orbits<V, NN, 1, W, 0>(fields, Y, Y2, node);
     }
   }
   if (LAYER) __syncthreads();  // every P of a shared DoF has been read
   if (act) {
-    tet_gather_back<V, NN>(Y, [&](int q, V y) { st(own(L.ys, L.yb, q), y); });
-    if constexpr (W) tet_gather_back<V, NN>(Y2, [&](int q, V y) { st(own(L.ws, L.wb, q), y); });
-    if (slot >= 0) sym_inject<NN, MODE, SG>(a, slot, e, s0 + ln, us, at, [&](int q) { return own(L.ys, L.yb, q); });
+    tet_gather_back<V, NN>(Y, [&](int q, V y) { st(own(L.ys, L.yb, slot_of(q)), y); });
+    if constexpr (W) tet_gather_back<V, NN>(Y2, [&](int q, V y) { st(own(L.ws, L.wb, slot_of(q)), y); });
+    if (slot >= 0)
+      sym_inject<NN, MODE, SG>(
+          a, slot, e, s0 + ln, us, [&](int q) { return at(c_slot[q]); },
+          [&](int q) { return own(L.ys, L.yb, c_slot[q]); });
   }
   constexpr int B = 2;
   SymRound<SG, B> first;

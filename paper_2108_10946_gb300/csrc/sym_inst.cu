@@ -11,7 +11,8 @@ constexpr int NN = D == 2 ? (KMV_K == 2 ? 7 : KMV_K == 3 ? 12 : KMV_K == 4 ? 18 
                           : (KMV_K == 2 ? 15 : 32);
 constexpr int NS = D == 2 ? 3 * KMV_K : (KMV_K == 2 ? 14 : 28);
 constexpr int SG = KMV_SG;
-constexpr int NSYM = 320;
+constexpr int NSYM = D == 3 && NN == 32 ? 768 : 300;
+__constant__ int c_slot[NN];  // slot of every local node (sym_slot_node)
 __constant__ float c_sym[NSYM];
 __constant__ float2 c_sym2[NSYM];  // every coefficient twice: operands of packed multiply-adds
 // Shots per thread of groups of two and four: pairs issue half the instructions, but at KMV5 a
@@ -90,11 +91,26 @@ int launch(const StepArgs& a, cudaStream_t st, cudaStream_t stl) {
 
 int upload(const float* w, const float* sym, int nsym) {
   if (nsym > NSYM) return (int)cudaErrorInvalidValue;
+  float tab[NSYM] = {0.f}, ws[NN];
   float2 dup[NSYM];
-  for (int i = 0; i < nsym; ++i) dup[i] = make_float2(sym[i], sym[i]);
-  cudaError_t e = cudaMemcpyToSymbol(c_w, w, sizeof(float) * NN);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_sym, sym, sizeof(float) * nsym);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_sym2, dup, sizeof(float2) * nsym);
+  int slot[NN];
+  for (int i = 0; i < nsym; ++i) tab[i] = sym[i];
+  if constexpr (D == 3 && NN == 32)  // the rolled loop's table: every axis, [orbit][axis][output][mode]
+    for (int o = 0; o < 8; ++o)
+      for (int i = 0; i < 96; ++i) {
+        const int d = i / 32, z = i / 8 % 4;
+        tab[o * 96 + i] = sym[tet_at<NN>(o, d, z, z ^ (d + 1), i % 8)];
+      }
+  for (int i = 0; i < NSYM; ++i) dup[i] = make_float2(tab[i], tab[i]);
+  for (int j = 0; j < NN; ++j) {
+    const int q = sym_slot_node(D, NN, j);
+    slot[q] = j;
+    ws[j] = w[q];
+  }
+  cudaError_t e = cudaMemcpyToSymbol(c_w, ws, sizeof ws);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_slot, slot, sizeof slot);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_sym, tab, sizeof tab);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_sym2, dup, sizeof dup);
   return (int)e;
 }
 }  // namespace
