@@ -133,6 +133,7 @@ struct fwi_mesh {
   std::vector<int32_t> sdesc;                     // [nch][8]
   std::vector<uint16_t> smeta;
   int T_max = 0, SH_max = 0;
+  int halo_layer = 0;         // first halo DoF of the layer (they are the last)
   int p_own = 0, p_halo = 0;  // layer index of an owned / halo DoF of the layer: DoF - shift
   std::vector<double> verts;
   std::vector<int32_t> cells;      // user order
@@ -833,6 +834,7 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
         }
       m->p_own = lo;
       m->p_halo = h0 - (m->N_own - lo);
+      m->halo_layer = h0;
       for (int i = lo; i < m->N_own; ++i) m->pidx[i] = i - m->p_own;
       for (int i = h0; i < N; ++i) m->pidx[i] = i - m->p_halo;
       m->Nl = (m->N_own - lo) + (N - h0);
@@ -1319,7 +1321,7 @@ StepArgs base_args(fwi_batch* b) {
     a.splain = m->d_splain;
     a.lpsi = m->d_lpsi;
     a.lcs = m->d_lcs;
-    a.comb = m->dim == 3 ? 1 : 0;
+    a.halo_layer = m->Nl > 0 ? m->halo_layer : m->N;
     a.T_max = m->T_max;
     a.SH_max = m->SH_max;
     a.p_own = m->p_own;

@@ -16,9 +16,10 @@
 //
 // Owned DoFs are read and written by this CTA only; halo DoFs are only read here.
 #pragma once
-#include "sym_tet.cuh"
-#include "update.cuh"
 #include <type_traits>
+
+#include "lanes.cuh"
+#include "sym_tet.cuh"
 
 namespace fwi {
 
@@ -87,61 +88,6 @@ __device__ __forceinline__ void sym_prefetch(const float* p, int n) {  // to L2
   if (r.bytes) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(r.src), "r"(r.bytes) : "memory");
 }
 
-template <int SG>
-struct alignas(4 * SG) Lanes {  // one DoF's values of SG consecutive shots
-  float x[SG];
-};
-template <int SG>
-__device__ __forceinline__ Lanes<SG> lanes_ld(const float* p) {
-  return *reinterpret_cast<const Lanes<SG>*>(p);
-}
-template <int SG>
-__device__ __forceinline__ void lanes_st(float* p, const Lanes<SG>& v) {
-  *reinterpret_cast<Lanes<SG>*>(p) = v;
-}
-template <int SG>
-__device__ __forceinline__ void lanes_add(float* p, const Lanes<SG>& v) {  // global, no result
-  if constexpr (SG == 4) atomicAdd(reinterpret_cast<float4*>(p), make_float4(v.x[0], v.x[1], v.x[2], v.x[3]));
-  else if constexpr (SG == 2) atomicAdd(reinterpret_cast<float2*>(p), make_float2(v.x[0], v.x[1]));
-  else atomicAdd(p, v.x[0]);
-}
-// y += z, and y = a y + b z, on every shot
-template <int SG>
-__device__ __forceinline__ void lanes_acc(Lanes<SG>& y, const Lanes<SG>& z) {
-  if constexpr (SG == 1) {
-    y.x[0] += z.x[0];
-  } else {
-#pragma unroll
-    for (int k = 0; k < SG; k += 2) {
-      const float2 t = add2(make_float2(y.x[k], y.x[k + 1]), make_float2(z.x[k], z.x[k + 1]));
-      y.x[k] = t.x;
-      y.x[k + 1] = t.y;
-    }
-  }
-}
-template <int SG>
-__device__ __forceinline__ Lanes<SG> lanes_fma(float a, const Lanes<SG>& x, const Lanes<SG>& y) {  // a x + y
-  Lanes<SG> r;
-  if constexpr (SG == 1) {
-    r.x[0] = fmaf(a, x.x[0], y.x[0]);
-  } else {
-#pragma unroll
-    for (int k = 0; k < SG; k += 2) {
-      const float2 t = fma2(dup<float2>(a), make_float2(x.x[k], x.x[k + 1]), make_float2(y.x[k], y.x[k + 1]));
-      r.x[k] = t.x;
-      r.x[k + 1] = t.y;
-    }
-  }
-  return r;
-}
-template <int SG>
-__device__ __forceinline__ Lanes<SG> lanes_mul(float a, const Lanes<SG>& x) {
-  Lanes<SG> r;
-#pragma unroll
-  for (int k = 0; k < SG; ++k) r.x[k] = a * x.x[k];
-  return r;
-}
-
 constexpr int SYM_PE = sym_pe(D, NN);  // most elements of a chunk, stride of its tables
 
 // A CTA's threads: one element for LANES shots each.
@@ -156,33 +102,35 @@ struct SymMap {
 struct SymSmem {
   int u, f, c2, ps, om, ys, yb, p1, gs, gb, ws, wb, ss, sb, ids, meta, total;
 };
-// Floats per DoF of the layer's nodal coefficients: Psi2 c^2 (2D adjoint), sigma (3D).
+// Floats per DoF of the layer's nodal coefficients in the table: Psi2 c^2 (2D adjoint; the three
+// sigma of a 3D DoF are read where they are used, the table would take the second CTA's room).
 template <int D, int MODE>
-__host__ __device__ constexpr int sym_psi() { return D == 3 ? 4 : MODE != 0 ? 1 : 0; }
+__host__ __device__ constexpr int sym_psi() { return D == 2 && MODE != 0 ? 1 : 0; }
 
 template <int D, int NN, int NS, int SG, int MODE, bool LAYER>
 __host__ __device__ inline SymSmem sym_smem(int T, int SH, int H) {
   constexpr int PE = SYM_PE, NI = NN - NS, NE = NS * PE * SG, NB = (NI * PE * SG + 3) / 4 * 4;
-  constexpr bool GRAD = MODE == 2;
+  constexpr bool GRAD = MODE == 2, L3 = LAYER && D == 3;
   auto up = [](int n) { return (n + 7) & ~3; };  // a multiple of 4 with room for a run's shift
+  auto most = [](int x, int y) { return x > y ? x : y; };
   SymSmem m{};
   int o = 4;  // the mbarrier
   m.u = o, o += up(T * SG);
-  m.f = o, o += GRAD ? up(T * SG) : 0;
+  m.f = o, o += GRAD && !L3 ? up(T * SG) : 0;
   m.c2 = o, o += up(T);
   m.ps = o, o += LAYER ? up(T * sym_psi<D, MODE>()) : 0;
-  m.om = o, o += LAYER && D == 3 && MODE == 0 ? up(T * SG) : 0;  // the omega state
   // the shared DoFs' layer auxiliaries P lie where the elements' sums go once all have read P (in
   // 2D gradient steps that place holds the forward field's derivatives)
   constexpr bool APART = GRAD && D == 2;
-  m.ys = o, m.yb = o + NE, m.p1 = o + (APART ? NE + NB : 0);
-  if (LAYER && APART) o += NE + NB + up(D * SH * SG);
-  else o += LAYER && up(D * SH * SG) > NE + NB ? up(D * SH * SG) : NE + NB;
+  constexpr int SUMS = (NE + NB) * (L3 && MODE != 0 ? 2 : 1);  // y, and the omega row's (3D adjoint)
+  m.ys = o, m.yb = o + NE, m.ws = o + NE + NB, m.wb = m.ws + NE, m.p1 = o + (APART ? SUMS : 0);
+  o += !LAYER ? SUMS : APART ? SUMS + up(D * SH * SG) : most(SUMS, up(D * SH * SG));
   m.gs = o, o += GRAD ? NE : 0;
   m.gb = o, o += GRAD ? NB : 0;
-  m.ws = o, o += LAYER && D == 3 && MODE != 0 ? NE : 0;  // the omega row's sums
-  m.wb = o, o += LAYER && D == 3 && MODE != 0 ? NB : 0;
-  m.ss = o, o += LAYER ? D * NE : 0;
+  // 3D: the second field (the forward field; omega in forward steps) lies where the layer sums go
+  m.om = m.ss = o;
+  if (L3 && GRAD) m.f = o;
+  o += LAYER ? most(D * NE, L3 && MODE != 1 ? up(T * SG) : 0) : 0;
   m.sb = o, o += LAYER ? up(D * NB) : 0;  // bubbles: P, then each (element, shot)'s own layer sums
   m.ids = o, o += up(H);
   m.meta = o, o += up(NS * PE + (SH + 16) / 2);  // table positions, incidence list, its pointers
@@ -258,6 +206,7 @@ __device__ __forceinline__ void sym_load(const StepArgs& a, const SymDesc& cd, c
       sym_prefetch(a.cf + 2 * (size_t)a.N + cd.own, on);
     }
     if (LAYER) sym_prefetch(a.lcs + pi0 * SYM_LCS<D>, on * SYM_LCS<D>);
+    if (LAYER && D == 3) sym_prefetch(a.lpsi + pi0 * 4, on * 4);
     if (LAYER && D == 3 && S == SG) sym_prefetch(a.Y + pi0 * SG, on * SG);
     // and the ranges of the chunk a wave of CTAs further on
     const int nc = blockIdx.x + a.ch0 + a.wave;
@@ -773,9 +722,8 @@ __device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
       if (sym_slot_node(3, NN, i) == q) j = i;
     return j;
   };
-  TetCoef<V, NN> Y, Y2;
+  TetCoef<V, NN> U, F, Y, Y2;
   if (act) {
-    TetCoef<V, NN> U, F;
     if constexpr (GRAD) {
       const float* fs = sm + L.f + sym_shift(a.ring_u + i0) + ln;
       tet_analyse<V, NN>(F, [&](int q) { return ld(fs + at(slot_of(q)) * SG); });
@@ -784,9 +732,13 @@ __device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
       const float* om = sm + L.om + sym_shift(a.Y + pi0 * S + s0) + ln;
       tet_analyse<V, NN>(F, [&](int q) { return ld(om + at(slot_of(q)) * SG); });
     }
+  }
+  if (LAYER && NF == 2) __syncthreads();  // the second field's place is the layer sums' from here
+  if (act) {
     const float* p1 = sm + L.p1 + (LAYER ? sym_shift(a.P + (pi0 * S + s0) * 3) : 0) + ln;
     float* p2 = sm + L.sb + (LAYER ? sym_shift(a.P + ((pi0 + cd.nsh) * S + s0) * 3) : 0) + el * NI * 3 * SG + ln;
-    const float* sig = sm + L.ps + (LAYER ? sym_shift(a.lpsi + pi0 * 4) : 0);
+    const int* ids = reinterpret_cast<const int*>(sm + L.ids);
+    const float4* sig = reinterpret_cast<const float4*>(a.lpsi);
     tet_analyse<V, NN>(U, [&](int q) { return ld(us + at(slot_of(q)) * SG); });
     tet_zero(Y);
     if constexpr (W) tet_zero(Y2);
@@ -804,7 +756,9 @@ __device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
         st(own(L.gs, L.gb, q), mul2(dup<V>(w), fma2(h0, x[1][0], fma2(h1, x[1][1], mul2(h2, x[1][2])))));
       V f[3] = {mul2(wc, h0), mul2(wc, h1), mul2(wc, h2)};
       if constexpr (LAYER) {
-        const float s1 = sig[4 * l], s2 = sig[4 * l + 1], s3 = sig[4 * l + 2], tr = s1 + s2 + s3;
+        const int on = cd.nsh + nb;
+        const float4 sg = __ldg(sig + (l < on ? (int)pi0 + l : ids[l - on] - a.p_halo));
+        const float s1 = sg.x, s2 = sg.y, s3 = sg.z, tr = s1 + s2 + s3;
         const float psi2[3] = {c2 * (2.f * s1 - tr), c2 * (2.f * s2 - tr), c2 * (2.f * s3 - tr)};
         const float psi3[3] = {c2 * s2 * s3, c2 * s1 * s3, c2 * s1 * s2};
         float* p = q < NS ? const_cast<float*>(p1) + (l - (l >= cd.nsh ? nb : 0)) * 3 * SG : p2 + bi(q) * 3 * SG;

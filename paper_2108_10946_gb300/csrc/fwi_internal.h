@@ -28,6 +28,7 @@ struct StepArgs {
                        // multiple of 32 (16-byte aligned rows for vector and cp.async loads)
   int log2S;
   int h0, hcnt;        // node kernel range: DoFs [h0, h0 + hcnt), r indexed from h0
+  int halo_layer;      // chunked layout: first halo DoF of the damping layer (they are the last)
   // chunked layout (layout 0)
   int O_max, H_max;    // largest owned-DoF range and halo list of a chunk
   int nch, nch0, ch0, N_own, L_max, PE, SG;  // chunks, owned DoFs, largest chunk table, elements per
@@ -62,7 +63,6 @@ struct StepArgs {
   const float* lcf;    // [Nl][LCF] layer coefficients (see layer_coef_layout)
   const float* lpsi;   // of the layer DoFs: 2D [Nl] Psi2_xx c^2 = -Psi2_zz c^2; 3D [Nl][4] sigma
   const float* lcs;    // [Nl][8 or 12] the update's layer coefficients (chunk_sym.cuh)
-  int comb;            // 3D forward: Pacc holds Psi2 c^2 G u - Psi3 c^2 G omega in one sum
   float* u;
   float* u_out;        // where u^{n+1} goes (symmetry-adapted kernels; u itself elsewhere)
   float* v;

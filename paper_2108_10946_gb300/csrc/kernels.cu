@@ -2,6 +2,7 @@
 // the final M^-1 scaling and mask of Eq. (gradient3), and the misfit reduction.
 #include <algorithm>
 
+#include "halo.cuh"
 #include "update.cuh"
 
 namespace fwi {
@@ -27,17 +28,14 @@ const KernelSet* kernel_set(int dim, int k) {
 }
 
 void launch_node_update(const StepArgs& a, int dim, cudaStream_t st) {
-  const int bs = 256;
-  if (a.S % 4 == 0) {  // one thread per (DoF, four shots)
-    const int64_t items4 = (int64_t)a.hcnt * (a.S / 4);
-    if (items4 == 0) return;
-    const unsigned blocks4 = (unsigned)((items4 + bs - 1) / bs);
-    if (dim == 2)
-      node_kernel4<2><<<blocks4, bs, 0, st>>>(a);
-    else
-      node_kernel4<3><<<blocks4, bs, 0, st>>>(a);
-    return;
+  if (a.sdesc != nullptr) {  // chunked layout
+    switch (a.SG) {
+      case 4: return dim == 2 ? launch_halo_t<2, 4>(a, st) : launch_halo_t<3, 4>(a, st);
+      case 2: return dim == 2 ? launch_halo_t<2, 2>(a, st) : launch_halo_t<3, 2>(a, st);
+      default: return dim == 2 ? launch_halo_t<2, 1>(a, st) : launch_halo_t<3, 1>(a, st);
+    }
   }
+  const int bs = 256;
   const int64_t items = (int64_t)a.hcnt * a.S;
   if (items == 0) return;
   const unsigned blocks = (unsigned)((items + (int64_t)bs * NODE_ITEMS - 1) / ((int64_t)bs * NODE_ITEMS));
