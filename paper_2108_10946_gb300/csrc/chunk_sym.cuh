@@ -432,20 +432,31 @@ __device__ __forceinline__ void sym_inject(const StepArgs& a, int slot, int e, i
   }
 }
 
-// The element phase's walk over the orbits of a triangle: derivatives, node(q, v, r, t) for each
+// One orbit of kind K (first slot qb, coefficients at `at`): derivatives, node(q, v, r, t) for each
 // node, divergence (of the fluxes that node leaves in r, t; not for a field that is only read).
+template <class V, int NN, bool DIV, char K, class F>
+__device__ __forceinline__ void sym_tri_orbit(int qb, int at, const TriCoef<V, NN>& U, TriCoef<V, NN>& Y, F node) {
+  constexpr int SIDES = K == 'X' ? 2 : 1, NV = K == 'C' ? 1 : 3;
+  V r[2][3], t[2][3];
+  tri_grad<V, NN, K>(at, U, r, t);
+#pragma unroll
+  for (int k = 0; k < SIDES; ++k)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) node(qb + TriSym<NN>::place(K, v, k), v, r[k][v], t[k][v]);
+  if constexpr (DIV) tri_div<V, NN, K>(at, r, t, Y);
+}
+// The element phase's walk over the orbits of a triangle. KMV5's like orbits share their code (its
+// seven orbits unrolled are some 3,000 instructions, which miss the instruction caches).
 template <class V, int NN, bool DIV, int O, class F>
 __device__ __forceinline__ void sym_tri_orbits(const TriCoef<V, NN>& U, TriCoef<V, NN>& Y, F node) {
   using T = TriSym<NN>;
-  if constexpr (O < T::NO) {
-    constexpr int SIDES = T::kind(O) == 'X' ? 2 : 1, NV = T::kind(O) == 'C' ? 1 : 3;
-    V r[2][3], t[2][3];
-    tri_grad<V, NN, O>(U, r, t);
-#pragma unroll
-    for (int k = 0; k < SIDES; ++k)
-#pragma unroll
-      for (int v = 0; v < NV; ++v) node(T::node(O, v, k), v, r[k][v], t[k][v]);
-    if constexpr (DIV) tri_div<V, NN, O>(r, t, Y);
+  if constexpr (T::ROLL) {
+#pragma unroll 1
+    for (int k = 0; k < T::NX; ++k) sym_tri_orbit<V, NN, DIV, 'X'>(T::roll_x(k), k * T::XTAB, U, Y, node);
+#pragma unroll 1
+    for (int k = 0; k < T::NT; ++k) sym_tri_orbit<V, NN, DIV, 'T'>(T::roll_t(k), T::NX * T::XTAB + k * T::TTAB, U, Y, node);
+  } else if constexpr (O < T::NO) {
+    sym_tri_orbit<V, NN, DIV, T::kind(O)>(T::base(O), T::tab(O), U, Y, node);
     sym_tri_orbits<V, NN, DIV, O + 1>(U, Y, node);
   }
 }
@@ -563,7 +574,10 @@ __device__ __forceinline__ void sym_tri_body(const StepArgs& a, float* sm) {
   if (LAYER && !GRAD) __syncthreads();  // every P of a shared DoF has been read
   if (act) {
     tri_gather_back<V, NN>(Y, [&](int q, V y) { st(own(L.ys, L.yb, q), y); });
-    if (slot >= 0) sym_inject<NN, MODE, SG>(a, slot, e, s0 + ln, us, at, [&](int q) { return own(L.ys, L.yb, q); });
+    if (slot >= 0)
+      sym_inject<NN, MODE, SG>(
+          a, slot, e, s0 + ln, us, [&](int q) { return at(c_slot[q]); },
+          [&](int q) { return own(L.ys, L.yb, c_slot[q]); });
   }
   constexpr int B = 4;
   SymRound<SG, B> first;

@@ -564,6 +564,11 @@ void fp32_tables(const Element& el, std::vector<float>& dhat32, std::vector<floa
 namespace {
 // Nodal pattern of each input coordinate of a triangle's field (inverse of tri_analyse) and
 // the coordinates of a nodal field (tri_analyse), in the order s1, s2, e1, e2.
+// local node of orbit o at vertex v
+template <int NN>
+int tri_node(int o, int v, int side = 0) {
+  return fwi::sym_slot_node(2, NN, fwi::TriSym<NN>::node(o, v, side));
+}
 template <int NN>
 struct TriCoords {
   using T = fwi::TriSym<NN>;
@@ -573,13 +578,13 @@ struct TriCoords {
     for (int o = 0; o < T::NO; ++o) {
       const int i = T::vec(o);
       if (T::kind(o) == 'C') {
-        c[S1 + o] = u[T::node(o, 0)];
+        c[S1 + o] = u[tri_node<NN>(o, 0)];
         continue;
       }
       ld p[3], m[3];
       for (int v = 0; v < 3; ++v) {
         const bool x = T::kind(o) == 'X';
-        const ld a = u[T::node(o, v, 0)], b = x ? u[T::node(o, v, 1)] : 0;
+        const ld a = u[tri_node<NN>(o, v, 0)], b = x ? u[tri_node<NN>(o, v, 1)] : 0;
         p[v] = a + b;
         m[v] = a - b;
       }
@@ -597,7 +602,7 @@ struct TriCoords {
     for (int o = 0; o < T::NO; ++o) {
       const int i = T::vec(o);
       if (T::kind(o) == 'C') {
-        u[T::node(o, 0)] = c[S1 + o];
+        u[tri_node<NN>(o, 0)] = c[S1 + o];
         continue;
       }
       const ld s = c[S1 + o] / 3, a = c[E1 + i] * 2 / 3, b = c[E2 + i] / 2;
@@ -611,8 +616,8 @@ struct TriCoords {
         m[2] = ms - mb / 2 + ma;
       }
       for (int v = 0; v < 3; ++v) {
-        u[T::node(o, v, 0)] = x ? (p[v] + m[v]) / 2 : p[v];
-        if (x) u[T::node(o, v, 1)] = (p[v] - m[v]) / 2;
+        u[tri_node<NN>(o, v, 0)] = x ? (p[v] + m[v]) / 2 : p[v];
+        if (x) u[tri_node<NN>(o, v, 1)] = (p[v] - m[v]) / 2;
       }
     }
   }
@@ -632,13 +637,13 @@ bool tri_sym_tables(const Element& el, std::vector<float>& tab, std::string& err
   // the layout's node order is the element's
   for (int o = 0; o < T::NO; ++o)
     for (int v = 0; v < 3; ++v) {
-      const double* b0 = &el.bary[(size_t)T::node(o, v, 0) * 3];
-      const double* b1 = &el.bary[(size_t)T::node(o, v, T::kind(o) == 'X') * 3];
+      const double* b0 = &el.bary[(size_t)tri_node<NN>(o, v, 0) * 3];
+      const double* b1 = &el.bary[(size_t)tri_node<NN>(o, v, T::kind(o) == 'X') * 3];
       const int w = (v + 1) % 3, z = (v + 2) % 3;
       bool ok = std::fabs(b0[v] - b1[v]) < 1e-12 && std::fabs(b0[w] - b1[z]) < 1e-12 &&
                 std::fabs(b0[z] - b1[w]) < 1e-12;
       if (v > 0) {  // the orbit's generator, rotated
-        const double* g = &el.bary[(size_t)T::node(o, 0, 0) * 3];
+        const double* g = &el.bary[(size_t)tri_node<NN>(o, 0, 0) * 3];
         ok = ok && std::fabs(b0[v] - g[0]) < 1e-12 && std::fabs(b0[w] - g[1]) < 1e-12;
       }
       if (!ok) {
@@ -666,15 +671,15 @@ bool tri_sym_tables(const Element& el, std::vector<float>& tab, std::string& err
     std::vector<Out> out;
     for (int o = 0; o < T::NO; ++o) {
       if (T::kind(o) == 'C') {
-        Out x{false, true, {0, deriv(u, T::node(o, 0), 0, 0), deriv(u, T::node(o, 0), 0, 1)}};
+        Out x{false, true, {0, deriv(u, tri_node<NN>(o, 0), 0, 0), deriv(u, tri_node<NN>(o, 0), 0, 1)}};
         out.push_back(x);
         continue;
       }
       for (int k = 0; k < 2; ++k) {
         ld a[3], b[3];
         for (int v = 0; v < 3; ++v) {
-          a[v] = deriv(u, T::node(o, v, 0), v, k);
-          b[v] = T::kind(o) == 'X' ? deriv(u, T::node(o, v, 1), v, k) : a[v];
+          a[v] = deriv(u, tri_node<NN>(o, v, 0), v, k);
+          b[v] = T::kind(o) == 'X' ? deriv(u, tri_node<NN>(o, v, 1), v, k) : a[v];
         }
         for (int h = 0; h < (T::kind(o) == 'X' ? 2 : 1); ++h) {
           ld x[3];

@@ -38,6 +38,9 @@ constexpr int NT = SymMap<SG>::NT;
 // 120k: 8.9 and 9.8 ms).
 template <int MODE, bool LAYER>
 constexpr int registers() {
+#ifdef SYM_REGS
+  return SYM_REGS;
+#endif
   if (KMV_DIM == 3 && KMV_K == 3) return LAYER ? 255 : MODE == 2 ? 204 : 168;
   return KMV_K == 5 && MODE == 2 ? 168 : 128;
 }
@@ -101,6 +104,18 @@ int upload(const float* w, const float* sym, int nsym) {
         const int d = i / 32, z = i / 8 % 4;
         tab[o * 96 + i] = sym[tet_at<NN>(o, d, z, z ^ (d + 1), i % 8)];
       }
+#if KMV_DIM == 2
+  if (TriSym<NN>::ROLL) {  // X orbits first, then T orbits
+    using T = TriSym<NN>;
+    int x = 0, t = T::NX * T::XTAB;
+    for (int o = 0; o < T::NO; ++o) {
+      int& to = T::kind(o) == 'X' ? x : t;
+      const int n = T::kind(o) == 'X' ? T::XTAB : T::TTAB;
+      for (int i = 0; i < n; ++i) tab[to + i] = sym[T::tab(o) + i];
+      to += n;
+    }
+  }
+#endif
   for (int i = 0; i < NSYM; ++i) dup[i] = make_float2(tab[i], tab[i]);
   for (int j = 0; j < NN; ++j) {
     const int q = sym_slot_node(D, NN, j);

@@ -7,8 +7,8 @@
 // its orbits, in the library's local node order.
 //
 // Triangles: the full group S3. Orbit kinds:
-//   'V' the three vertices, node v at vertex v
-//   'T' (a, a, b): one node on each median, node base + 2 - v on the median of vertex v
+//   'T' (a, a, b): one node on each median, slot base + 2 - v on the median of vertex v (the
+//       vertices, first, are numbered the other way round in the local order: sym_slot_node)
 //   'X' (g0, g1, g2): two nodes for every vertex v, mirror images in its median
 //   'C' the centroid
 // Tetrahedra: the four-group of the even pair swaps, h = 0..3 = identity, (01)(23), (02)(13),
@@ -35,22 +35,22 @@ struct TriOrbits;
 template <>
 struct TriOrbits<7> {
   static constexpr int NO = 3;
-  FWI_HD static constexpr char kind(int o) { return "VTC"[o]; }
+  FWI_HD static constexpr char kind(int o) { return "TTC"[o]; }
 };
 template <>
 struct TriOrbits<12> {
   static constexpr int NO = 3;
-  FWI_HD static constexpr char kind(int o) { return "VXT"[o]; }
+  FWI_HD static constexpr char kind(int o) { return "TXT"[o]; }
 };
 template <>
 struct TriOrbits<18> {
   static constexpr int NO = 5;
-  FWI_HD static constexpr char kind(int o) { return "VTXTT"[o]; }
+  FWI_HD static constexpr char kind(int o) { return "TTXTT"[o]; }
 };
 template <>
 struct TriOrbits<30> {
   static constexpr int NO = 7;
-  FWI_HD static constexpr char kind(int o) { return "VXXTTTX"[o]; }
+  FWI_HD static constexpr char kind(int o) { return "TXXTTTX"[o]; }
 };
 
 template <int NN>
@@ -67,17 +67,16 @@ struct TriSym : TriOrbits<NN> {
   // three-vector) and NV two-component vectors
   static constexpr int NA1 = NO, NA2 = odd(NO), NV = vec(NO);
   static_assert(base(NO) == NN, "orbits cover the node set");
-  // local node of orbit o at vertex v (side 0 / 1: the two nodes of an X orbit)
-  FWI_HD static constexpr int node(int o, int v, int side = 0) {
-    return base(o) + (B::kind(o) == 'V' ? v
-                      : B::kind(o) == 'T' ? 2 - v
-                      : B::kind(o) == 'C' ? 0
-                                          : side == 0 ? (v == 0 ? 4 : v == 1 ? 3 : 0)
-                                                      : (v == 0 ? 5 : v == 1 ? 1 : 2));
+  // slot of orbit o's node at vertex v (side 0 / 1: the two nodes of an X orbit)
+  FWI_HD static constexpr int place(char k, int v, int side) {  // in its orbit
+    return k == 'T' ? 2 - v
+           : k == 'C' ? 0
+                      : side == 0 ? (v == 0 ? 4 : v == 1 ? 3 : 0) : (v == 0 ? 5 : v == 1 ? 1 : 2);
   }
+  FWI_HD static constexpr int node(int o, int v, int side = 0) { return base(o) + place(B::kind(o), v, side); }
   // Coefficient table, output three-vector by output three-vector. An even output has NA1
   // coefficients for its sum and NV for its vector part, an odd one NA2 and NV; the centroid's
-  // gradient is one vector (NV). A V or T orbit gives the radial (even) and the tangential
+  // gradient is one vector (NV). A T orbit gives the radial (even) and the tangential
   // (odd) derivative; an X orbit radial sums (even) and differences (odd), tangential sums
   // (odd) and differences (even).
   static constexpr int EVEN = NA1 + NV, ODD = NA2 + NV;
@@ -87,6 +86,12 @@ struct TriSym : TriOrbits<NN> {
                                   : B::kind(o - 1) == 'C' ? NV : EVEN + ODD);
   }
   static constexpr int TAB = tab(NO);
+  // Rolled form (KMV5): the table holds the X orbits' coefficients, then the T orbits'; first slots
+  // of the k-th X and T orbit.
+  static constexpr bool ROLL = NN == 30;
+  static constexpr int NX = NA2, NT = NO - NA2, XTAB = 2 * (EVEN + ODD), TTAB = EVEN + ODD;
+  FWI_HD static constexpr int roll_x(int k) { return k == 2 ? 24 : 3 + 6 * k; }
+  FWI_HD static constexpr int roll_t(int k) { return k == 0 ? 0 : 12 + 3 * k; }
 };
 
 // Tetrahedra. Character x: 0 trivial, k = 1..3 (+1 on h = 0 and h = k, -1 on the others); products
@@ -150,10 +155,11 @@ FWI_HD constexpr int tet_at(int o, int d, int z, int y, int i) {
          TetSym<NN>::turn_mode(i, y, d);
 }
 
-// Order of an element's nodes in the chunk tables: the local order, except at KMV3 tetrahedra, whose
-// orbit loop is rolled and takes its nodes orbit by orbit (slot 4 o + h; the interior orbit last).
+// Order of an element's nodes in the chunk tables (local node at slot j): the local order, but a
+// triangle's vertices backwards, like its other T orbits; at KMV3 tetrahedra orbit by orbit (slot
+// 4 o + h; the interior orbit last). So a loop over like orbits need not be unrolled.
 FWI_HD constexpr int sym_slot_node(int dim, int nn, int j) {
-  return dim == 3 && nn == 32 ? TetSym<32>::node(j / 4, j % 4) : j;
+  return dim == 3 ? (nn == 32 ? TetSym<32>::node(j / 4, j % 4) : j) : j < 3 ? 2 - j : j;
 }
 
 }  // namespace fwi

@@ -129,34 +129,34 @@ __device__ __forceinline__ void tri_gather_back(const TriCoef<V, NN>& c, F store
   }
 }
 
-// The NV coefficients at position AT of c_sym times the vector coordinates, and the transpose.
-template <class V, int NN, int AT>
-__device__ __forceinline__ void tri_dot(const TriCoef<V, NN>& c, V& E1, V& E2) {
+// The NV coefficients at position `at` of c_sym times the vector coordinates, and the transpose.
+template <class V, int NN>
+__device__ __forceinline__ void tri_dot(int at, const TriCoef<V, NN>& c, V& E1, V& E2) {
   E1 = E2 = dup<V>(0.f);
 #pragma unroll
   for (int i = 0; i < TriSym<NN>::NV; ++i) {
-    E1 = fma2(coef<V>(AT + i), c.e1[i], E1);
-    E2 = fma2(coef<V>(AT + i), c.e2[i], E2);
+    E1 = fma2(coef<V>(at + i), c.e1[i], E1);
+    E2 = fma2(coef<V>(at + i), c.e2[i], E2);
   }
 }
-template <class V, int NN, int AT>
-__device__ __forceinline__ void tri_axpy(V E1, V E2, TriCoef<V, NN>& c) {
+template <class V, int NN>
+__device__ __forceinline__ void tri_axpy(int at, V E1, V E2, TriCoef<V, NN>& c) {
 #pragma unroll
   for (int i = 0; i < TriSym<NN>::NV; ++i) {
-    c.e1[i] = fma2(coef<V>(AT + i), E1, c.e1[i]);
-    c.e2[i] = fma2(coef<V>(AT + i), E2, c.e2[i]);
+    c.e1[i] = fma2(coef<V>(at + i), E1, c.e1[i]);
+    c.e2[i] = fma2(coef<V>(at + i), E2, c.e2[i]);
   }
 }
 
-// One output three-vector whose coefficients start at position AT.
-template <class V, int NN, int AT, bool ODD>
-__device__ __forceinline__ void tri_out(const TriCoef<V, NN>& c, V (&x)[3]) {
+// One output three-vector whose coefficients start at position `at`.
+template <class V, int NN, bool ODD>
+__device__ __forceinline__ void tri_out(int at, const TriCoef<V, NN>& c, V (&x)[3]) {
   using T = TriSym<NN>;
   constexpr int NA = ODD ? T::NA2 : T::NA1;
   V S = dup<V>(0.f), E1, E2;
 #pragma unroll
-  for (int i = 0; i < NA; ++i) S = fma2(coef<V>(AT + i), ODD ? c.s2[i] : c.s1[i], S);
-  tri_dot<V, NN, AT + NA>(c, E1, E2);
+  for (int i = 0; i < NA; ++i) S = fma2(coef<V>(at + i), ODD ? c.s2[i] : c.s1[i], S);
+  tri_dot<V, NN>(at + NA, c, E1, E2);
   if constexpr (ODD) {
     const V t = NA > 0 ? fma2(dup<V>(-0.5f), E2, S) : mul2(dup<V>(-0.5f), E2);
     x[0] = NA > 0 ? add2(S, E2) : E2;
@@ -171,58 +171,55 @@ __device__ __forceinline__ void tri_out(const TriCoef<V, NN>& c, V (&x)[3]) {
 }
 
 // The transpose: adds the three-vector f to the coordinates.
-template <class V, int NN, int AT, bool ODD>
-__device__ __forceinline__ void tri_in(const V (&f)[3], TriCoef<V, NN>& c) {
+template <class V, int NN, bool ODD>
+__device__ __forceinline__ void tri_in(int at, const V (&f)[3], TriCoef<V, NN>& c) {
   using T = TriSym<NN>;
   constexpr int NA = ODD ? T::NA2 : T::NA1;
   const V h = add2(f[1], f[2]), S = add2(f[0], h), t = fma2(dup<V>(-0.5f), h, f[0]);
   const V E1 = ODD ? sub2(f[2], f[1]) : t, E2 = ODD ? t : mul2(dup<V>(0.75f), sub2(f[1], f[2]));
 #pragma unroll
   for (int i = 0; i < NA; ++i) {
-    if (ODD) c.s2[i] = fma2(coef<V>(AT + i), S, c.s2[i]);
-    else c.s1[i] = fma2(coef<V>(AT + i), S, c.s1[i]);
+    if (ODD) c.s2[i] = fma2(coef<V>(at + i), S, c.s2[i]);
+    else c.s1[i] = fma2(coef<V>(at + i), S, c.s1[i]);
   }
-  tri_axpy<V, NN, AT + NA>(E1, E2, c);
+  tri_axpy<V, NN>(at + NA, E1, E2, c);
 }
 
-// Radial and tangential derivatives at the nodes of orbit O: r[side][v], t[side][v].
-template <class V, int NN, int O>
-__device__ __forceinline__ void tri_grad(const TriCoef<V, NN>& c, V (&r)[2][3], V (&t)[2][3]) {
+// Radial and tangential derivatives r[side][v], t[side][v] at the nodes of an orbit of kind K whose
+// coefficients start at position `at`.
+template <class V, int NN, char K>
+__device__ __forceinline__ void tri_grad(int at, const TriCoef<V, NN>& c, V (&r)[2][3], V (&t)[2][3]) {
   using T = TriSym<NN>;
-  constexpr char K = T::kind(O);
-  constexpr int AT = T::tab(O);
   if constexpr (K == 'C') {
-    tri_dot<V, NN, AT>(c, r[0][0], t[0][0]);
+    tri_dot<V, NN>(at, c, r[0][0], t[0][0]);
   } else if constexpr (K == 'X') {
     V p[3], m[3];
-    tri_out<V, NN, AT, false>(c, p);
-    tri_out<V, NN, AT + T::EVEN, true>(c, m);
+    tri_out<V, NN, false>(at, c, p);
+    tri_out<V, NN, true>(at + T::EVEN, c, m);
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
       r[0][v] = add2(p[v], m[v]);
       r[1][v] = sub2(p[v], m[v]);
     }
-    tri_out<V, NN, AT + T::EVEN + T::ODD, true>(c, p);
-    tri_out<V, NN, AT + T::EVEN + 2 * T::ODD, false>(c, m);
+    tri_out<V, NN, true>(at + T::EVEN + T::ODD, c, p);
+    tri_out<V, NN, false>(at + T::EVEN + 2 * T::ODD, c, m);
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
       t[0][v] = add2(p[v], m[v]);
       t[1][v] = sub2(p[v], m[v]);
     }
   } else {
-    tri_out<V, NN, AT, false>(c, r[0]);
-    tri_out<V, NN, AT + T::EVEN, true>(c, t[0]);
+    tri_out<V, NN, false>(at, c, r[0]);
+    tri_out<V, NN, true>(at + T::EVEN, c, t[0]);
   }
 }
 
 // The transpose of tri_grad: adds the nodes' fluxes to the coordinates of y.
-template <class V, int NN, int O>
-__device__ __forceinline__ void tri_div(const V (&r)[2][3], const V (&t)[2][3], TriCoef<V, NN>& c) {
+template <class V, int NN, char K>
+__device__ __forceinline__ void tri_div(int at, const V (&r)[2][3], const V (&t)[2][3], TriCoef<V, NN>& c) {
   using T = TriSym<NN>;
-  constexpr char K = T::kind(O);
-  constexpr int AT = T::tab(O);
   if constexpr (K == 'C') {
-    tri_axpy<V, NN, AT>(r[0][0], t[0][0], c);
+    tri_axpy<V, NN>(at, r[0][0], t[0][0], c);
   } else if constexpr (K == 'X') {
     V p[3], m[3];
 #pragma unroll
@@ -230,18 +227,18 @@ __device__ __forceinline__ void tri_div(const V (&r)[2][3], const V (&t)[2][3], 
       p[v] = add2(r[0][v], r[1][v]);
       m[v] = sub2(r[0][v], r[1][v]);
     }
-    tri_in<V, NN, AT, false>(p, c);
-    tri_in<V, NN, AT + T::EVEN, true>(m, c);
+    tri_in<V, NN, false>(at, p, c);
+    tri_in<V, NN, true>(at + T::EVEN, m, c);
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
       p[v] = add2(t[0][v], t[1][v]);
       m[v] = sub2(t[0][v], t[1][v]);
     }
-    tri_in<V, NN, AT + T::EVEN + T::ODD, true>(p, c);
-    tri_in<V, NN, AT + T::EVEN + 2 * T::ODD, false>(m, c);
+    tri_in<V, NN, true>(at + T::EVEN + T::ODD, p, c);
+    tri_in<V, NN, false>(at + T::EVEN + 2 * T::ODD, m, c);
   } else {
-    tri_in<V, NN, AT, false>(r[0], c);
-    tri_in<V, NN, AT + T::EVEN, true>(t[0], c);
+    tri_in<V, NN, false>(at, r[0], c);
+    tri_in<V, NN, true>(at + T::EVEN, t[0], c);
   }
 }
 
