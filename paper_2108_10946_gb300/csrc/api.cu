@@ -184,6 +184,7 @@ struct fwi_batch {
   float* d_src_phi = nullptr;
   int* d_rslot_ptr = nullptr;
   int* d_rslot_rec = nullptr;
+  int *d_rslot_elem = nullptr, *d_cslot = nullptr;
   float* d_rslot_phi = nullptr;
   int* d_rec_elem = nullptr;
   float* d_rec_phi = nullptr;
@@ -195,7 +196,8 @@ struct fwi_batch {
   float* ring = nullptr;   // K x [N][S]
   float* gseg = nullptr;                                   // [S][N] FP32 segment sums
   double *gsum = nullptr, *gcomp = nullptr, *misfit = nullptr;  // [S][N], [S][N], [S]
-  int* status = nullptr;
+  int* status = nullptr;       // [0] status bits; [32] meeting counter of the launches of several steps
+  unsigned meet = 0;           // that counter's value once all queued work is done
   cudaStream_t st2 = nullptr;  // second stream of the chunked step (layer chunks)
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   // staging for host pointers
@@ -374,41 +376,46 @@ int locate(const fwi_mesh* m, const double* pts, int npts, std::vector<int>& use
   return 0;
 }
 
-// Injection slots: every element holding a source of the batch or a receiver gets a slot;
-// a slot lists its receivers (id and basis values). sptr is padded to S + R + 1 entries so
-// that sources can be moved later without reallocating.
+// Injection slots: every element holding a source of the batch or a receiver gets a slot, in element
+// order; a slot lists its receivers (id, element and basis values). sptr is padded to S + R + 1
+// entries so that sources can be moved later without reallocating. cslot: the chunks' first slots.
 void build_injection(const fwi_mesh* m, const fwi_batch* b, std::vector<int>& inj,
-                     std::vector<int>& sptr, std::vector<int>& srec, std::vector<float>& sphi) {
+                     std::vector<int>& sptr, std::vector<int>& srec, std::vector<float>& sphi,
+                     std::vector<int>& selem, std::vector<int>& cslot) {
   const int n = m->nn, S = b->S, nrec = b->R;
   inj.assign((size_t)m->Es + 32, -1);  // padded to the element row stride
-  std::vector<int> slot_elems;
-  auto slot_of = [&](int e) {
-    if (inj[e] < 0) {
-      inj[e] = (int)slot_elems.size();
-      slot_elems.push_back(e);
-    }
-    return inj[e];
-  };
-  for (int s = 0; s < S; ++s) slot_of(b->src_elem[s]);
-  for (int r = 0; r < nrec; ++r) slot_of(b->rec_elem[r]);
+  std::vector<int> slot_elems(b->src_elem.begin(), b->src_elem.end());
+  slot_elems.insert(slot_elems.end(), b->rec_elem.begin(), b->rec_elem.end());
+  std::sort(slot_elems.begin(), slot_elems.end());
+  slot_elems.erase(std::unique(slot_elems.begin(), slot_elems.end()), slot_elems.end());
   const int ns = (int)slot_elems.size();
+  for (int t = 0; t < ns; ++t) inj[slot_elems[t]] = t;
   sptr.assign(S + nrec + 1, 0);
   srec.clear();
   sphi.clear();
+  selem.clear();
   std::vector<std::vector<int>> lists(ns);
   for (int r = 0; r < nrec; ++r) lists[inj[b->rec_elem[r]]].push_back(r);
   for (int t = 0; t < ns; ++t) {
     sptr[t + 1] = sptr[t] + (int)lists[t].size();
     for (int r : lists[t]) {
       srec.push_back(r);
+      selem.push_back(slot_elems[t]);
       for (int k = 0; k < n; ++k) sphi.push_back(b->rec_phi[(size_t)r * n + k]);
     }
   }
   for (int t = ns + 1; t < (int)sptr.size(); ++t) sptr[t] = sptr[ns];
   if (srec.empty()) {
     srec.push_back(0);
+    selem.push_back(0);
     sphi.assign(n, 0.f);
   }
+  cslot.assign(m->layout == 0 ? m->nch() + 1 : 1, 0);
+  if (m->layout == 0)
+    for (int c = 0, t = 0; c <= m->nch(); ++c) {
+      while (t < ns && slot_elems[t] < m->ch_e0[c]) ++t;
+      cslot[c] = t;
+    }
 }
 
 // Gershgorin bound of rho(M^-1 K) on the assembled stiffness (Eq. spectral).
@@ -1190,7 +1197,7 @@ int fwi_batch_free(fwi_batch* b) {
   if (b->ev_fork) cudaEventDestroy(b->ev_fork);
   if (b->ev_join) cudaEventDestroy(b->ev_join);
   if (b->st2) cudaStreamDestroy(b->st2);
-  void* ptrs[] = {b->d_inj, b->d_src_elem, b->d_src_phi, b->d_rslot_ptr, b->d_rslot_rec,
+  void* ptrs[] = {b->d_inj, b->d_src_elem, b->d_src_phi, b->d_rslot_ptr, b->d_rslot_rec, b->d_rslot_elem, b->d_cslot,
                   b->d_rslot_phi, b->d_rec_elem, b->d_rec_phi, b->u, b->v, b->r, b->P, b->Pacc,
                   b->PaccY, b->Y, b->Yacc, b->ua, b->va, b->Pa, b->Ya, b->ckpt, b->ring,
                   b->gseg, b->gsum, b->gcomp, b->misfit, b->status, b->wav_dev, b->rec_dev, b->res_dev, b->stage_in, b->stage_out,
@@ -1243,9 +1250,9 @@ int fwi_batch_create(fwi_mesh* m, int nshots, const double* src, int nrec, const
       for (int k = 0; k < n; ++k) b->rec_phi[(size_t)r * n + k] = (float)phi[k];
     }
   }
-  std::vector<int> inj, sptr, srec;
+  std::vector<int> inj, sptr, srec, selem, cslot;
   std::vector<float> sphi;
-  build_injection(m, b.get(), inj, sptr, srec, sphi);
+  build_injection(m, b.get(), inj, sptr, srec, sphi, selem, cslot);
   std::vector<int> src_elem_dev(b->src_elem.begin(), b->src_elem.end());
   std::vector<int> rec_elem_dev(b->rec_elem.begin(), b->rec_elem.end());
   if (rec_elem_dev.empty()) rec_elem_dev.push_back(0);
@@ -1255,7 +1262,8 @@ int fwi_batch_create(fwi_mesh* m, int nshots, const double* src, int nrec, const
   const size_t NS_ = (size_t)N * S, LS = (size_t)m->Nl * d * S, YS = (size_t)m->Nl * S;
   if ((rc = upload(&b->d_inj, inj)) || (rc = upload(&b->d_src_elem, src_elem_dev)) ||
       (rc = upload(&b->d_src_phi, b->src_phi)) || (rc = upload(&b->d_rslot_ptr, sptr)) ||
-      (rc = upload(&b->d_rslot_rec, srec)) || (rc = upload(&b->d_rslot_phi, sphi)) ||
+      (rc = upload(&b->d_rslot_rec, srec)) ||
+      (rc = upload(&b->d_rslot_elem, selem)) || (rc = upload(&b->d_cslot, cslot)) || (rc = upload(&b->d_rslot_phi, sphi)) ||
       (rc = upload(&b->d_rec_elem, rec_elem_dev)) || (rc = upload(&b->d_rec_phi, rec_phi_dev)) ||
       (rc = dalloc(&b->u, NS_)) || (rc = dalloc(&b->v, NS_)) || (rc = dalloc(&b->r, NS_)) ||
       (rc = dalloc(&b->P, LS)) || (rc = dalloc(&b->Pacc, LS)) || (rc = dalloc(&b->PaccY, LS)) ||
@@ -1264,7 +1272,7 @@ int fwi_batch_create(fwi_mesh* m, int nshots, const double* src, int nrec, const
       (rc = dalloc(&b->ckpt, b->state_floats() * b->C)) ||
       (rc = dalloc(&b->ring, NS_ * (b->K / b->gstride))) || (rc = dalloc(&b->gseg, NS_)) ||
       (rc = dalloc(&b->gsum, NS_)) || (rc = dalloc(&b->gcomp, NS_)) ||
-      (rc = dalloc(&b->misfit, (size_t)S)) || (rc = dalloc(&b->status, 1)))
+      (rc = dalloc(&b->misfit, (size_t)S)) || (rc = dalloc(&b->status, 64)))
     return rc;
   if (m->layout == 0) {
     CUDA_TRY(cudaStreamCreateWithFlags(&b->st2, cudaStreamNonBlocking));
@@ -1281,7 +1289,7 @@ int fwi_batch_create(fwi_mesh* m, int nshots, const double* src, int nrec, const
   CUDA_TRY(cudaMemset(b->gsum, 0, NS_ * sizeof(double)));
   CUDA_TRY(cudaMemset(b->gcomp, 0, NS_ * sizeof(double)));
   CUDA_TRY(cudaMemset(b->misfit, 0, (size_t)S * sizeof(double)));
-  CUDA_TRY(cudaMemset(b->status, 0, sizeof(int)));
+  CUDA_TRY(cudaMemset(b->status, 0, 64 * sizeof(int)));
   *out = b.release();
   return 0;
 }
@@ -1352,6 +1360,8 @@ StepArgs base_args(fwi_batch* b) {
   a.rslot_ptr = b->d_rslot_ptr;
   a.rslot_rec = b->d_rslot_rec;
   a.rslot_phi = b->d_rslot_phi;
+  a.rslot_elem = b->d_rslot_elem;
+  a.cslot = b->d_cslot;
   a.R = b->R;
   a.gseg = b->gseg;
   a.grad_lanes = b->grad_lanes;
@@ -1398,6 +1408,30 @@ void run_step(fwi_batch* b, const StepArgs& a, cudaStream_t st) {
   if (e) cudaEventRecord(e[2], st);
   // chunked layout: one launch per non-empty chunk class (without / with layer elements)
   g_launches += 1 + (m->layout == 0 ? (m->nch0 > 0) + (m->nch() > m->nch0) : 1);
+}
+
+// `steps` steps from time index n in direction dir in one launch (symmetry-adapted kernels), if the
+// mesh is small enough for that to be faster; false: nothing was launched. ring, rel0, stride: see
+// RunArgs.
+bool run_many(fwi_batch* b, const StepArgs& a, int steps, int n, int dir, float* ring, int rel0, int stride,
+              cudaStream_t st) {
+  if (b->m->layout != 0 || b->prof || steps < 1 || (a.tc && a.mode != 0) || b->launch_error) return false;
+  fwi::RunArgs r{};
+  r.steps = steps;
+  r.n0 = n;
+  r.dir = dir;
+  r.rel0 = rel0;
+  r.stride = stride;
+  r.ring = ring;
+  r.level = (size_t)b->m->N * b->S;
+  r.count = reinterpret_cast<unsigned*>(b->status + 32);
+  r.base = b->meet;
+  const int grid = b->m->ks->run(a, r, st);
+  if (grid < 0) b->launch_error = -grid;
+  if (grid <= 0) return grid < 0;
+  b->meet += (unsigned)grid * 2u * (unsigned)steps;
+  g_launches += 1;
+  return true;
 }
 
 // Adds the recorded event intervals to the batch's totals (the stream must be complete).
@@ -1463,8 +1497,9 @@ int check_status(fwi_batch* b, cudaStream_t st) {
   CUDA_TRY(cudaGetLastError());
   if (b->prof) collect_profile(b);
   if (h) {
-    cudaMemsetAsync(b->status, 0, sizeof(int), st);
-    if (h & 2) return fail(FWI_ETIMEDOUT, "a bounded wait on the tensor cores gave up (the kernel returned early)");
+    cudaMemsetAsync(b->status, 0, 64 * sizeof(int), st);
+    b->meet = 0;
+    if (h & 2) return fail(FWI_ETIMEDOUT, "a bounded wait inside a kernel gave up (the kernel returned early)");
     return fail(FWI_ERANGE, "non-finite value in the wavefield (time step above the stability limit?)");
   }
   return 0;
@@ -1485,15 +1520,59 @@ void forward_steps(fwi_batch* b, int n0, int n1, const float* wav, float* recs, 
   a.Y = b->Y;
   a.wavelet = wav;
   a.rec = recs;
-  for (int n = n0; n < n1; ++n) {
+  for (int n = n0; n < n1;) {
+    const int stop = ckpts ? std::min(n1, (n / b->K + 1) * b->K) : n1;
     if (ckpts && n % b->K == 0) {
       float *cu, *cv, *cP, *cY;
       ckpt_ptrs(b, n / b->K, &cu, &cv, &cP, &cY);
       copy_state(b, cu, cv, cP, cY, b->u, b->v, b->P, b->Y, st);
     }
+    if (!run_many(b, a, stop - n, n, 1, nullptr, 0, 1, st))
+      for (int k = n; k < stop; ++k) {
+        a.n = k;
+        run_step(b, a, st);
+      }
+    n = stop;
+  }
+}
+
+// Forward field of the levels n0 .. n1-1 of an adjoint segment from its checkpoint: the levels
+// n = 0 (mod r) of the segment end up in the ring. The steps write them there themselves, reading
+// the level before from where it was written (plain layout: in place, then copied).
+int recompute_ring(fwi_batch* b, int c, int n0, int n1, cudaStream_t st) {
+  const size_t NS_ = (size_t)b->m->N * b->S;
+  const int r = b->gstride;
+  float *cu, *cv, *cP, *cY;
+  ckpt_ptrs(b, c, &cu, &cv, &cP, &cY);
+  if (b->m->layout == 1) {
+    if (int rc = copy_state(b, b->u, b->v, b->P, b->Y, cu, cv, cP, cY, st)) return rc;
+    CUDA_TRY(cudaMemcpyAsync(b->ring, b->u, NS_ * sizeof(float), cudaMemcpyDeviceToDevice, st));
+    for (int n = n0; n < n1 - 1; ++n) {
+      forward_steps(b, n, n + 1, b->wav_dev, nullptr, false, st);
+      if ((n + 1) % r == 0)
+        CUDA_TRY(cudaMemcpyAsync(b->ring + NS_ * (size_t)((n + 1 - n0) / r), b->u, NS_ * sizeof(float),
+                                 cudaMemcpyDeviceToDevice, st));
+    }
+    return 0;
+  }
+  if (int rc = copy_state(b, b->ring, b->v, b->P, b->Y, cu, cv, cP, cY, st)) return rc;
+  StepArgs a = base_args(b);
+  a.mode = 0;
+  a.tc = 0;
+  a.u = a.u_out = b->u;
+  a.v = b->v;
+  a.P = b->P;
+  a.Y = b->Y;
+  a.wavelet = b->wav_dev;
+  if (run_many(b, a, n1 - 1 - n0, n0, 1, b->ring, 0, r, st)) return 0;
+  auto level = [&](int rel) { return rel % r == 0 ? b->ring + NS_ * (size_t)(rel / r) : b->u; };
+  for (int n = n0; n < n1 - 1; ++n) {
+    a.u = level(n - n0);
+    a.u_out = level(n + 1 - n0);
     a.n = n;
     run_step(b, a, st);
   }
+  return 0;
 }
 
 }  // namespace
@@ -1539,6 +1618,7 @@ int adjoint_device(fwi_batch* b, const float* res, cudaStream_t st) {
   if (b->acc_lanes >= 0 && b->acc_lanes != b->grad_lanes)
     return fail(FWI_EINVAL, "the gradient accumulators hold sums of the other kind: call "
                             "fwi_gradient* before changing fwi_batch_set_gradient_lanes");
+  const fwi_mesh* mc = b->m;
   b->acc_lanes = b->grad_lanes;
   const size_t rn = (size_t)b->S * (b->nt + 1) * b->R;
   fwi::launch_misfit(res, (int64_t)rn / b->S, b->S, b->misfit, st);
@@ -1557,30 +1637,31 @@ int adjoint_device(fwi_batch* b, const float* res, cudaStream_t st) {
   a.ring_u = nullptr;
   run_step(b, a, st);
   const size_t NS_ = (size_t)b->m->N * b->S;
+  const int r = b->gstride;
   for (int c = b->C - 1; c >= 0; --c) {
     const int n0 = c * b->K, n1 = std::min(n0 + b->K, nt);
-    float *cu, *cv, *cP, *cY;
-    ckpt_ptrs(b, c, &cu, &cv, &cP, &cY);
-    if (int rc = copy_state(b, b->u, b->v, b->P, b->Y, cu, cv, cP, cY, st)) return rc;
-    // the ring keeps U^n for the levels n = 0 (mod r) of the segment (n0 is one of them)
-    const int r = b->gstride;
-    CUDA_TRY(cudaMemcpyAsync(b->ring, b->u, NS_ * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    for (int n = n0; n < n1 - 1; ++n) {
-      forward_steps(b, n, n + 1, b->wav_dev, nullptr, false, st);
-      if ((n + 1) % r == 0)
-        CUDA_TRY(cudaMemcpyAsync(b->ring + NS_ * (size_t)((n + 1 - n0) / r), b->u,
-                                 NS_ * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    }
-    for (int mm = n1 - 1; mm >= std::max(n0, 1); --mm) {
-      a.n = mm;
-      // the gradient integrand at the subsampled levels only (the others: adjoint step alone)
-      a.ring_u = mm % r == 0 ? b->ring + NS_ * (size_t)((mm - n0) / r) : nullptr;
-      run_step(b, a, st);
+    if (int rc = recompute_ring(b, c, n0, n1, st)) return rc;
+    // the gradient integrand at the subsampled levels only (the others: adjoint step alone)
+    const int last = std::max(n0, 1);
+    a.n = n1 - 1;
+    a.ring_u = b->ring;
+    if (r == 1 && run_many(b, a, n1 - last, n1 - 1, -1, b->ring, n1 - 1 - n0, 1, st)) {
+      // one launch did them all
+    } else {
+      for (int mm = n1 - 1; mm >= last; --mm) {
+        a.n = mm;
+        a.ring_u = mm % r == 0 ? b->ring + NS_ * (size_t)((mm - n0) / r) : nullptr;
+        run_step(b, a, st);
+      }
     }
     fwi::launch_fold(b->gseg, b->gsum, b->gcomp, (int64_t)b->m->N * (b->grad_lanes ? b->S : 1),
                      (double)r, st);
     g_launches += 1;
   }
+  // the batch's forward state is the last level of the segment recomputed last, as u, v, P, Y
+  const int end = std::min(b->K, nt) - 1;
+  if (mc->layout == 0 && end % r == 0)
+    CUDA_TRY(cudaMemcpyAsync(b->u, b->ring + NS_ * (size_t)(end / r), NS_ * sizeof(float), cudaMemcpyDeviceToDevice, st));
   return check_status(b, st);
 }
 
@@ -1817,13 +1898,15 @@ int fwi_batch_set_sources(fwi_batch* b, const double* src) {
     m->el.basis(&xh[(size_t)s * d], phi.data());
     for (int k = 0; k < n; ++k) b->src_phi[(size_t)s * n + k] = (float)phi[k];
   }
-  std::vector<int> inj, sptr, srec;
+  std::vector<int> inj, sptr, srec, selem, cslot;
   std::vector<float> sphi;
-  build_injection(m, b, inj, sptr, srec, sphi);
+  build_injection(m, b, inj, sptr, srec, sphi, selem, cslot);
   std::vector<int> se(b->src_elem.begin(), b->src_elem.end());
   CUDA_TRY(cudaMemcpy(b->d_inj, inj.data(), inj.size() * sizeof(int), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMemcpy(b->d_rslot_ptr, sptr.data(), sptr.size() * sizeof(int), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMemcpy(b->d_rslot_rec, srec.data(), srec.size() * sizeof(int), cudaMemcpyHostToDevice));
+  CUDA_TRY(cudaMemcpy(b->d_rslot_elem, selem.data(), selem.size() * sizeof(int), cudaMemcpyHostToDevice));
+  CUDA_TRY(cudaMemcpy(b->d_cslot, cslot.data(), cslot.size() * sizeof(int), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMemcpy(b->d_rslot_phi, sphi.data(), sphi.size() * sizeof(float), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMemcpy(b->d_src_elem, se.data(), se.size() * sizeof(int), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaMemcpy(b->d_src_phi, b->src_phi.data(), b->src_phi.size() * sizeof(float),

@@ -46,15 +46,15 @@ __device__ __forceinline__ void sym_bar_init(uint64_t* bar) {
 __device__ __forceinline__ void sym_bar_expect(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
 }
-// Waits for phase 0 of the barrier; false if it gave up (bounded: 2^22 polls, each of which the
+// Waits for a phase of the barrier; false if it gave up (bounded: 2^22 polls, each of which the
 // hardware may suspend for a while).
-__device__ __forceinline__ bool sym_bar_wait(uint64_t* bar) {
+__device__ __forceinline__ bool sym_bar_wait(uint64_t* bar, uint32_t parity) {
   for (int i = 0; i < (1 << 22); ++i) {
     uint32_t done;
     asm volatile(
-        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\nselp.u32 %0, 1, 0, p;\n}"
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
         : "=r"(done)
-        : "r"(smem_addr(bar))
+        : "r"(smem_addr(bar)), "r"(parity)
         : "memory");
     if (done) return true;
   }
@@ -95,6 +95,16 @@ template <int SG>
 struct SymMap {
   static constexpr int LANES = SYM_LANES < SG ? SYM_LANES : SG, PER = SG / LANES, NT = SYM_PE * PER;
   typedef typename std::conditional<LANES == 2, float2, float>::type V;
+};
+
+// What changes from step to step: fields in and out, the forward field (gradient steps), the time
+// index, and the parity of the copies' barrier.
+struct SymStep {
+  const float* u;
+  float* u_out;
+  const float* ring_u;
+  int n;
+  uint32_t parity;
 };
 
 // Dynamic shared memory of one chunk (offsets in floats). T: largest chunk table, SH: most shared
@@ -158,9 +168,16 @@ __device__ __forceinline__ SymDesc sym_desc(const StepArgs& a, int c) {
 
 // Phase 1 of one chunk. The table: owned shared DoFs [0, nsh), bubbles, halo DoFs. The runs' shifts
 // follow from their addresses (sym_shift).
-template <int D, int NN, int NS, int SG, int MODE, bool LAYER>
-__device__ __forceinline__ void sym_load(const StepArgs& a, const SymDesc& cd, const SymSmem& L, float* sm, uint64_t* bar,
-                                         int s0, int tid) {
+// RUN (several steps in one launch): what other CTAs wrote in an earlier step comes from L2 (copies
+// of four and eight bytes would go through L1).
+template <int BYTES, bool RUN>
+__device__ __forceinline__ void sym_cp_live(float* dst, const float* src) {
+  if constexpr (RUN && BYTES < 16) lanes_st<BYTES / 4>(dst, lanes_ldcg<BYTES / 4>(src));
+  else sym_cp<BYTES>(dst, src);
+}
+template <int D, int NN, int NS, int SG, int MODE, bool LAYER, bool RUN>
+__device__ __forceinline__ void sym_load(const StepArgs& a, const SymStep& x, const SymDesc& cd, const SymSmem& L,
+                                         float* sm, uint64_t* bar, int s0, int tid) {
   constexpr int NI = NN - NS, NT = SymMap<SG>::NT;
   constexpr bool GRAD = MODE == 2, OM = LAYER && D == 3 && MODE == 0;
   constexpr int PSI = LAYER ? sym_psi<D, MODE>() : 0;
@@ -173,8 +190,8 @@ __device__ __forceinline__ void sym_load(const StepArgs& a, const SymDesc& cd, c
                  me = sym_run(reinterpret_cast<const float*>(a.smeta) + cd.meta, cd.meta_n);
     SymRun u{}, f{}, ps{}, om{}, p1{}, p2{};
     if (S == SG) {
-      u = sym_run(a.u + i0, on * SG);
-      if (GRAD) f = sym_run(a.ring_u + i0, on * SG);
+      u = sym_run(x.u + i0, on * SG);
+      if (GRAD) f = sym_run(x.ring_u + i0, on * SG);
     }
     if (LAYER) {
       if (S == SG) {
@@ -210,21 +227,21 @@ __device__ __forceinline__ void sym_load(const StepArgs& a, const SymDesc& cd, c
     if (LAYER && D == 3 && S == SG) sym_prefetch(a.Y + pi0 * SG, on * SG);
     // and the ranges of the chunk a wave of CTAs further on
     const int nc = blockIdx.x + a.ch0 + a.wave;
-    if (nc < a.ch1) {
+    if (!RUN && nc < a.ch1) {
       const SymDesc nx = sym_desc(a, nc);
       const int nn = nx.nsh + nx.ne * NI;
       sym_prefetch(reinterpret_cast<const float*>(a.smeta) + nx.meta, nx.meta_n);
       sym_prefetch(reinterpret_cast<const float*>(a.halo) + nx.hp, nx.hn);
       sym_prefetch(a.c2 + nx.own, nn);
       if (S == SG) {
-        sym_prefetch(a.u + (size_t)nx.own * S, nn * SG);
-        if (GRAD) sym_prefetch(a.ring_u + (size_t)nx.own * S, nn * SG);
+        sym_prefetch(x.u + (size_t)nx.own * S, nn * SG);
+        if (GRAD) sym_prefetch(x.ring_u + (size_t)nx.own * S, nn * SG);
         if (LAYER) sym_prefetch(a.P + (size_t)(nx.own - a.p_own) * D * SG, nn * D * SG);
       }
     }
   }
-  float* us = sm + L.u + sym_shift(a.u + i0);
-  float* fs = sm + L.f + (GRAD ? sym_shift(a.ring_u + i0) : 0);
+  float* us = sm + L.u + sym_shift(x.u + i0);
+  float* fs = sm + L.f + (GRAD ? sym_shift(x.ring_u + i0) : 0);
   float* cs = sm + L.c2 + sym_shift(a.c2 + cd.own);
   float *ps = sm + L.ps, *om = sm + L.om, *p1 = sm + L.p1, *p2 = sm + L.sb;
   if (LAYER) {
@@ -236,8 +253,8 @@ __device__ __forceinline__ void sym_load(const StepArgs& a, const SymDesc& cd, c
   if (S != SG) {  // the group's shots are a part of each DoF's run
     for (int l = tid; l < on; l += NT) {
       const size_t dof = (size_t)(cd.own + l);
-      sym_cp<4 * SG>(us + l * SG, a.u + dof * S + s0);
-      if (GRAD) sym_cp<4 * SG>(fs + l * SG, a.ring_u + dof * S + s0);
+      sym_cp<4 * SG>(us + l * SG, x.u + dof * S + s0);
+      if (GRAD) sym_cp<4 * SG>(fs + l * SG, x.ring_u + dof * S + s0);
       if (LAYER)
 #pragma unroll
         for (int k = 0; k < D; ++k)
@@ -250,15 +267,15 @@ __device__ __forceinline__ void sym_load(const StepArgs& a, const SymDesc& cd, c
   for (int h = tid; h < cd.hn; h += NT) {
     const int id = __ldg(a.halo + cd.hp + h), l = on + h;
     reinterpret_cast<int*>(sm + L.ids)[h] = id;
-    sym_cp<4 * SG>(us + l * SG, a.u + (size_t)id * S + s0);
-    if (GRAD) sym_cp<4 * SG>(fs + l * SG, a.ring_u + (size_t)id * S + s0);
+    sym_cp_live<4 * SG, RUN>(us + l * SG, x.u + (size_t)id * S + s0);
+    if (GRAD) sym_cp<4 * SG>(fs + l * SG, x.ring_u + (size_t)id * S + s0);
     sym_cp<4>(cs + l, a.c2 + id);
     if (LAYER) {
       const size_t pi = (size_t)(id - a.p_halo);
 #pragma unroll
-      for (int k = 0; k < D; ++k) sym_cp<4 * SG>(p1 + ((cd.nsh + h) * D + k) * SG, a.P + (pi * D + k) * S + s0);
+      for (int k = 0; k < D; ++k) sym_cp_live<4 * SG, RUN>(p1 + ((cd.nsh + h) * D + k) * SG, a.P + (pi * D + k) * S + s0);
       if (PSI) sym_cp<4 * (PSI ? PSI : 1)>(ps + l * PSI, a.lpsi + pi * PSI);
-      if (OM) sym_cp<4 * SG>(om + l * SG, a.Y + pi * S + s0);
+      if (OM) sym_cp_live<4 * SG, RUN>(om + l * SG, a.Y + pi * S + s0);
     }
   }
 }
@@ -295,15 +312,15 @@ struct SymRound {
 // v' = c1 v - c2 y - c3 u, u' = u + v'. chk collects 0 * u', which stays zero while every value is
 // finite.
 template <int D, int NN, int NS, int MODE, bool LAYER, int SG, int B>
-__device__ __forceinline__ void sym_finish(const StepArgs& a, const SymDesc& cd, const SymSmem& L, const float* sm,
-                                           int s0, int tid, SymRound<SG, B>& cur, float& chk) {
+__device__ __forceinline__ void sym_finish(const StepArgs& a, const SymStep& x, const SymDesc& cd, const SymSmem& L,
+                                           const float* sm, int s0, int tid, SymRound<SG, B>& cur, float& chk) {
   constexpr int PE = SYM_PE, NI = NN - NS, NT = SymMap<SG>::NT;
   constexpr bool GRAD = MODE == 2;
   const int S = a.S, nb = cd.ne * NI, on = cd.nsh + nb;
   const uint16_t* ge = reinterpret_cast<const uint16_t*>(sm + L.meta) + NS * PE;
   const uint16_t* gp = ge + NS * PE;
   const int* ids = reinterpret_cast<const int*>(sm + L.ids);
-  const float* us = sm + L.u + sym_shift(a.u + (size_t)cd.own * S + s0);
+  const float* us = sm + L.u + sym_shift(x.u + (size_t)cd.own * S + s0);
   for (int l0 = tid; l0 < on; l0 += B * NT) {
     SymRound<SG, B> nxt;
     nxt.load(a, cd, on, s0, l0 + B * NT, NT);
@@ -334,7 +351,7 @@ __device__ __forceinline__ void sym_finish(const StepArgs& a, const SymDesc& cd,
         for (int j = 0; j < SG; ++j) chk = fmaf(0.f, un.x[j], chk);
         const size_t gi = (size_t)(cd.own + l) * S + s0;
         lanes_st<SG>(a.v + gi, vn);
-        lanes_st<SG>(a.u_out + gi, un);
+        lanes_st<SG>(x.u_out + gi, un);
       }
     }
     cur = nxt;
@@ -405,29 +422,50 @@ __device__ __forceinline__ void sym_finish(const StepArgs& a, const SymDesc& cd,
   }
 }
 
-// Sources and receivers of an element (few have any), for the lanes of a thread: shots s, s + 1, ...;
-// u: their nodal values, y(q): their sums at node q.
-template <int NN, int MODE, int SG, class A, class F>
-__device__ __forceinline__ void sym_inject(const StepArgs& a, int slot, int e, int s1, const float* u, A at, F y) {
-  const int rb = __ldg(a.rslot_ptr + slot), re = __ldg(a.rslot_ptr + slot + 1);
-#pragma unroll 1
-  for (int k = 0; k < SymMap<SG>::LANES; ++k) {
-    const int s = s1 + k;
-    for (int r = rb; r < re; ++r) {
-      const float* phi = a.rslot_phi + (size_t)r * NN;
-      const size_t at_rec = ((size_t)s * (a.nt + 1) + a.n) * a.R + __ldg(a.rslot_rec + r);
-      if constexpr (MODE != 0) {
-        const float res = __ldg(a.resid + at_rec);
-        for (int q = 0; q < NN; ++q) y(q)[k] += res * __ldg(phi + q);
-      } else if (a.rec != nullptr) {
+// Sources and receivers of a chunk (between the element phase and the update, each after a barrier;
+// few chunks have any). Their elements' nodal values are still in the table, their sums in the
+// threads' places. All threads share the work: one takes a receiver's record of one shot, or a
+// node's sum over an element's receivers. (Done by the element's own thread, receiver by receiver,
+// this was the longest chain of a step wherever receivers crowd: 4 us with three in an element.)
+template <int D, int NN, int NS, int MODE, int SG>
+__device__ __forceinline__ void sym_inject(const StepArgs& a, const SymStep& x, const SymDesc& cd, const SymSmem& L,
+                                           float* sm, int s0, int tid, int b, int e) {
+  constexpr int PE = SYM_PE, NI = NN - NS, NT = SymMap<SG>::NT;
+  const uint16_t* lq = reinterpret_cast<const uint16_t*>(sm + L.meta);
+  const float* us = sm + L.u + sym_shift(x.u + (size_t)cd.own * a.S + s0);
+  auto place = [&](int q, int el) {
+    return sm + (q < NS ? L.ys + (c_slot[q] * PE + el) * SG : L.yb + (el * NI + q - NS) * SG);
+  };
+  if constexpr (MODE == 0) {
+    if (a.rec != nullptr) {
+      const int r0 = __ldg(a.rslot_ptr + b), n = (__ldg(a.rslot_ptr + e) - r0) * SG;
+      for (int t = tid; t < n; t += NT) {
+        const int r = r0 + t / SG, k = t % SG, el = __ldg(a.rslot_elem + r) - cd.e0;
         float acc = 0.f;
-        for (int q = 0; q < NN; ++q) acc = fmaf(__ldg(phi + q), u[at(q) * SG + k], acc);
-        a.rec[at_rec] = acc;
+#pragma unroll 8
+        for (int q = 0; q < NN; ++q) {
+          const int l = q < NS ? (int)lq[c_slot[q] * PE + el] : cd.nsh + el * NI + q - NS;
+          acc = fmaf(__ldg(a.rslot_phi + (size_t)r * NN + q), us[l * SG + k], acc);
+        }
+        a.rec[((size_t)(s0 + k) * (a.nt + 1) + x.n) * a.R + __ldg(a.rslot_rec + r)] = acc;
       }
     }
-    if (MODE == 0 && __ldg(a.src_elem + s) == e) {
-      const float wv = __ldg(a.wavelet + (size_t)s * a.nt + a.n);
-      for (int q = 0; q < NN; ++q) y(q)[k] -= wv * __ldg(a.src_phi + (size_t)s * NN + q);
+    for (int k = 0; k < SG; ++k) {
+      const int el = __ldg(a.src_elem + s0 + k) - cd.e0;
+      if (el < 0 || el >= cd.ne) continue;
+      const float wv = __ldg(a.wavelet + (size_t)(s0 + k) * a.nt + x.n);
+      for (int q = tid; q < NN; q += NT) place(q, el)[k] -= wv * __ldg(a.src_phi + (size_t)(s0 + k) * NN + q);
+    }
+  } else {
+    for (int t = tid; t < (e - b) * NN * SG; t += NT) {
+      const int k = t % SG, q = t / SG % NN, slot = b + t / (SG * NN);
+      const int rb = __ldg(a.rslot_ptr + slot), re = __ldg(a.rslot_ptr + slot + 1);
+      if (rb == re) continue;
+      const float* res = a.resid + ((size_t)(s0 + k) * (a.nt + 1) + x.n) * a.R;
+      float acc = 0.f;
+#pragma unroll 4
+      for (int r = rb; r < re; ++r) acc = fmaf(__ldg(res + __ldg(a.rslot_rec + r)), __ldg(a.rslot_phi + (size_t)r * NN + q), acc);
+      place(q, __ldg(a.rslot_elem + rb) - cd.e0)[k] += acc;
     }
   }
 }
@@ -456,29 +494,31 @@ __device__ __forceinline__ void sym_tri_orbits(const TriCoef<V, NN>& U, TriCoef<
 #pragma unroll 1
     for (int k = 0; k < T::NT; ++k) sym_tri_orbit<V, NN, DIV, 'T'>(T::roll_t(k), T::NX * T::XTAB + k * T::TTAB, U, Y, node);
   } else if constexpr (O < T::NO) {
-    sym_tri_orbit<V, NN, DIV, T::kind(O)>(T::base(O), T::tab(O), U, Y, node);
+    constexpr int QB = T::base(O), AT = T::tab(O);
+    sym_tri_orbit<V, NN, DIV, T::kind(O)>(QB, AT, U, Y, node);
     sym_tri_orbits<V, NN, DIV, O + 1>(U, Y, node);
   }
 }
 
 // One step of a triangle chunk. MODE: 0 forward, 1 adjoint, 2 adjoint with the gradient integrand.
-template <int NN, int NS, int MODE, bool LAYER, int SG>
-__device__ __forceinline__ void sym_tri_body(const StepArgs& a, float* sm) {
+template <int NN, int NS, int MODE, bool LAYER, int SG, bool RUN>
+__device__ __forceinline__ bool sym_tri_body(const StepArgs& a, const SymStep& x, float* sm, int chunk, int s0) {
   using M = SymMap<SG>;
   using V = typename M::V;
   constexpr int NI = NN - NS, PE = SYM_PE;
   constexpr bool ADJ = MODE != 0, GRAD = MODE == 2;
-  const int tid = threadIdx.x, S = a.S, s0 = blockIdx.y * SG;
+  const int tid = threadIdx.x, S = a.S;
   const SymSmem L = sym_smem<2, NN, NS, SG, MODE, LAYER>(a.T_max, a.SH_max, a.H_max);
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm);
-  if (tid == 0) sym_bar_init(bar);  // (the thread that issues the barrier's copies)
-  const SymDesc cd = sym_desc(a, blockIdx.x + a.ch0);
-  sym_load<2, NN, NS, SG, MODE, LAYER>(a, cd, L, sm, bar, s0, tid);
-  __syncthreads();  // the barrier is set up before anyone asks it
+  if (!RUN && tid == 0) sym_bar_init(bar);  // (the thread that issues the barrier's copies)
+  const SymDesc cd = sym_desc(a, chunk);
+  sym_load<2, NN, NS, SG, MODE, LAYER, RUN>(a, x, cd, L, sm, bar, s0, tid);
+  if (!RUN) __syncthreads();  // the barrier is set up before anyone asks it
   const int el = tid / M::PER, ln = tid % M::PER * M::LANES;  // element, first shot of the group
   const bool act = el < cd.ne;
   const int ee = act ? el : 0, e = cd.e0 + ee, nb = cd.ne * NI;
-  const int slot = act ? __ldg(a.inj + e) : -1, bub = cd.nsh + ee * NI;
+  const int bub = cd.nsh + ee * NI;
+  const int in0 = __ldg(a.cslot + chunk), in1 = __ldg(a.cslot + chunk + 1);  // sources' and receivers' elements
   const size_t i0 = (size_t)cd.own * S + s0, pi0 = (size_t)(cd.own - a.p_own);
   const uint16_t* lq = reinterpret_cast<const uint16_t*>(sm + L.meta) + ee;
   float H0[3], A0[2][2];
@@ -488,15 +528,15 @@ __device__ __forceinline__ void sym_tri_body(const StepArgs& a, float* sm) {
 #pragma unroll
     for (int c = 0; c < 4; ++c) A0[c >> 1][c & 1] = __ldg(a.lgeo + (size_t)c * (a.E - a.E0) + (e - a.E0));
   sym_cp_wait();
-  const bool ok = sym_bar_wait(bar);
+  const bool ok = sym_bar_wait(bar, x.parity);
   if (__syncthreads_or(!ok)) {  // a copy did not arrive: report it and leave the fields alone
-    sym_bar_wait(bar);
+    sym_bar_wait(bar, x.parity);
     if (tid == 0) atomicOr(a.status, 2);
-    return;
+    return false;
   }
 
   // ---- elements --------------------------------------------------------------------------
-  const float* us = sm + L.u + sym_shift(a.u + i0) + ln;
+  const float* us = sm + L.u + sym_shift(x.u + i0) + ln;
   const float* cs = sm + L.c2 + sym_shift(a.c2 + cd.own);
   // a thread's own places for node q: the sums' ([node][element][shot], bubbles in DoF order), ...
   const int ps = el * SG + ln, pb = el * NI * SG + ln;
@@ -508,7 +548,7 @@ __device__ __forceinline__ void sym_tri_body(const StepArgs& a, float* sm) {
   if (act) {
     TriCoef<V, NN> U;
     if constexpr (GRAD) {  // the forward field's derivatives wait in places that are filled later
-      const float* fs = sm + L.f + sym_shift(a.ring_u + i0) + ln;
+      const float* fs = sm + L.f + sym_shift(x.ring_u + i0) + ln;
       tri_analyse<V, NN>(U, [&](int q) { return ld(fs + at(q) * SG); });
       sym_tri_orbits<V, NN, false, 0>(U, Y, [&](int q, int, V& r, V& t) {
         st(own(L.gs, L.gb, q), r);
@@ -574,19 +614,20 @@ __device__ __forceinline__ void sym_tri_body(const StepArgs& a, float* sm) {
   if (LAYER && !GRAD) __syncthreads();  // every P of a shared DoF has been read
   if (act) {
     tri_gather_back<V, NN>(Y, [&](int q, V y) { st(own(L.ys, L.yb, q), y); });
-    if (slot >= 0)
-      sym_inject<NN, MODE, SG>(
-          a, slot, e, s0 + ln, us, [&](int q) { return at(c_slot[q]); },
-          [&](int q) { return own(L.ys, L.yb, c_slot[q]); });
   }
   constexpr int B = 4;
   SymRound<SG, B> first;
   first.load(a, cd, cd.nsh + nb, s0, tid, M::NT);
   __syncthreads();
+  if (in0 < in1) {
+    sym_inject<2, NN, NS, MODE, SG>(a, x, cd, L, sm, s0, tid, in0, in1);
+    __syncthreads();
+  }
 
   float chk = 0.f;
-  sym_finish<2, NN, NS, MODE, LAYER, SG, B>(a, cd, L, sm, s0, tid, first, chk);
+  sym_finish<2, NN, NS, MODE, LAYER, SG, B>(a, x, cd, L, sm, s0, tid, first, chk);
   if (!(chk == 0.f)) atomicOr(a.status, 1);
+  return true;
 }
 
 // The walk over the orbits of a tetrahedron: derivatives of N fields, node(q, g) for each node with
@@ -684,24 +725,25 @@ __device__ __forceinline__ void sym_tet_roll(const TetCoef<V, 32>* const (&U)[N]
 
 // One step of a tetrahedra chunk. Fields: u; the forward field (gradient steps); omega (forward
 // steps in the layer).
-template <int NN, int NS, int MODE, bool LAYER, int SG>
-__device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
+template <int NN, int NS, int MODE, bool LAYER, int SG, bool RUN>
+__device__ __forceinline__ bool sym_tet_body(const StepArgs& a, const SymStep& x, float* sm, int chunk, int s0) {
   using M = SymMap<SG>;
   using V = typename M::V;
   constexpr int NI = NN - NS, PE = SYM_PE;
   constexpr bool ADJ = MODE != 0, GRAD = MODE == 2, OM = LAYER && !ADJ, W = LAYER && ADJ;
   constexpr int NF = 1 + (GRAD || OM);
-  const int tid = threadIdx.x, S = a.S, s0 = blockIdx.y * SG;
+  const int tid = threadIdx.x, S = a.S;
   const SymSmem L = sym_smem<3, NN, NS, SG, MODE, LAYER>(a.T_max, a.SH_max, a.H_max);
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm);
-  if (tid == 0) sym_bar_init(bar);  // (the thread that issues the barrier's copies)
-  const SymDesc cd = sym_desc(a, blockIdx.x + a.ch0);
-  sym_load<3, NN, NS, SG, MODE, LAYER>(a, cd, L, sm, bar, s0, tid);
-  __syncthreads();  // the barrier is set up before anyone asks it
+  if (!RUN && tid == 0) sym_bar_init(bar);  // (the thread that issues the barrier's copies)
+  const SymDesc cd = sym_desc(a, chunk);
+  sym_load<3, NN, NS, SG, MODE, LAYER, RUN>(a, x, cd, L, sm, bar, s0, tid);
+  if (!RUN) __syncthreads();  // the barrier is set up before anyone asks it
   const int el = tid / M::PER, ln = tid % M::PER * M::LANES;  // element, first shot of the group
   const bool act = el < cd.ne;
   const int ee = act ? el : 0, e = cd.e0 + ee, nb = cd.ne * NI;
-  const int slot = act ? __ldg(a.inj + e) : -1, bub = cd.nsh + ee * NI;
+  const int bub = cd.nsh + ee * NI;
+  const int in0 = __ldg(a.cslot + chunk), in1 = __ldg(a.cslot + chunk + 1);  // sources' and receivers' elements
   const size_t i0 = (size_t)cd.own * S + s0, pi0 = (size_t)(cd.own - a.p_own);
   const uint16_t* lq = reinterpret_cast<const uint16_t*>(sm + L.meta) + ee;
   float G[6], A[3][3];  // |J| J^-1 J^-T and |J| J^-1 in the cube's axes
@@ -711,15 +753,15 @@ __device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
 #pragma unroll
     for (int c = 0; c < 9; ++c) A[c / 3][c % 3] = __ldg(a.lgeo + (size_t)c * (a.E - a.E0) + (e - a.E0));
   sym_cp_wait();
-  const bool ok = sym_bar_wait(bar);
+  const bool ok = sym_bar_wait(bar, x.parity);
   if (__syncthreads_or(!ok)) {  // a copy did not arrive: report it and leave the fields alone
-    sym_bar_wait(bar);
+    sym_bar_wait(bar, x.parity);
     if (tid == 0) atomicOr(a.status, 2);
-    return;
+    return false;
   }
 
   // ---- elements --------------------------------------------------------------------------
-  const float* us = sm + L.u + sym_shift(a.u + i0) + ln;
+  const float* us = sm + L.u + sym_shift(x.u + i0) + ln;
   const float* cs = sm + L.c2 + sym_shift(a.c2 + cd.own);
   const int ps = el * SG + ln, pb = el * NI * SG + ln;  // a thread's own places (see sym_tri_body)
   // q: a node's slot (sym_slot_node: the local node, at KMV3 orbit by orbit)
@@ -739,7 +781,7 @@ __device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
   TetCoef<V, NN> U, F, Y, Y2;
   if (act) {
     if constexpr (GRAD) {
-      const float* fs = sm + L.f + sym_shift(a.ring_u + i0) + ln;
+      const float* fs = sm + L.f + sym_shift(x.ring_u + i0) + ln;
       tet_analyse<V, NN>(F, [&](int q) { return ld(fs + at(slot_of(q)) * SG); });
     }
     if constexpr (OM) {
@@ -758,16 +800,16 @@ __device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
     if constexpr (W) tet_zero(Y2);
     // one node: x[0] in are the field's derivatives, out the flux (x[1]: the other field's; out, in
     // the layer's adjoint, the omega row's flux)
-    auto node = [&](int q, auto& x) {
+    auto node = [&](int q, auto& g) {
       const float w = c_w[q];
       const int l = at(q);
       const float c2 = cs[l];
-      const V wc = dup<V>(w * c2), g0 = x[0][0], g1 = x[0][1], g2 = x[0][2];
+      const V wc = dup<V>(w * c2), g0 = g[0][0], g1 = g[0][1], g2 = g[0][2];
       const V h0 = fma2(dup<V>(G[0]), g0, fma2(dup<V>(G[1]), g1, mul2(dup<V>(G[2]), g2)));
       const V h1 = fma2(dup<V>(G[1]), g0, fma2(dup<V>(G[3]), g1, mul2(dup<V>(G[4]), g2)));
       const V h2 = fma2(dup<V>(G[2]), g0, fma2(dup<V>(G[4]), g1, mul2(dup<V>(G[5]), g2)));
       if constexpr (GRAD)  // w (Ghat grad u_dag) . grad u
-        st(own(L.gs, L.gb, q), mul2(dup<V>(w), fma2(h0, x[1][0], fma2(h1, x[1][1], mul2(h2, x[1][2])))));
+        st(own(L.gs, L.gb, q), mul2(dup<V>(w), fma2(h0, g[1][0], fma2(h1, g[1][1], mul2(h2, g[1][2])))));
       V f[3] = {mul2(wc, h0), mul2(wc, h1), mul2(wc, h2)};
       if constexpr (LAYER) {
         const int on = cd.nsh + nb;
@@ -782,7 +824,7 @@ __device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
           P[k] = ld(p + k * SG);
           s[k] = fma2(dup<V>(A[0][k]), g0, fma2(dup<V>(A[1][k]), g1, mul2(dup<V>(A[2][k]), g2)));
           if constexpr (OM) {  // both gradients, each with its Psi c^2
-            const V y = fma2(dup<V>(A[0][k]), x[1][0], fma2(dup<V>(A[1][k]), x[1][1], mul2(dup<V>(A[2][k]), x[1][2])));
+            const V y = fma2(dup<V>(A[0][k]), g[1][0], fma2(dup<V>(A[1][k]), g[1][1], mul2(dup<V>(A[2][k]), g[1][2])));
             s[k] = fma2(dup<V>(-psi3[k]), y, mul2(dup<V>(psi2[k]), s[k]));
           }
           s[k] = mul2(dup<V>(w), s[k]);
@@ -794,12 +836,12 @@ __device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
         for (int d = 0; d < 3; ++d) {
           f[d] = fma2(dup<V>(A[d][0]), Q[0], fma2(dup<V>(A[d][1]), Q[1], fma2(dup<V>(A[d][2]), Q[2], f[d])));
           if constexpr (W)
-            x[1][d] = fma2(dup<V>(w * psi3[0] * A[d][0]), P[0],
+            g[1][d] = fma2(dup<V>(w * psi3[0] * A[d][0]), P[0],
                            fma2(dup<V>(w * psi3[1] * A[d][1]), P[1], mul2(dup<V>(w * psi3[2] * A[d][2]), P[2])));
         }
       }
 #pragma unroll
-      for (int d = 0; d < 3; ++d) x[0][d] = f[d];
+      for (int d = 0; d < 3; ++d) g[0][d] = f[d];
     };
     if constexpr (NF == 2) {
       const TetCoef<V, NN>* const fields[2] = {&U, &F};
@@ -815,19 +857,20 @@ __device__ __forceinline__ void sym_tet_body(const StepArgs& a, float* sm) {
   if (act) {
     tet_gather_back<V, NN>(Y, [&](int q, V y) { st(own(L.ys, L.yb, slot_of(q)), y); });
     if constexpr (W) tet_gather_back<V, NN>(Y2, [&](int q, V y) { st(own(L.ws, L.wb, slot_of(q)), y); });
-    if (slot >= 0)
-      sym_inject<NN, MODE, SG>(
-          a, slot, e, s0 + ln, us, [&](int q) { return at(c_slot[q]); },
-          [&](int q) { return own(L.ys, L.yb, c_slot[q]); });
   }
   constexpr int B = 2;
   SymRound<SG, B> first;
   first.load(a, cd, cd.nsh + nb, s0, tid, M::NT);
   __syncthreads();
+  if (in0 < in1) {
+    sym_inject<3, NN, NS, MODE, SG>(a, x, cd, L, sm, s0, tid, in0, in1);
+    __syncthreads();
+  }
 
   float chk = 0.f;
-  sym_finish<3, NN, NS, MODE, LAYER, SG, B>(a, cd, L, sm, s0, tid, first, chk);
+  sym_finish<3, NN, NS, MODE, LAYER, SG, B>(a, x, cd, L, sm, s0, tid, first, chk);
   if (!(chk == 0.f)) atomicOr(a.status, 1);
+  return true;
 }
 
 }  // namespace fwi

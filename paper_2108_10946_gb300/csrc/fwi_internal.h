@@ -77,7 +77,9 @@ struct StepArgs {
   const int* src_elem;     // [S]
   const float* src_phi;    // [S][NN]
   const float* wavelet;    // [S][nt]
-  const int* rslot_ptr;    // [nslot+1]
+  const int* rslot_ptr;    // [nslot+1], slots in element order
+  const int* cslot;        // [nch+1] first slot of every chunk (chunked layout)
+  const int* rslot_elem;   // element of every receiver, in slot order
   const int* rslot_rec;    // receiver ids
   const float* rslot_phi;  // [entries][NN]
   int R;
@@ -100,10 +102,22 @@ struct StepArgs {
 //            6D+2: dt detPsi1; 6D+3: dt / M
 inline int layer_coef_count(int dim) { return dim == 2 ? 4 * 2 : 6 * 3 + 4; }
 
+// Several steps in one launch (sym_inst.cu): time indices n0, n0 + dir, ...; the ring of forward
+// fields (level floats apart, every stride-th level of the segment from its first on; rel0 the
+// first step's level in it; adjoint: stride 1); the CTAs' meeting counter and its value so far.
+struct RunArgs {
+  int steps, n0, dir, rel0, stride;
+  float* ring;
+  size_t level;
+  unsigned* count;
+  unsigned base;
+};
+
 // Entry points of one symmetry-adapted unit (sym_inst.cu).
 struct SymKernels {
   int (*upload)(const float* w, const float* sym, int nsym);
   int (*launch)(const StepArgs& a, cudaStream_t st, cudaStream_t st_layer);
+  int (*run)(const StepArgs& a, const RunArgs& r, cudaStream_t st);
 };
 
 // Per-(dim,k) entry points, defined in the instantiation units.
@@ -115,6 +129,9 @@ struct KernelSet {
   // chunked layout: chunks without layer elements on st, layer chunks on st_layer (the two
   // launches are independent and may overlap; st_layer may be st)
   int (*launch_chunk)(const StepArgs& a, cudaStream_t st, cudaStream_t st_layer);
+  // chunked layout: several steps in one launch; its CTAs, or 0 (nothing done: launch the steps), or
+  // minus a cudaError_t
+  int (*run)(const StepArgs& a, const RunArgs& r, cudaStream_t st);
   void (*launch_record)(const StepArgs& a, const int* rec_elem, const float* rec_phi,
                         cudaStream_t st);  // d^n for every receiver and shot
 };

@@ -12,18 +12,12 @@
 
 namespace fwi {
 
+// DoF dof, shots s0, s0 + 1, ...; u: the field, u_out: where it goes.
 template <int D, int SG, int MODE>
-__global__ void __launch_bounds__(128) halo_kernel(const StepArgs a, int plain_blocks) {
-  const bool layer = (int)blockIdx.x >= plain_blocks;
-  const int S = a.S, ngrp = S / SG;
-  const int64_t t = (int64_t)(layer ? (int)blockIdx.x - plain_blocks : (int)blockIdx.x) * 128 + threadIdx.x;
-  const int64_t i = ngrp == 1 ? t : t / ngrp;
-  const int s0 = ngrp == 1 ? 0 : (int)(t - i * ngrp) * SG;
-  const int lo = layer ? a.halo_layer : a.h0, hi = layer ? a.h0 + a.hcnt : a.halo_layer;
-  if (i >= hi - lo) return;
-  const int dof = lo + (int)i;
+__device__ __forceinline__ void halo_dof(const StepArgs& a, const float* u, float* u_out, int dof, int s0, bool layer) {
+  const int S = a.S;
   const size_t ix = (size_t)dof * S + s0, rx = (size_t)(dof - a.h0) * S + s0;
-  const Lanes<SG> uo = lanes_ld<SG>(a.u + ix), vo = lanes_ld<SG>(a.v + ix);
+  const Lanes<SG> uo = lanes_ld<SG>(u + ix), vo = lanes_ld<SG>(a.v + ix);
   const Lanes<SG> y = lanes_ldcg<SG>(a.r + rx);
   const float c1 = __ldg(a.cf + dof), c2 = __ldg(a.cf + (size_t)a.N + dof), c3 = __ldg(a.cf + 2 * (size_t)a.N + dof);
   Lanes<SG> zero, vn;
@@ -75,11 +69,22 @@ __global__ void __launch_bounds__(128) halo_kernel(const StepArgs a, int plain_b
   lanes_acc<SG>(un, vn);
   lanes_st<SG>(a.r + rx, zero);
   lanes_st<SG>(a.v + ix, vn);
-  lanes_st<SG>(a.u_out + ix, un);
+  lanes_st<SG>(u_out + ix, un);
   float chk = 0.f;
 #pragma unroll
   for (int k = 0; k < SG; ++k) chk = fmaf(0.f, un.x[k], chk);
   if (!(chk == 0.f)) atomicOr(a.status, 1);
+}
+
+template <int D, int SG, int MODE>
+__global__ void __launch_bounds__(128) halo_kernel(const StepArgs a, int plain_blocks) {
+  const bool layer = (int)blockIdx.x >= plain_blocks;
+  const int ngrp = a.S / SG;
+  const int64_t t = (int64_t)(layer ? (int)blockIdx.x - plain_blocks : (int)blockIdx.x) * 128 + threadIdx.x;
+  const int64_t i = ngrp == 1 ? t : t / ngrp;
+  const int s0 = ngrp == 1 ? 0 : (int)(t - i * ngrp) * SG;
+  const int lo = layer ? a.halo_layer : a.h0, hi = layer ? a.h0 + a.hcnt : a.halo_layer;
+  if (i < hi - lo) halo_dof<D, SG, MODE>(a, a.u, a.u_out, lo + (int)i, s0, layer);
 }
 
 template <int D, int SG>

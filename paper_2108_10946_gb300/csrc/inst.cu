@@ -84,6 +84,12 @@ int launch_chunk_tc_t(const StepArgs& a, int ch0, int nch, cudaStream_t st) {
 
 #endif
 
+const SymKernels& sym(const StepArgs& a) {
+  return a.SG == 4   ? SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 4)
+         : a.SG == 2 ? SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 2)
+                     : SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 1);
+}
+
 // chunks [0, nch0) hold no damping-layer element, chunks [nch0, nch) do
 int launch_chunk(const StepArgs& a, cudaStream_t st, cudaStream_t stl) {
   const int mode = a.mode == 0 ? 0 : (a.ring_u != nullptr ? 2 : 1);
@@ -102,11 +108,9 @@ int launch_chunk(const StepArgs& a, cudaStream_t st, cudaStream_t stl) {
     return rc;
   }
 #endif
-  return (a.SG == 4   ? SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 4)
-          : a.SG == 2 ? SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 2)
-                      : SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, 1))
-      .launch(a, st, stl);
+  return sym(a).launch(a, st, stl);
 }
+int run(const StepArgs& a, const RunArgs& r, cudaStream_t st) { return sym(a).run(a, r, st); }
 
 int upload(const float* dhat, const float* w, const float* sym, int nsym) {
   cudaError_t e = cudaMemcpyToSymbol(c_dhat, dhat, sizeof(float) * D * NN * NN);
@@ -143,5 +147,5 @@ void launch_record(const StepArgs& a, const int* rec_elem, const float* rec_phi,
 extern const KernelSet KMV_CAT(kernels_, KMV_DIM, _, KMV_K) = {D,           KMV_K,       NN,
                                                               NS,          NN - NS,     upload,
                                                               launch_step, launch_chunk,
-                                                              launch_record};
+                                                              run,         launch_record};
 }  // namespace fwi

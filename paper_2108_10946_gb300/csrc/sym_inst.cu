@@ -27,6 +27,7 @@ __constant__ float c_w[NN];
 }  // namespace fwi
 
 #include "chunk_sym.cuh"
+#include "halo.cuh"
 
 namespace fwi {
 namespace {
@@ -36,11 +37,12 @@ constexpr int NT = SymMap<SG>::NT;
 // spills (marine mesh, one gradient of 75 steps: 128.5 ms at 168, 133.1 ms at 128); every other
 // kernel is best at 128 (KMV4, S = 4, 250k triangles: 8.0 ms for 100 steps, 10.9 ms at 204; KMV3,
 // 120k: 8.9 and 9.8 ms).
+#ifndef RUN_MAX
+#define RUN_MAX 304  // most CTAs of a launch of several steps
+#endif
+
 template <int MODE, bool LAYER>
 constexpr int registers() {
-#ifdef SYM_REGS
-  return SYM_REGS;
-#endif
   if (KMV_DIM == 3 && KMV_K == 3) return LAYER ? 255 : MODE == 2 ? 204 : 168;
   return KMV_K == 5 && MODE == 2 ? 168 : 128;
 }
@@ -48,9 +50,123 @@ constexpr int registers() {
 template <int MODE, bool LAYER>
 __global__ void __launch_bounds__(NT, 65536 / (registers<MODE, LAYER>() * NT)) k_sym(const StepArgs a) {
   extern __shared__ __align__(16) float smem_sym[];
-  if constexpr (D == 2) sym_tri_body<NN, NS, MODE, LAYER, SG>(a, smem_sym);
-  else sym_tet_body<NN, NS, MODE, LAYER, SG>(a, smem_sym);
+  const SymStep x{a.u, a.u_out, a.ring_u, a.n, 0};
+  const int c = blockIdx.x + a.ch0, s0 = blockIdx.y * SG;
+  if constexpr (D == 2) sym_tri_body<NN, NS, MODE, LAYER, SG, false>(a, x, smem_sym, c, s0);
+  else sym_tet_body<NN, NS, MODE, LAYER, SG, false>(a, x, smem_sym, c, s0);
 }
+
+// Several steps in one cooperative launch, for meshes whose steps are shorter than launching them:
+// every CTA takes its chunks, all CTAs meet, every thread finishes its halo DoFs, all meet again.
+// A chunk and a halo DoF stay with their CTA, so only what crosses CTAs has to come from L2. Both
+// kinds of chunks are one kernel here.
+__device__ __forceinline__ bool run_meet(unsigned* count, unsigned target) {
+  asm volatile("fence.proxy.async;" ::: "memory");  // (the fields are written as usual, read by bulk copies)
+  __syncthreads();
+  bool ok = true;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(count, 1u);
+    ok = false;
+    for (int i = 0; i < (1 << 22); ++i) {  // bounded: a CTA that gave up never arrives
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+      if ((int)(v - target) >= 0) {
+        ok = true;
+        break;
+      }
+    }
+    asm volatile("fence.proxy.async;" ::: "memory");
+  }
+  return __syncthreads_and(ok);
+}
+
+// (Not inlined: the two kinds' code side by side in the step loop would spill.)
+template <int MODE, bool LAYER>
+__device__ __noinline__ bool run_chunk(const StepArgs& a, const SymStep& x, float* sm, int c, int s0) {
+  if constexpr (D == 2) return sym_tri_body<NN, NS, MODE, LAYER, SG, true>(a, x, sm, c, s0);
+  else return sym_tet_body<NN, NS, MODE, LAYER, SG, true>(a, x, sm, c, s0);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(NT, 65536 / (registers<MODE, true>() * NT))
+    k_run(const __grid_constant__ StepArgs a, const RunArgs r) {
+  extern __shared__ __align__(16) float smem_sym[];
+  const int ngrp = a.S / SG, nwork = a.nch * ngrp, tid = threadIdx.x;
+  if (tid == 0) sym_bar_init(reinterpret_cast<uint64_t*>(smem_sym));
+  __syncthreads();
+  unsigned target = r.base;
+  SymStep x{nullptr, nullptr, nullptr, 0, 0};
+  for (int k = 0; k < r.steps; ++k) {
+    const int rel = r.rel0 + k * r.dir;  // time level less the segment's first
+    x.n = r.n0 + k * r.dir;
+    if (MODE == 0) {  // the levels the gradient needs go to the ring, the others stay in u
+      x.u = r.ring && rel % r.stride == 0 ? r.ring + (size_t)(rel / r.stride) * r.level : a.u;
+      x.u_out = r.ring && (rel + 1) % r.stride == 0 ? r.ring + (size_t)((rel + 1) / r.stride) * r.level : a.u_out;
+    } else {
+      x.u = a.u;
+      x.u_out = a.u_out;
+      x.ring_u = r.ring + (size_t)rel * r.level;
+    }
+    for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
+      const int c = a.nch - 1 - w / ngrp, s0 = w % ngrp * SG;  // the layer's chunks, the longer ones, first
+      const bool ok = c < a.nch0 ? run_chunk<MODE, false>(a, x, smem_sym, c, s0) : run_chunk<MODE, true>(a, x, smem_sym, c, s0);
+      if (!ok) return;
+      x.parity ^= 1;
+      asm volatile("fence.proxy.async;" ::: "memory");  // the next chunk's copies come after these reads
+      __syncthreads();
+    }
+    if (!run_meet(r.count, target += gridDim.x)) {
+      if (tid == 0) atomicOr(a.status, 2);
+      return;
+    }
+    const int64_t items = (int64_t)a.hcnt * ngrp;
+    for (int64_t t = (int64_t)blockIdx.x * NT + tid; t < items; t += (int64_t)gridDim.x * NT) {
+      const int dof = a.h0 + (int)(t / ngrp);
+      halo_dof<D, SG, MODE == 0 ? 0 : 1>(a, x.u, x.u_out, dof, (int)(t % ngrp) * SG, dof >= a.halo_layer);
+    }
+    if (!run_meet(r.count, target += gridDim.x)) {
+      if (tid == 0) atomicOr(a.status, 2);
+      return;
+    }
+  }
+}
+
+// Returns the CTAs of the launch, 0 if the steps are better launched one by one (nothing done), or
+// minus a cudaError_t.
+template <int MODE>
+int run_t(const StepArgs& a, const RunArgs& r, cudaStream_t st) {
+  const size_t bytes =
+      sizeof(float) * (size_t)(a.nch > a.nch0 ? sym_smem<D, NN, NS, SG, MODE, true>(a.T_max, a.SH_max, a.H_max).total
+                                              : sym_smem<D, NN, NS, SG, MODE, false>(a.T_max, a.SH_max, a.H_max).total);
+  if (bytes > 227 * 1024) return 0;
+  static size_t configured[64] = {0};
+  static int nsm[64] = {0};
+  int dev = 0, per = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64) return 0;
+  cudaError_t e = cudaSuccess;
+  if (bytes > configured[dev]) {
+    e = cudaFuncSetAttribute(k_run<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return -(int)e;
+    configured[dev] = bytes;
+  }
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_run<MODE>, NT, bytes);
+  if (e != cudaSuccess) return -(int)e;
+  const int64_t nwork = (int64_t)a.nch * (a.S / SG);
+  const int64_t room = (int64_t)per * nsm[dev];
+  if (nwork > RUN_MAX || nwork > room) return 0;
+  const int grid = (int)std::min(nwork, room);
+  StepArgs b = a;
+  RunArgs q = r;
+  b.ch0 = 0;
+  b.ch1 = a.nch;
+  void* args[] = {&b, &q};
+  e = cudaLaunchCooperativeKernel((const void*)k_run<MODE>, dim3((unsigned)grid), dim3(NT), args, bytes, st);
+  return e == cudaSuccess ? grid : -(int)e;
+}
+int run(const StepArgs& a, const RunArgs& r, cudaStream_t st) { return a.mode == 0 ? run_t<0>(a, r, st) : run_t<2>(a, r, st); }
 
 template <int MODE, bool LAYER>
 int launch_t(const StepArgs& a, int ch0, int nch, cudaStream_t st) {
@@ -132,5 +248,5 @@ int upload(const float* w, const float* sym, int nsym) {
 
 #define SYM_CAT2(a, b, c, d) a##b##_##c##_##d
 #define SYM_CAT(a, b, c, d) SYM_CAT2(a, b, c, d)
-extern const SymKernels SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, KMV_SG) = {upload, launch};
+extern const SymKernels SYM_CAT(sym_kernels_, KMV_DIM, KMV_K, KMV_SG) = {upload, launch, run};
 }  // namespace fwi

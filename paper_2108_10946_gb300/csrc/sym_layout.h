@@ -60,9 +60,22 @@ struct TriSym : TriOrbits<NN> {
   FWI_HD static constexpr int size_of(char k) { return k == 'X' ? 6 : k == 'C' ? 1 : 3; }
   FWI_HD static constexpr int vecs_of(char k) { return k == 'X' ? 2 : k == 'C' ? 0 : 1; }
   // first local node, first three-vector and number of odd three-vectors before orbit o
-  FWI_HD static constexpr int base(int o) { return o == 0 ? 0 : base(o - 1) + size_of(B::kind(o - 1)); }
-  FWI_HD static constexpr int vec(int o) { return o == 0 ? 0 : vec(o - 1) + vecs_of(B::kind(o - 1)); }
-  FWI_HD static constexpr int odd(int o) { return o == 0 ? 0 : odd(o - 1) + (B::kind(o - 1) == 'X'); }
+  // (loops, not recursion: a device function that is not folded must not call itself)
+  FWI_HD static constexpr int base(int o) {
+    int n = 0;
+    for (int i = 0; i < o; ++i) n += size_of(B::kind(i));
+    return n;
+  }
+  FWI_HD static constexpr int vec(int o) {
+    int n = 0;
+    for (int i = 0; i < o; ++i) n += vecs_of(B::kind(i));
+    return n;
+  }
+  FWI_HD static constexpr int odd(int o) {
+    int n = 0;
+    for (int i = 0; i < o; ++i) n += B::kind(i) == 'X';
+    return n;
+  }
   // coordinates: NA1 symmetric sums (one per orbit), NA2 antisymmetric sums (one per odd
   // three-vector) and NV two-component vectors
   static constexpr int NA1 = NO, NA2 = odd(NO), NV = vec(NO);
@@ -81,9 +94,9 @@ struct TriSym : TriOrbits<NN> {
   // (odd) and differences (even).
   static constexpr int EVEN = NA1 + NV, ODD = NA2 + NV;
   FWI_HD static constexpr int tab(int o) {
-    return o == 0 ? 0
-                  : tab(o - 1) + (B::kind(o - 1) == 'X' ? 2 * (EVEN + ODD)
-                                  : B::kind(o - 1) == 'C' ? NV : EVEN + ODD);
+    int n = 0;
+    for (int i = 0; i < o; ++i) n += B::kind(i) == 'X' ? 2 * (EVEN + ODD) : B::kind(i) == 'C' ? NV : EVEN + ODD;
+    return n;
   }
   static constexpr int TAB = tab(NO);
   // Rolled form (KMV5): the table holds the X orbits' coefficients, then the T orbits'; first slots

@@ -70,30 +70,30 @@ __device__ __forceinline__ void tri_analyse(TriCoef<V, NN>& c, F load) {
   using T = TriSym<NN>;
   if constexpr (O < T::NO) {
     constexpr char K = T::kind(O);
+    constexpr int QB = T::base(O), I = T::vec(O), J = T::odd(O);
     if constexpr (K == 'C') {
-      c.s1[O] = load(T::node(O, 0));
+      c.s1[O] = load(QB + T::place(K, 0, 0));
     } else if constexpr (K == 'X') {
       V p[3], m[3];
 #pragma unroll
       for (int v = 0; v < 3; ++v) {
-        const V a = load(T::node(O, v, 0)), b = load(T::node(O, v, 1));
+        const V a = load(QB + T::place(K, v, 0)), b = load(QB + T::place(K, v, 1));
         p[v] = add2(a, b);
         m[v] = sub2(a, b);
       }
-      constexpr int i = T::vec(O);
       const V h = add2(p[1], p[2]), g = add2(m[1], m[2]);
       c.s1[O] = add2(p[0], h);
-      c.e1[i] = fma2(dup<V>(-0.5f), h, p[0]);
-      c.e2[i] = sub2(p[1], p[2]);
-      c.s2[T::odd(O)] = add2(m[0], g);
-      c.e1[i + 1] = mul2(dup<V>(0.75f), sub2(m[2], m[1]));
-      c.e2[i + 1] = fma2(dup<V>(-0.5f), g, m[0]);
+      c.e1[I] = fma2(dup<V>(-0.5f), h, p[0]);
+      c.e2[I] = sub2(p[1], p[2]);
+      c.s2[J] = add2(m[0], g);
+      c.e1[I + 1] = mul2(dup<V>(0.75f), sub2(m[2], m[1]));
+      c.e2[I + 1] = fma2(dup<V>(-0.5f), g, m[0]);
     } else {
-      const V x0 = load(T::node(O, 0)), x1 = load(T::node(O, 1)), x2 = load(T::node(O, 2));
+      const V x0 = load(QB + T::place(K, 0, 0)), x1 = load(QB + T::place(K, 1, 0)), x2 = load(QB + T::place(K, 2, 0));
       const V h = add2(x1, x2);
       c.s1[O] = add2(x0, h);
-      c.e1[T::vec(O)] = fma2(dup<V>(-0.5f), h, x0);
-      c.e2[T::vec(O)] = sub2(x1, x2);
+      c.e1[I] = fma2(dup<V>(-0.5f), h, x0);
+      c.e2[I] = sub2(x1, x2);
     }
     tri_analyse<V, NN, O + 1>(c, load);
   }
@@ -105,24 +105,24 @@ __device__ __forceinline__ void tri_gather_back(const TriCoef<V, NN>& c, F store
   using T = TriSym<NN>;
   if constexpr (O < T::NO) {
     constexpr char K = T::kind(O);
+    constexpr int QB = T::base(O), I = T::vec(O), J = T::odd(O);
     if constexpr (K == 'C') {
-      store(T::node(O, 0), c.s1[O]);
+      store(QB + T::place(K, 0, 0), c.s1[O]);
     } else {
-      constexpr int i = T::vec(O);
-      const V t = fma2(dup<V>(-0.5f), c.e1[i], c.s1[O]);
-      const V p[3] = {add2(c.s1[O], c.e1[i]), add2(t, c.e2[i]), sub2(t, c.e2[i])};
+      const V t = fma2(dup<V>(-0.5f), c.e1[I], c.s1[O]);
+      const V p[3] = {add2(c.s1[O], c.e1[I]), add2(t, c.e2[I]), sub2(t, c.e2[I])};
       if constexpr (K == 'X') {
-        const V s = c.s2[T::odd(O)];
-        const V r = fma2(dup<V>(-0.5f), c.e2[i + 1], s);
-        const V m[3] = {add2(s, c.e2[i + 1]), fma2(dup<V>(-0.75f), c.e1[i + 1], r), fma2(dup<V>(0.75f), c.e1[i + 1], r)};
+        const V s = c.s2[J];
+        const V r = fma2(dup<V>(-0.5f), c.e2[I + 1], s);
+        const V m[3] = {add2(s, c.e2[I + 1]), fma2(dup<V>(-0.75f), c.e1[I + 1], r), fma2(dup<V>(0.75f), c.e1[I + 1], r)};
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
-          store(T::node(O, v, 0), add2(p[v], m[v]));
-          store(T::node(O, v, 1), sub2(p[v], m[v]));
+          store(QB + T::place(K, v, 0), add2(p[v], m[v]));
+          store(QB + T::place(K, v, 1), sub2(p[v], m[v]));
         }
       } else {
 #pragma unroll
-        for (int v = 0; v < 3; ++v) store(T::node(O, v), p[v]);
+        for (int v = 0; v < 3; ++v) store(QB + T::place(K, v, 0), p[v]);
       }
     }
     tri_gather_back<V, NN, O + 1>(c, store);
