@@ -177,7 +177,7 @@ __device__ __forceinline__ void sym_cp_live(float* dst, const float* src) {
 }
 template <int D, int NN, int NS, int SG, int MODE, bool LAYER, bool RUN>
 __device__ __forceinline__ void sym_load(const StepArgs& a, const SymStep& x, const SymDesc& cd, const SymSmem& L,
-                                         float* sm, uint64_t* bar, int s0, int tid) {
+                                         float* sm, uint64_t* bar, int chunk, int s0, int tid) {
   constexpr int NI = NN - NS, NT = SymMap<SG>::NT;
   constexpr bool GRAD = MODE == 2, OM = LAYER && D == 3 && MODE == 0;
   constexpr int PSI = LAYER ? sym_psi<D, MODE>() : 0;
@@ -226,8 +226,8 @@ __device__ __forceinline__ void sym_load(const StepArgs& a, const SymStep& x, co
     if (LAYER && D == 3) sym_prefetch(a.lpsi + pi0 * 4, on * 4);
     if (LAYER && D == 3 && S == SG) sym_prefetch(a.Y + pi0 * SG, on * SG);
     // and the ranges of the chunk a wave of CTAs further on
-    const int nc = blockIdx.x + a.ch0 + a.wave;
-    if (!RUN && nc < a.ch1) {
+    const int nc = chunk + a.wave;
+    if (!RUN && nc >= (LAYER ? a.nch0 : 0) && nc < (LAYER ? a.nch : a.nch0)) {
       const SymDesc nx = sym_desc(a, nc);
       const int nn = nx.nsh + nx.ne * NI;
       sym_prefetch(reinterpret_cast<const float*>(a.smeta) + nx.meta, nx.meta_n);
@@ -512,7 +512,7 @@ __device__ __forceinline__ bool sym_tri_body(const StepArgs& a, const SymStep& x
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm);
   if (!RUN && tid == 0) sym_bar_init(bar);  // (the thread that issues the barrier's copies)
   const SymDesc cd = sym_desc(a, chunk);
-  sym_load<2, NN, NS, SG, MODE, LAYER, RUN>(a, x, cd, L, sm, bar, s0, tid);
+  sym_load<2, NN, NS, SG, MODE, LAYER, RUN>(a, x, cd, L, sm, bar, chunk, s0, tid);
   if (!RUN) __syncthreads();  // the barrier is set up before anyone asks it
   const int el = tid / M::PER, ln = tid % M::PER * M::LANES;  // element, first shot of the group
   const bool act = el < cd.ne;
@@ -615,7 +615,10 @@ __device__ __forceinline__ bool sym_tri_body(const StepArgs& a, const SymStep& x
   if (act) {
     tri_gather_back<V, NN>(Y, [&](int q, V y) { st(own(L.ys, L.yb, q), y); });
   }
-  constexpr int B = 4;
+  // DoFs per thread whose update reads are in flight at a time. More hide more latency and take
+  // registers from CTAs: KMV2, one shot (2M triangles, 50 steps): 4.69 ms with four, 3.71 ms with one;
+  // KMV4 segments 6.90 and 6.71 ms with four and two; KMV5, one shot, 6.26 and 6.54 ms.
+  constexpr int B = NN == 7 ? 1 : NN == 30 && SG == 1 ? 4 : 2;
   SymRound<SG, B> first;
   first.load(a, cd, cd.nsh + nb, s0, tid, M::NT);
   __syncthreads();
@@ -737,7 +740,7 @@ __device__ __forceinline__ bool sym_tet_body(const StepArgs& a, const SymStep& x
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm);
   if (!RUN && tid == 0) sym_bar_init(bar);  // (the thread that issues the barrier's copies)
   const SymDesc cd = sym_desc(a, chunk);
-  sym_load<3, NN, NS, SG, MODE, LAYER, RUN>(a, x, cd, L, sm, bar, s0, tid);
+  sym_load<3, NN, NS, SG, MODE, LAYER, RUN>(a, x, cd, L, sm, bar, chunk, s0, tid);
   if (!RUN) __syncthreads();  // the barrier is set up before anyone asks it
   const int el = tid / M::PER, ln = tid % M::PER * M::LANES;  // element, first shot of the group
   const bool act = el < cd.ne;

@@ -43,7 +43,8 @@ struct StepArgs {
   // (node * PE + element), their pointers (PE = sym_pe)
   const int* sdesc;
   const unsigned short* smeta;
-  int ch1, wave;                // one past the last chunk of a launch; CTAs that run at a time
+  int both;                     // 1: both kinds of chunks (with and without layer) in one launch
+  int wave;                     // how many chunks further on a CTA of the next wave works
   const unsigned char* splain;  // [nch] 1: c1 = 1 and c3 = 0 for every owned DoF
   int T_max, SH_max;   // largest chunk table and most shared DoFs of a chunk
   int p_own, p_halo;   // layer index of an owned / halo DoF of a layer chunk: dof - shift

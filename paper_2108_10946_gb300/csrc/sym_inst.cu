@@ -36,7 +36,8 @@ constexpr int NT = SymMap<SG>::NT;
 // the others. KMV5 gradient steps hold more at a time and lose less to a fourth CTA less than to
 // spills (marine mesh, one gradient of 75 steps: 128.5 ms at 168, 133.1 ms at 128); every other
 // kernel is best at 128 (KMV4, S = 4, 250k triangles: 8.0 ms for 100 steps, 10.9 ms at 204; KMV3,
-// 120k: 8.9 and 9.8 ms).
+// 120k: 8.9 and 9.8 ms), but KMV2's at one shot, which do little with what they load (2M triangles,
+// 50 steps: 3.54 ms at 48, 3.71 ms at 80).
 #ifndef RUN_MAX
 #define RUN_MAX 304  // most CTAs of a launch of several steps
 #endif
@@ -44,7 +45,7 @@ constexpr int NT = SymMap<SG>::NT;
 template <int MODE, bool LAYER>
 constexpr int registers() {
   if (KMV_DIM == 3 && KMV_K == 3) return LAYER ? 255 : MODE == 2 ? 204 : 168;
-  return KMV_K == 5 && MODE == 2 ? 168 : 128;
+  return KMV_K == 5 && MODE == 2 ? 168 : KMV_DIM == 2 && KMV_K == 2 && SG == 1 ? 48 : 128;
 }
 
 template <int MODE, bool LAYER>
@@ -54,6 +55,21 @@ __global__ void __launch_bounds__(NT, 65536 / (registers<MODE, LAYER>() * NT)) k
   const int c = blockIdx.x + a.ch0, s0 = blockIdx.y * SG;
   if constexpr (D == 2) sym_tri_body<NN, NS, MODE, LAYER, SG, false>(a, x, smem_sym, c, s0);
   else sym_tet_body<NN, NS, MODE, LAYER, SG, false>(a, x, smem_sym, c, s0);
+}
+
+// Both kinds of chunks in one launch, the layer's (the longer ones) first.
+template <int MODE>
+__global__ void __launch_bounds__(NT, 65536 / (registers<MODE, true>() * NT)) k_both(const StepArgs a) {
+  extern __shared__ __align__(16) float smem_sym[];
+  const SymStep x{a.u, a.u_out, a.ring_u, a.n, 0};
+  const int c = a.nch - 1 - blockIdx.x, s0 = blockIdx.y * SG;
+  if (c >= a.nch0) {
+    if constexpr (D == 2) sym_tri_body<NN, NS, MODE, true, SG, false>(a, x, smem_sym, c, s0);
+    else sym_tet_body<NN, NS, MODE, true, SG, false>(a, x, smem_sym, c, s0);
+  } else {
+    if constexpr (D == 2) sym_tri_body<NN, NS, MODE, false, SG, false>(a, x, smem_sym, c, s0);
+    else sym_tet_body<NN, NS, MODE, false, SG, false>(a, x, smem_sym, c, s0);
+  }
 }
 
 // Several steps in one cooperative launch, for meshes whose steps are shorter than launching them:
@@ -161,51 +177,52 @@ int run_t(const StepArgs& a, const RunArgs& r, cudaStream_t st) {
   StepArgs b = a;
   RunArgs q = r;
   b.ch0 = 0;
-  b.ch1 = a.nch;
   void* args[] = {&b, &q};
   e = cudaLaunchCooperativeKernel((const void*)k_run<MODE>, dim3((unsigned)grid), dim3(NT), args, bytes, st);
   return e == cudaSuccess ? grid : -(int)e;
 }
 int run(const StepArgs& a, const RunArgs& r, cudaStream_t st) { return a.mode == 0 ? run_t<0>(a, r, st) : run_t<2>(a, r, st); }
 
-template <int MODE, bool LAYER>
-int launch_t(const StepArgs& a, int ch0, int nch, cudaStream_t st) {
+// One launch of `kernel` over chunks [ch0, ch0 + nch), downwards from the last if down.
+int launch_t(void (*kernel)(const StepArgs), int which, size_t bytes, const StepArgs& a, int ch0, int nch, bool down,
+             cudaStream_t st) {
   if (nch <= 0) return 0;
-  const size_t bytes =
-      sizeof(float) * (size_t)sym_smem<D, NN, NS, SG, MODE, LAYER>(a.T_max, a.SH_max, a.H_max).total;
   if (bytes > 227 * 1024) return (int)cudaErrorInvalidValue;
-  static size_t configured[64] = {0};
+  static size_t configured[9][64] = {{0}};
+  static int wave[9][64] = {{0}};  // CTAs that run at a time
   int dev = 0;
   cudaGetDevice(&dev);
-  static int wave[64] = {0};  // CTAs that run at a time
   if (dev < 0 || dev >= 64) return (int)cudaErrorInvalidDevice;
-  if (bytes > configured[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(k_sym<MODE, LAYER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (bytes > configured[which][dev]) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     int per = 0, nsm = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sym<MODE, LAYER>, NT, bytes);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, NT, bytes);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return (int)e;
-    wave[dev] = per * nsm;
-    configured[dev] = bytes;
+    wave[which][dev] = per * nsm;
+    configured[which][dev] = bytes;
   }
   StepArgs b = a;
   b.ch0 = ch0;
-  b.ch1 = ch0 + nch;
-  b.wave = wave[dev];
-  k_sym<MODE, LAYER><<<dim3((unsigned)nch, (unsigned)(a.S / SG)), NT, bytes, st>>>(b);
+  b.wave = down ? -wave[which][dev] : wave[which][dev];
+  kernel<<<dim3((unsigned)nch, (unsigned)(a.S / SG)), NT, bytes, st>>>(b);
   return 0;
 }
+template <int MODE>
+int launch_mode(const StepArgs& a, cudaStream_t st, cudaStream_t stl) {
+  const size_t plain = sizeof(float) * (size_t)sym_smem<D, NN, NS, SG, MODE, false>(a.T_max, a.SH_max, a.H_max).total;
+  const size_t layer = sizeof(float) * (size_t)sym_smem<D, NN, NS, SG, MODE, true>(a.T_max, a.SH_max, a.H_max).total;
+  if (a.both) return launch_t(k_both<MODE>, 6 + MODE, std::max(plain, layer), a, 0, a.nch, true, st);
+  const int rc = launch_t(k_sym<MODE, false>, MODE, plain, a, 0, a.nch0, false, st);
+  return rc ? rc : launch_t(k_sym<MODE, true>, 3 + MODE, layer, a, a.nch0, a.nch - a.nch0, false, stl);
+}
 
-// chunks [0, nch0) hold no damping-layer element, chunks [nch0, nch) do
+// Chunks [0, nch0) hold no damping-layer element, chunks [nch0, nch) do: one launch each, on st and
+// stl, or (a.both) both in one on st.
 int launch(const StepArgs& a, cudaStream_t st, cudaStream_t stl) {
-  const int mode = a.mode == 0 ? 0 : (a.ring_u != nullptr ? 2 : 1), nl = a.nch - a.nch0;
-  int rc = mode == 0   ? launch_t<0, false>(a, 0, a.nch0, st)
-           : mode == 1 ? launch_t<1, false>(a, 0, a.nch0, st)
-                       : launch_t<2, false>(a, 0, a.nch0, st);
-  if (rc) return rc;
-  return mode == 0   ? launch_t<0, true>(a, a.nch0, nl, stl)
-         : mode == 1 ? launch_t<1, true>(a, a.nch0, nl, stl)
-                     : launch_t<2, true>(a, a.nch0, nl, stl);
+  return a.mode == 0             ? launch_mode<0>(a, st, stl)
+         : a.ring_u == nullptr ? launch_mode<1>(a, st, stl)
+                                 : launch_mode<2>(a, st, stl);
 }
 
 int upload(const float* w, const float* sym, int nsym) {
