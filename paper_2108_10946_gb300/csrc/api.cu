@@ -156,7 +156,8 @@ struct fwi_mesh {
   float* d_c = nullptr;
   float* d_cf = nullptr;     // [3][N]
   float* d_lcf = nullptr;    // [Nl][count]
-  double* d_M = nullptr;
+  double *d_M = nullptr, *d_Mb = nullptr, *d_sigma = nullptr;  // lumped masses, damping profile [N][dim]
+  double* d_c64 = nullptr;   // [N] the velocity as given
   unsigned char* d_mask = nullptr;
   int* d_bub = nullptr;
   int* d_chunks = nullptr;   // [nch][6]: e0, ne, own_lo, own_n, nsh, halo_ptr
@@ -561,6 +562,7 @@ void build_incidence(fwi_mesh* m) {
     for (int l = 0; l <= nloc; ++l) gp[l] = (uint16_t)cnt[l];
     for (int e = e0; e < e0 + ne; ++e)
       for (int q = 0; q < ns; ++q) ge[cnt[place(q, e)]++] = (uint16_t)(q * P + e - e0);
+    // (the second entry's bit 16, any undamped DoF, follows once the damping profile is known)
     const int d[8] = {e0, ne, own, nsh, hp, hn, (int)(at / 2), (int)(size / 2)};
     std::copy(d, d + 8, &m->sdesc[(size_t)c * 8]);
     m->T_max = std::max(m->T_max, own_n + hn);
@@ -853,6 +855,18 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
         if (m->pidx[i] < 0) m->pidx[i] = m->Nl++;
       }
   }
+  if (m->layout == 0)  // chunks with an undamped DoF: the others' gradient is masked whatever c is
+    for (int c = 0; c < m->nch(); ++c) {
+      auto undamped = [&](int i) {
+        double t = 0;
+        for (int k = 0; k < d; ++k) t += m->sigma[(size_t)i * d + k];
+        return !(t > 0);
+      };
+      bool keep = c < m->nch0;
+      for (int i = m->ch_own_lo[c]; i < m->ch_own_lo[c + 1] && !keep; ++i) keep = undamped(i);
+      for (int h = m->ch_halo_ptr[c]; h < m->ch_halo_ptr[c + 1] && !keep; ++h) keep = undamped(m->halo_ids[h]);
+      m->sdesc[(size_t)c * 8 + 1] |= keep ? 1 << 16 : 0;
+    }
   // lumped boundary mass: facets owned by one element
   m->Mb.assign(N, 0);
   if (m->p.absorbing) {
@@ -985,7 +999,8 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
   }
   if ((rc = upload(&m->d_conn, conn_dev)) || (rc = upload(&m->d_geo, geo)) ||
       (rc = upload(&m->d_lgeo, lgeo)) || (rc = upload(&m->d_pidx, m->pidx)) ||
-      (rc = upload(&m->d_M, m->M))) {
+      (rc = upload(&m->d_M, m->M)) || (rc = upload(&m->d_Mb, m->Mb)) ||
+      (rc = upload(&m->d_sigma, m->sigma))) {
     fwi_mesh_free(m.release());
     return rc;
   }
@@ -1094,92 +1109,49 @@ int fwi_set_velocity(fwi_mesh* m, const double* c) {
     double rho = gershgorin(m);
     m->dt = m->p.cfl_factor * 2.0 / std::sqrt(rho);
   }
-  const double dt = m->dt;
-  std::vector<float> c2(N), cv(N), cf((size_t)3 * N);
-  const int LC = fwi::layer_coef_count(d);
-  std::vector<float> lcf((size_t)m->Nl * LC, 0.f);
-  std::vector<float> lpsi((size_t)m->Nl * (d == 2 ? 1 : 4)), lcs((size_t)m->Nl * (d == 2 ? 8 : 12));
-  std::vector<unsigned char> mask(N);
-  for (int i = 0; i < N; ++i) {
-    const double* s = &m->sigma[(size_t)i * d];
-    double tr = 0, m3, det1 = 1;
-    for (int k = 0; k < d; ++k) tr += s[k];
-    if (d == 2) {
-      m3 = s[0] * s[1];
-    } else {
-      m3 = s[0] * s[1] + s[0] * s[2] + s[1] * s[2];
-      det1 = s[0] * s[1] * s[2];
-    }
-    const double a = tr + c[i] * m->Mb[i] / m->M[i];
-    const double den = 1.0 + 0.5 * a * dt;
-    c2[i] = (float)(c[i] * c[i]);
-    cv[i] = (float)c[i];
-    cf[i] = (float)((1.0 - 0.5 * a * dt) / den);
-    cf[(size_t)N + i] = (float)(dt * dt / (m->M[i] * den));
-    cf[(size_t)2 * N + i] = (float)(dt * dt * m3 / den);
-    const bool damped = tr > 0;
-    mask[i] = (!damped && !(m->p.water_speed > 0 && c[i] < m->p.water_speed)) ? 1 : 0;
-    if (m->pidx[i] >= 0) {
-      float* L = &lcf[(size_t)m->pidx[i] * LC];
-      for (int k = 0; k < d; ++k) {
-        double others = tr - s[k];
-        double psi2 = s[k] - others;
-        double dk = 1.0 + 0.5 * dt * s[k];
-        L[k] = (float)((1.0 - 0.5 * dt * s[k]) / dk);
-        L[d + k] = (float)(dt * psi2 * c[i] * c[i] / (m->M[i] * dk));
-        L[2 * d + k] = (float)(dt / (m->M[i] * dk));
-        L[3 * d + k] = (float)(psi2 * c[i] * c[i]);
-        if (d == 2 && k == 0) lpsi[m->pidx[i]] = L[3 * d];
-        if (d == 3) {
-          double psi3 = 1;
-          for (int l = 0; l < 3; ++l)
-            if (l != k) psi3 *= s[l];
-          L[4 * d + k] = (float)(dt * psi3 * c[i] * c[i] / (m->M[i] * dk));
-          L[5 * d + k] = (float)(psi3 * c[i] * c[i]);
-        }
-      }
-      if (d == 3) {
-        L[6 * d + 0] = (float)(dt * dt * det1 / den);
-        L[6 * d + 1] = (float)(dt * dt / den);
-        L[6 * d + 2] = (float)(dt * det1);
-        L[6 * d + 3] = (float)(dt / m->M[i]);
-      }
-      if (m->layout == 0) {
-        float* Q = &lcs[(size_t)m->pidx[i] * (d == 2 ? 8 : 12)];
-        if (d == 2) {
-          std::copy(L, L + 8, Q);
-        } else {
-          const float q[12] = {L[0], L[1], L[2], L[18], L[6], L[7], L[8], L[21], L[19], L[20], 0.f, 0.f};
-          std::copy(q, q + 12, Q);
-          for (int k = 0; k < 3; ++k) lpsi[(size_t)m->pidx[i] * 4 + k] = (float)s[k];
-        }
-      }
-    }
+  // the coefficients of every DoF, and what depends on them per chunk, are formed on the device
+  const size_t Nl = (size_t)m->Nl;
+  const bool lcf = m->layout == 1 || m->use_tc;  // the layer records of the plain and tensor-core steps
+  int rc = 0;
+  auto room = [&](auto** p, size_t count) {  // allocated by the first call
+    if (!rc && !*p) rc = dalloc(p, count);
+  };
+  room(&m->d_c64, (size_t)N);
+  room(&m->d_c2, (size_t)N);
+  room(&m->d_c, (size_t)N);
+  room(&m->d_cf, (size_t)3 * N);
+  room(&m->d_mask, (size_t)N);
+  if (lcf) room(&m->d_lcf, Nl * fwi::layer_coef_count(d));
+  if (m->layout == 0) {
+    room(&m->d_lpsi, Nl * (d == 2 ? 1 : 4));
+    room(&m->d_lcs, Nl * (d == 2 ? 8 : 12));
+    room(&m->d_splain, (size_t)m->nch());
   }
-  // chunks whose owned DoFs are neither damped nor on an absorbing boundary: v' = v - c2 y
-  std::vector<unsigned char> plain(m->layout == 0 ? m->nch() : 0, 1);
-  for (size_t ch = 0; ch < plain.size(); ++ch)
-    for (int i = m->ch_own_lo[ch]; i < m->ch_own_lo[ch + 1] && plain[ch]; ++i)
-      plain[ch] = cf[i] == 1.f && cf[(size_t)2 * N + i] == 0.f;
-  dfree(m->d_c2);
-  dfree(m->d_c);
-  dfree(m->d_cf);
-  dfree(m->d_lcf);
-  dfree(m->d_mask);
-  dfree(m->d_splain);
-  dfree(m->d_lpsi);
-  m->d_splain = nullptr;
-  m->d_lpsi = nullptr;
-  dfree(m->d_lcs);
-  m->d_lcs = nullptr;
-  m->d_c2 = m->d_c = m->d_cf = m->d_lcf = nullptr;
-  m->d_mask = nullptr;
-  int rc;
-  if ((rc = upload(&m->d_c2, c2)) || (rc = upload(&m->d_c, cv)) || (rc = upload(&m->d_cf, cf)) ||
-      (rc = upload(&m->d_lcf, lcf)) || (rc = upload(&m->d_mask, mask)) ||
-      (rc = upload(&m->d_splain, plain)) || (rc = upload(&m->d_lpsi, lpsi)) ||
-      (rc = upload(&m->d_lcs, lcs)))
-    return rc;
+  if (rc) return rc;
+  CUDA_TRY(cudaMemcpy(m->d_c64, c, (size_t)N * sizeof(double), cudaMemcpyHostToDevice));
+  fwi::VelocityArgs v{};
+  v.N = N;
+  v.dim = d;
+  v.nch = m->layout == 0 ? m->nch() : 0;
+  v.dt = m->dt;
+  v.water = m->p.water_speed;
+  v.c = m->d_c64;
+  v.M = m->d_M;
+  v.Mb = m->d_Mb;
+  v.sigma = m->d_sigma;
+  v.pidx = m->d_pidx;
+  v.sdesc = m->d_sdesc;
+  v.c2 = m->d_c2;
+  v.cvel = m->d_c;
+  v.cf = m->d_cf;
+  v.lcf = lcf ? m->d_lcf : nullptr;
+  v.lpsi = m->d_lpsi;
+  v.lcs = m->d_lcs;
+  v.mask = m->d_mask;
+  v.splain = m->d_splain;
+  fwi::launch_velocity(v);
+  CUDA_TRY(cudaGetLastError());
+  CUDA_TRY(cudaStreamSynchronize(nullptr));
   m->have_velocity = true;
   return 0;
 }
@@ -1987,7 +1959,7 @@ int fwi_profile_read(fwi_batch* b, double* ms, int64_t* steps) {
 int fwi_mesh_free(fwi_mesh* m) {
   if (!m) return 0;
   void* ptrs[] = {m->d_conn, m->d_geo, m->d_lgeo, m->d_pidx, m->d_c2, m->d_c, m->d_cf,
-                  m->d_lcf, m->d_M, m->d_mask, m->d_bub, m->d_chunks, m->d_halo, m->d_lconn,
+                  m->d_lcf, m->d_M, m->d_Mb, m->d_sigma, m->d_c64, m->d_mask, m->d_bub, m->d_chunks, m->d_halo, m->d_lconn,
                   m->d_sdesc, m->d_smeta, m->d_splain, m->d_lpsi, m->d_lcs};
   for (void* p : ptrs) dfree(p);
   delete m;

@@ -154,13 +154,13 @@ template <int D>
 constexpr int SYM_LCS = D == 2 ? 8 : 12;
 
 struct SymDesc {
-  int e0, ne, own, nsh, hp, hn, meta, meta_n, plain;
+  int e0, ne, own, nsh, hp, hn, meta, meta_n, plain, keep;  // keep: an undamped DoF
 };
 __device__ __forceinline__ SymDesc sym_desc(const StepArgs& a, int c) {
   SymDesc d;
   const int4* p = reinterpret_cast<const int4*>(a.sdesc) + 2 * c;
   const int4 x = __ldg(p), y = __ldg(p + 1);
-  d.e0 = x.x, d.ne = x.y, d.own = x.z, d.nsh = x.w;
+  d.e0 = x.x, d.ne = x.y & 0xffff, d.keep = x.y >> 16, d.own = x.z, d.nsh = x.w;
   d.hp = y.x, d.hn = y.y, d.meta = y.z, d.meta_n = y.w;
   d.plain = __ldg(a.splain + c);
   return d;
@@ -191,7 +191,7 @@ __device__ __forceinline__ void sym_load(const StepArgs& a, const SymStep& x, co
     SymRun u{}, f{}, ps{}, om{}, p1{}, p2{};
     if (S == SG) {
       u = sym_run(x.u + i0, on * SG);
-      if (GRAD) f = sym_run(x.ring_u + i0, on * SG);
+      if (GRAD && (D == 3 || cd.keep)) f = sym_run(x.ring_u + i0, on * SG);
     }
     if (LAYER) {
       if (S == SG) {
@@ -254,7 +254,7 @@ __device__ __forceinline__ void sym_load(const StepArgs& a, const SymStep& x, co
     for (int l = tid; l < on; l += NT) {
       const size_t dof = (size_t)(cd.own + l);
       sym_cp<4 * SG>(us + l * SG, x.u + dof * S + s0);
-      if (GRAD) sym_cp<4 * SG>(fs + l * SG, x.ring_u + dof * S + s0);
+      if (GRAD && (D == 3 || cd.keep)) sym_cp<4 * SG>(fs + l * SG, x.ring_u + dof * S + s0);
       if (LAYER)
 #pragma unroll
         for (int k = 0; k < D; ++k)
@@ -268,7 +268,7 @@ __device__ __forceinline__ void sym_load(const StepArgs& a, const SymStep& x, co
     const int id = __ldg(a.halo + cd.hp + h), l = on + h;
     reinterpret_cast<int*>(sm + L.ids)[h] = id;
     sym_cp_live<4 * SG, RUN>(us + l * SG, x.u + (size_t)id * S + s0);
-    if (GRAD) sym_cp<4 * SG>(fs + l * SG, x.ring_u + (size_t)id * S + s0);
+    if (GRAD && (D == 3 || cd.keep)) sym_cp<4 * SG>(fs + l * SG, x.ring_u + (size_t)id * S + s0);
     sym_cp<4>(cs + l, a.c2 + id);
     if (LAYER) {
       const size_t pi = (size_t)(id - a.p_halo);
@@ -403,7 +403,7 @@ __device__ __forceinline__ void sym_finish(const StepArgs& a, const SymStep& x, 
       if constexpr (D == 3 && MODE != 0) lanes_add<SG>(a.Yacc + pi * S + s0, sym_sum<SG>(sm + L.ws, ge, b, e));
     }
   }
-  if constexpr (GRAD) {  // 2 c of the integrand here, once per DoF
+  if (GRAD && (D == 3 || cd.keep)) {  // 2 c of the integrand here, once per DoF
     auto put = [&](int dof, const Lanes<SG>& g) {
       const float c = 2.f * __ldg(a.cvel + dof);
       if (a.grad_lanes) {  // one segment accumulator per shot, [S][N]
@@ -518,6 +518,9 @@ __device__ __forceinline__ bool sym_tri_body(const StepArgs& a, const SymStep& x
   const bool act = el < cd.ne;
   const int ee = act ? el : 0, e = cd.e0 + ee, nb = cd.ne * NI;
   const int bub = cd.nsh + ee * NI;
+  // a damped chunk's gradient is masked: a plain adjoint step there. (Marine mesh: 87 -> 82 ms a
+  // gradient. Tetrahedra lose more to the second path's registers: 22.9 -> 23.8 ms, KMV2.)
+  const bool grad = GRAD && (!LAYER || cd.keep);
   const int in0 = __ldg(a.cslot + chunk), in1 = __ldg(a.cslot + chunk + 1);  // sources' and receivers' elements
   const size_t i0 = (size_t)cd.own * S + s0, pi0 = (size_t)(cd.own - a.p_own);
   const uint16_t* lq = reinterpret_cast<const uint16_t*>(sm + L.meta) + ee;
@@ -547,7 +550,7 @@ __device__ __forceinline__ bool sym_tri_body(const StepArgs& a, const SymStep& x
   TriCoef<V, NN> Y;
   if (act) {
     TriCoef<V, NN> U;
-    if constexpr (GRAD) {  // the forward field's derivatives wait in places that are filled later
+    if (GRAD && grad) {  // the forward field's derivatives wait in places that are filled later
       const float* fs = sm + L.f + sym_shift(x.ring_u + i0) + ln;
       tri_analyse<V, NN>(U, [&](int q) { return ld(fs + at(q) * SG); });
       sym_tri_orbits<V, NN, false, 0>(U, Y, [&](int q, int, V& r, V& t) {
@@ -580,7 +583,7 @@ __device__ __forceinline__ bool sym_tri_body(const StepArgs& a, const SymStep& x
       const V ht = fma2(dup<V>(H[v][1]), gr, mul2(dup<V>(H[v][2]), gt));
       r = mul2(wc, hr);
       t = mul2(wc, ht);
-      if constexpr (GRAD) {  // w (Ghat grad u_dag) . grad u
+      if (GRAD && grad) {  // w (Ghat grad u_dag) . grad u
         float* g = own(L.gs, L.gb, q);
         st(g, mul2(dup<V>(w), fma2(hr, ld(g), mul2(ht, ld(own(L.ys, L.yb, q))))));
       }

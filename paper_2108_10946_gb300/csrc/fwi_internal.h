@@ -138,7 +138,19 @@ struct KernelSet {
 };
 const KernelSet* kernel_set(int dim, int k);
 
+// The coefficients that follow from the velocity (fwi_set_velocity): inputs in FP64, outputs
+// rounded once. Null outputs are not formed.
+struct VelocityArgs {
+  int N, dim, nch;
+  double dt, water;
+  const double *c, *M, *Mb, *sigma;
+  const int *pidx, *sdesc;
+  float *c2, *cvel, *cf, *lcf, *lpsi, *lcs;
+  unsigned char *mask, *splain;
+};
+
 // Generic (dimension-only) kernels.
+void launch_velocity(const VelocityArgs& v);
 void launch_node_update(const StepArgs& a, int dim, cudaStream_t st);
 void launch_fold(float* gseg, double* gsum, double* gcomp, int64_t N, double scale,
                  cudaStream_t st);

@@ -45,6 +45,86 @@ void launch_node_update(const StepArgs& a, int dim, cudaStream_t st) {
     node_kernel<3><<<blocks, bs, 0, st>>>(a);
 }
 
+// Coefficients of every DoF at velocity c, in FP64 (the formulas of update.cuh's records): c^2, c, the
+// increment update's c1..c3, the gradient's mask and, in the layer, the auxiliaries' coefficients.
+template <int D>
+__global__ void __launch_bounds__(256) velocity_kernel(const VelocityArgs v) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= v.N) return;
+  const double c = v.c[i], M = v.M[i], dt = v.dt, cc = c * c;
+  double s[D], tr = 0;
+#pragma unroll
+  for (int k = 0; k < D; ++k) tr += s[k] = v.sigma[(size_t)i * D + k];
+  const double m3 = D == 2 ? s[0] * s[1] : s[0] * s[1] + s[0] * s[D - 1] + s[1] * s[D - 1];
+  const double det1 = s[0] * s[1] * s[D - 1];  // (3D)
+  const double a = tr + c * v.Mb[i] / M, den = 1.0 + 0.5 * a * dt;
+  v.c2[i] = (float)cc;
+  v.cvel[i] = (float)c;
+  v.cf[i] = (float)((1.0 - 0.5 * a * dt) / den);
+  v.cf[(size_t)v.N + i] = (float)(dt * dt / (M * den));
+  v.cf[2 * (size_t)v.N + i] = (float)(dt * dt * m3 / den);
+  v.mask[i] = !(tr > 0) && !(v.water > 0 && c < v.water) ? 1 : 0;
+  const int pi = v.pidx[i];
+  if (pi < 0) return;
+  typedef LayerCoef<D> L;
+  float q[L::COUNT];
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    const double psi2 = 2.0 * s[k] - tr, dk = 1.0 + 0.5 * dt * s[k];
+    q[L::E1 + k] = (float)((1.0 - 0.5 * dt * s[k]) / dk);
+    q[L::E2F + k] = (float)(dt * psi2 * cc / (M * dk));
+    q[L::E2A + k] = (float)(dt / (M * dk));
+    q[L::PSI2 + k] = (float)(psi2 * cc);
+    if constexpr (D == 3) {
+      const double psi3 = k == 0 ? s[1] * s[2] : k == 1 ? s[0] * s[2] : s[0] * s[1];
+      q[L::E3F + k] = (float)(dt * psi3 * cc / (M * dk));
+      q[L::PSI3 + k] = (float)(psi3 * cc);
+    }
+  }
+  if constexpr (D == 3) {
+    q[L::C4] = (float)(dt * dt * det1 / den);
+    q[L::C5] = (float)(dt * dt / den);
+    q[L::DTDET] = (float)(dt * det1);
+    q[L::DTM] = (float)(dt / M);
+  }
+  if (v.lcf)
+#pragma unroll
+    for (int k = 0; k < L::COUNT; ++k) v.lcf[(size_t)pi * L::COUNT + k] = q[k];
+  if (!v.lcs) return;
+  if constexpr (D == 2) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v.lcs[(size_t)pi * 8 + k] = q[k];
+    v.lpsi[pi] = q[L::PSI2];
+  } else {
+    const float o[12] = {q[0], q[1], q[2], q[L::C4], q[L::E2A], q[L::E2A + 1], q[L::E2A + 2], q[L::DTM],
+                         q[L::C5], q[L::DTDET], 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 12; ++k) v.lcs[(size_t)pi * 12 + k] = o[k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v.lpsi[(size_t)pi * 4 + k] = k < 3 ? (float)s[k] : 0.f;
+  }
+}
+
+// splain: 1 for a chunk whose owned DoFs are neither damped nor on an absorbing boundary (c1 = 1 and
+// c3 = 0: v' = v - c2 y); one warp per chunk.
+__global__ void __launch_bounds__(256) splain_kernel(const VelocityArgs v) {
+  const int c = (blockIdx.x * 256 + threadIdx.x) / 32, lane = threadIdx.x & 31;
+  if (c >= v.nch) return;
+  const int lo = v.sdesc[8 * c + 2], hi = c + 1 < v.nch ? v.sdesc[8 * (c + 1) + 2] : v.N;
+  // (the last chunk's range runs into the halo here: it is plain only if that is, too)
+  bool plain = true;
+  for (int i = lo + lane; i < hi && plain; i += 32) plain = v.cf[i] == 1.f && v.cf[2 * (size_t)v.N + i] == 0.f;
+  plain = __all_sync(0xffffffffu, plain);
+  if (lane == 0) v.splain[c] = plain ? 1 : 0;
+}
+
+void launch_velocity(const VelocityArgs& v) {
+  const unsigned blocks = (unsigned)((v.N + 255) / 256);
+  if (v.dim == 2) velocity_kernel<2><<<blocks, 256>>>(v);
+  else velocity_kernel<3><<<blocks, 256>>>(v);
+  if (v.nch > 0) splain_kernel<<<(unsigned)((v.nch + 7) / 8), 256>>>(v);
+}
+
 // Kahan fold of the FP32 segment sum into (sum, comp); comp carries the lost low part
 // with the sign convention sum - comp ~ exact.
 __global__ void fold_kernel(float* __restrict__ gseg, double* __restrict__ gsum,
