@@ -413,11 +413,11 @@ def parity_sample(pkg, pool, info, k, S, T_par, workload="marine2d", gstore=Fals
                       f", N={info['N']}, {T_par} s, layer, absorbing boundary, residual 0.03 d"}
 
 
-# DRAM bytes (read + write) of one forward time step: the three launches of a step
-# (k_chunk_pt<0>, k_chunk<0,1>, node_kernel4<2>) from one ncu capture of this workload's mesh
-# (profiles/ncu_forward_marine2d_kmv5_S4.md), keyed by (workload, k, S, N) so that it is
-# reported only for the mesh, degree and shot count it was measured on.
-FORWARD_TRAFFIC = {("marine2d", 5, 4, 7477937): 745.2e6}
+# DRAM bytes (read + write) of one forward time step from an ncu capture of its launches, keyed by
+# (workload, k, S, N) so that it is reported only for the mesh, degree and shot count it was
+# measured on (none for the present kernels on this mesh; profiles/chunk_kernels.md has a graded
+# mesh of its size).
+FORWARD_TRAFFIC = {}
 
 NODES = {2: (7, 6), 3: (12, 9), 4: (18, 12), 5: (30, 15)}  # KMVktri: nodes, shared nodes
 NODES3 = {2: (15, 14), 3: (32, 28)}                           # KMVktet
@@ -567,8 +567,7 @@ def run_ours(args):
     S = args.shots
     shots = wl["srcs"][shots_for_rank(len(wl["srcs"]), S, rank, world)]
     batch = pkg.Batch(mesh, shots, wl["recs"])
-    # the gradient steps read the forward field's gradients stored by the recompute
-    # (fwi_batch_set_gradient_store; no effect on tetrahedra)
+    # (fwi_batch_set_gradient_store: accepted, without effect)
     batch.set_gradient_store(not args.no_gradient_store)
     R = len(wl["recs"])
     wav = np.stack([signals.ricker_samples(wl["f"], dt, nt)] * S)

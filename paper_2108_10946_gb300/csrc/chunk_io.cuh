@@ -1,5 +1,4 @@
-// Global <-> shared-memory traffic of one chunk, shared by the CUDA-core and the tensor-core
-// chunk kernels.
+// Global <-> shared-memory traffic of one chunk of the tensor-core kernel (triangles).
 //
 // Phase 1 (chunk_load) issues every global read of the chunk at once as asynchronous copies
 // (cp.async, 4 bytes each) into the chunk table, in two completion groups: group 0 holds what

@@ -1,4 +1,4 @@
-// Tensor-core chunk time step (2D). The same chunked assembly as chunk_kernel.cuh (one
+// Tensor-core chunk time step (2D). A chunked assembly (one
 // chunk of PE consecutive elements for a group of SG shots, assembled in shared memory), with
 // the element stiffness action of the whole chunk done as two batched contractions on the
 // fifth-generation tensor cores. Row r = (element, shot) of the chunk (r < 128):

@@ -179,6 +179,10 @@ int run_t(const StepArgs& a, const RunArgs& r, cudaStream_t st) {
   b.ch0 = 0;
   void* args[] = {&b, &q};
   e = cudaLaunchCooperativeKernel((const void*)k_run<MODE>, dim3((unsigned)grid), dim3(NT), args, bytes, st);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {  // a part of the device only
+    cudaGetLastError();
+    return 0;
+  }
   return e == cudaSuccess ? grid : -(int)e;
 }
 int run(const StepArgs& a, const RunArgs& r, cudaStream_t st) { return a.mode == 0 ? run_t<0>(a, r, st) : run_t<2>(a, r, st); }

@@ -333,8 +333,7 @@ class Batch:
         _check(_lib.fwi_batch_set_gradient_lanes(self._h, int(bool(per_shot))))
 
     def set_gradient_store(self, on=True):
-        """Store the forward field's gradients during the recompute (faster gradient steps,
-        more device memory; see fwi_batch_set_gradient_store)."""
+        """Accepted, without effect (see fwi_batch_set_gradient_store)."""
         _check(_lib.fwi_batch_set_gradient_store(self._h, int(bool(on))))
 
     def gradient_lanes(self, out, stream=None):
