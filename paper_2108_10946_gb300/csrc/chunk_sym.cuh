@@ -99,10 +99,12 @@ __device__ __forceinline__ void sym_prefetch(const float* p, int n) {  // to L2
 
 constexpr int SYM_PE = sym_pe(D, NN);  // most elements of a chunk, stride of its tables
 
-// A CTA's threads: one element for LANES shots each.
-template <int SG>
+// A CTA's threads: one element for LANES shots each. In launches of several steps (RUN: few chunks,
+// latency counts) at least 128, those beyond the elements sharing the loads and the update.
+template <int SG, bool RUN>
 struct SymMap {
-  static constexpr int LANES = SYM_LANES < SG ? SYM_LANES : SG, PER = SG / LANES, NT = SYM_PE * PER;
+  static constexpr int LANES = SYM_LANES < SG ? SYM_LANES : SG, PER = SG / LANES, WORK = SYM_PE * PER;
+  static constexpr int NT = RUN && WORK < 128 ? 128 : WORK;
   typedef typename std::conditional<LANES == 2, float2, float>::type V;
 };
 
@@ -187,7 +189,7 @@ __device__ __forceinline__ void sym_cp_live(float* dst, const float* src) {
 template <int D, int NN, int NS, int SG, int MODE, bool LAYER, bool RUN>
 __device__ __forceinline__ void sym_load(const StepArgs& a, const SymStep& x, const SymDesc& cd, const SymSmem& L,
                                          float* sm, uint64_t* bar, int chunk, int s0, int tid) {
-  constexpr int NI = NN - NS, NT = SymMap<SG>::NT;
+  constexpr int NI = NN - NS, NT = SymMap<SG, RUN>::NT;
   constexpr bool GRAD = MODE == 2, OM = LAYER && D == 3 && MODE == 0;
   constexpr int PSI = LAYER ? sym_psi<D, MODE>() : 0;
   const int S = a.S, on = cd.nsh + cd.ne * NI;
@@ -320,10 +322,10 @@ struct SymRound {
 // Phase 3 of one chunk (after a barrier); cur: its first round's reads, issued before the barrier.
 // v' = c1 v - c2 y - c3 u, u' = u + v'. chk collects 0 * u', which stays zero while every value is
 // finite.
-template <int D, int NN, int NS, int MODE, bool LAYER, int SG, int B>
+template <int D, int NN, int NS, int MODE, bool LAYER, int SG, bool RUN, int B>
 __device__ __forceinline__ void sym_finish(const StepArgs& a, const SymStep& x, const SymDesc& cd, const SymSmem& L,
                                            const float* sm, int s0, int tid, SymRound<SG, B>& cur, float& chk) {
-  constexpr int PE = SYM_PE, NI = NN - NS, NT = SymMap<SG>::NT;
+  constexpr int PE = SYM_PE, NI = NN - NS, NT = SymMap<SG, RUN>::NT;
   constexpr bool GRAD = MODE == 2;
   const int S = a.S, nb = cd.ne * NI, on = cd.nsh + nb;
   const uint16_t* ge = reinterpret_cast<const uint16_t*>(sm + L.meta) + NS * PE;
@@ -436,10 +438,10 @@ __device__ __forceinline__ void sym_finish(const StepArgs& a, const SymStep& x, 
 // threads' places. All threads share the work: one takes a receiver's record of one shot, or a
 // node's sum over an element's receivers. (Done by the element's own thread, receiver by receiver,
 // this was the longest chain of a step wherever receivers crowd: 4 us with three in an element.)
-template <int D, int NN, int NS, int MODE, int SG>
+template <int D, int NN, int NS, int MODE, int SG, bool RUN>
 __device__ __forceinline__ void sym_inject(const StepArgs& a, const SymStep& x, const SymDesc& cd, const SymSmem& L,
                                            float* sm, int s0, int tid, int b, int e) {
-  constexpr int PE = SYM_PE, NI = NN - NS, NT = SymMap<SG>::NT;
+  constexpr int PE = SYM_PE, NI = NN - NS, NT = SymMap<SG, RUN>::NT;
   const uint16_t* lq = reinterpret_cast<const uint16_t*>(sm + L.meta);
   const float* us = sm + L.u + sym_shift(x.u + (size_t)cd.own * a.S + s0);
   auto place = [&](int q, int el) {
@@ -512,7 +514,7 @@ __device__ __forceinline__ void sym_tri_orbits(const TriCoef<V, NN>& U, TriCoef<
 // One step of a triangle chunk. MODE: 0 forward, 1 adjoint, 2 adjoint with the gradient integrand.
 template <int NN, int NS, int MODE, bool LAYER, int SG, bool RUN>
 __device__ __forceinline__ bool sym_tri_body(const StepArgs& a, const SymStep& x, float* sm, int chunk, int s0) {
-  using M = SymMap<SG>;
+  using M = SymMap<SG, RUN>;
   using V = typename M::V;
   constexpr int NI = NN - NS, PE = SYM_PE;
   constexpr bool ADJ = MODE != 0, GRAD = MODE == 2;
@@ -635,12 +637,12 @@ __device__ __forceinline__ bool sym_tri_body(const StepArgs& a, const SymStep& x
   first.load(a, cd, cd.nsh + nb, s0, tid, M::NT);
   __syncthreads();
   if (in0 < in1) {
-    sym_inject<2, NN, NS, MODE, SG>(a, x, cd, L, sm, s0, tid, in0, in1);
+    sym_inject<2, NN, NS, MODE, SG, RUN>(a, x, cd, L, sm, s0, tid, in0, in1);
     __syncthreads();
   }
 
   float chk = 0.f;
-  sym_finish<2, NN, NS, MODE, LAYER, SG, B>(a, x, cd, L, sm, s0, tid, first, chk);
+  sym_finish<2, NN, NS, MODE, LAYER, SG, RUN, B>(a, x, cd, L, sm, s0, tid, first, chk);
   if (!(chk == 0.f)) atomicOr(a.status, 1);
   return true;
 }
@@ -742,7 +744,7 @@ __device__ __forceinline__ void sym_tet_roll(const TetCoef<V, 32>* const (&U)[N]
 // steps in the layer).
 template <int NN, int NS, int MODE, bool LAYER, int SG, bool RUN>
 __device__ __forceinline__ bool sym_tet_body(const StepArgs& a, const SymStep& x, float* sm, int chunk, int s0) {
-  using M = SymMap<SG>;
+  using M = SymMap<SG, RUN>;
   using V = typename M::V;
   constexpr int NI = NN - NS, PE = SYM_PE;
   constexpr bool ADJ = MODE != 0, GRAD = MODE == 2, OM = LAYER && !ADJ, W = LAYER && ADJ;
@@ -878,12 +880,12 @@ __device__ __forceinline__ bool sym_tet_body(const StepArgs& a, const SymStep& x
   first.load(a, cd, cd.nsh + nb, s0, tid, M::NT);
   __syncthreads();
   if (in0 < in1) {
-    sym_inject<3, NN, NS, MODE, SG>(a, x, cd, L, sm, s0, tid, in0, in1);
+    sym_inject<3, NN, NS, MODE, SG, RUN>(a, x, cd, L, sm, s0, tid, in0, in1);
     __syncthreads();
   }
 
   float chk = 0.f;
-  sym_finish<3, NN, NS, MODE, LAYER, SG, B>(a, x, cd, L, sm, s0, tid, first, chk);
+  sym_finish<3, NN, NS, MODE, LAYER, SG, RUN, B>(a, x, cd, L, sm, s0, tid, first, chk);
   if (!(chk == 0.f)) atomicOr(a.status, 1);
   return true;
 }

@@ -31,16 +31,17 @@ __constant__ float c_w[NN];
 
 namespace fwi {
 namespace {
-constexpr int NT = SymMap<SG>::NT;
+constexpr int NT = SymMap<SG, false>::NT, NT_RUN = SymMap<SG, true>::NT;
 // Registers a thread may take: enough CTAs per SM to hide the loads of one behind the arithmetic of
 // the others. KMV5 gradient steps hold more at a time and lose less to a fourth CTA less than to
 // spills (marine mesh, one gradient of 75 steps: 128.5 ms at 168, 133.1 ms at 128); every other
 // kernel is best at 128 (KMV4, S = 4, 250k triangles: 8.0 ms for 100 steps, 10.9 ms at 204; KMV3,
 // 120k: 8.9 and 9.8 ms), but KMV2's at one shot, which do little with what they load (2M triangles,
 // 50 steps: 3.54 ms at 48, 3.71 ms at 80).
-#ifndef RUN_MAX
-#define RUN_MAX 304  // most CTAs of a launch of several steps
-#endif
+// Most CTAs of a launch of several steps. 256 of them (KMV2, 8,192 triangles, one shot, 400 steps): 3.97
+// ms against 4.21 ms in launches per step; 1,560 (KMV5, 50k, one shot, a gradient of 75 steps): 15.4
+// against 6.3 ms, their meetings crowd one counter.
+constexpr int RUN_MAX = 304;
 
 template <int MODE, bool LAYER>
 constexpr int registers() {
@@ -105,7 +106,7 @@ __device__ __noinline__ bool run_chunk(const StepArgs& a, const SymStep& x, floa
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(NT, 65536 / (registers<MODE, true>() * NT))
+__global__ void __launch_bounds__(NT_RUN, 65536 / (registers<MODE, true>() * NT_RUN))
     k_run(const __grid_constant__ StepArgs a, const RunArgs r) {
   extern __shared__ __align__(16) float smem_sym[];
   const int ngrp = a.S / SG, nwork = a.nch * ngrp, tid = threadIdx.x;
@@ -137,7 +138,7 @@ __global__ void __launch_bounds__(NT, 65536 / (registers<MODE, true>() * NT))
       return;
     }
     const int64_t items = (int64_t)a.hcnt * ngrp;
-    for (int64_t t = (int64_t)blockIdx.x * NT + tid; t < items; t += (int64_t)gridDim.x * NT) {
+    for (int64_t t = (int64_t)blockIdx.x * NT_RUN + tid; t < items; t += (int64_t)gridDim.x * NT_RUN) {
       const int dof = a.h0 + (int)(t / ngrp);
       halo_dof<D, SG, MODE == 0 ? 0 : 1>(a, x.u, x.u_out, dof, (int)(t % ngrp) * SG, dof >= a.halo_layer);
     }
@@ -168,7 +169,7 @@ int run_t(const StepArgs& a, const RunArgs& r, cudaStream_t st) {
     if (e != cudaSuccess) return -(int)e;
     configured[dev] = bytes;
   }
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_run<MODE>, NT, bytes);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_run<MODE>, NT_RUN, bytes);
   if (e != cudaSuccess) return -(int)e;
   const int64_t nwork = (int64_t)a.nch * (a.S / SG);
   const int64_t room = (int64_t)per * nsm[dev];
@@ -178,7 +179,7 @@ int run_t(const StepArgs& a, const RunArgs& r, cudaStream_t st) {
   RunArgs q = r;
   b.ch0 = 0;
   void* args[] = {&b, &q};
-  e = cudaLaunchCooperativeKernel((const void*)k_run<MODE>, dim3((unsigned)grid), dim3(NT), args, bytes, st);
+  e = cudaLaunchCooperativeKernel((const void*)k_run<MODE>, dim3((unsigned)grid), dim3(NT_RUN), args, bytes, st);
   if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {  // a part of the device only
     cudaGetLastError();
     return 0;
