@@ -1,6 +1,7 @@
 // The symmetry-adapted chunk kernels of one KMV element and one group of shots per CTA,
 // instantiated once per (dimension, degree, shots): -DKMV_DIM=d -DKMV_K=k -DKMV_SG=1|2|4.
 #include <algorithm>
+#include <mutex>
 
 #include "fwi_internal.h"
 
@@ -149,6 +150,8 @@ __global__ void __launch_bounds__(NT_RUN, 65536 / (registers<MODE, true>() * NT_
   }
 }
 
+std::mutex g_limits;  // the kernels' shared-memory limits are raised by one thread at a time
+
 // Returns the CTAs of the launch, 0 if the steps are better launched one by one (nothing done), or
 // minus a cudaError_t.
 template <int MODE>
@@ -163,12 +166,14 @@ int run_t(const StepArgs& a, const RunArgs& r, cudaStream_t st) {
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64) return 0;
   cudaError_t e = cudaSuccess;
+  std::unique_lock<std::mutex> lk(g_limits);
   if (bytes > configured[dev]) {
     e = cudaFuncSetAttribute(k_run<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return -(int)e;
     configured[dev] = bytes;
   }
+  lk.unlock();
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_run<MODE>, NT_RUN, bytes);
   if (e != cudaSuccess) return -(int)e;
   const int64_t nwork = (int64_t)a.nch * (a.S / SG);
@@ -198,6 +203,7 @@ int launch_t(void (*kernel)(const StepArgs), int which, size_t bytes, const Step
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64) return (int)cudaErrorInvalidDevice;
+  std::unique_lock<std::mutex> lk(g_limits);
   if (bytes > configured[which][dev]) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     int per = 0, nsm = 0;
@@ -207,6 +213,7 @@ int launch_t(void (*kernel)(const StepArgs), int which, size_t bytes, const Step
     wave[which][dev] = per * nsm;
     configured[which][dev] = bytes;
   }
+  lk.unlock();
   StepArgs b = a;
   b.ch0 = ch0;
   b.wave = down ? -wave[which][dev] : wave[which][dev];
