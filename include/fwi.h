@@ -112,7 +112,8 @@ int fwi_mesh_upload(const double* verts, int64_t nverts, const int32_t* cells, i
 
 /* Host-only preparation of the same mesh (numbering, geometry, lumped and boundary mass,
  * damping profile) without touching a GPU: for inspection and tests. The handle supports
- * fwi_num_dofs, fwi_dof_coords, fwi_element, fwi_mesh_host_arrays and fwi_mesh_free. */
+ * fwi_num_dofs, fwi_dof_coords, fwi_element, fwi_mesh_host_arrays, fwi_mesh_chunk_tables and
+ * fwi_mesh_free. */
 int fwi_mesh_prepare_host(const double* verts, int64_t nverts, const int32_t* cells,
                           int64_t ncells, const fwi_params* params, fwi_mesh** out);
 
@@ -120,6 +121,15 @@ int fwi_mesh_prepare_host(const double* verts, int64_t nverts, const int32_t* ce
  * lumped mass[N], lumped boundary mass[N], sigma[N][dim]. Any pointer may be NULL. */
 int fwi_mesh_host_arrays(const fwi_mesh* m, int32_t* conn, double* mass, double* bmass,
                          double* sigma);
+
+/* The chunked layout's tables as the kernels read them (host; for inspection and tests; FWI_EINVAL
+ * for the plain layout). sizes[4]: chunks, the first chunk with damping-layer elements, the
+ * elements a table has room for (stride PE), 16-bit entries of all tables. desc[chunks][8] per
+ * chunk: first element, its elements (low 16 bits), first owned DoF, owned shared DoFs, start and
+ * length of its halo list, start and size of its table in pairs of entries. A table starts with
+ * the place [NS][PE] of every shared node of every element among the chunk's DoFs: owned ones,
+ * from 0 on, then those of the halo list. desc and tables may be NULL. */
+int fwi_mesh_chunk_tables(const fwi_mesh* m, int64_t* sizes, int32_t* desc, uint16_t* tables);
 
 /* Number of global DoFs N (vertex, edge, face and interior KMV nodes). */
 int fwi_num_dofs(const fwi_mesh* m, int64_t* n);

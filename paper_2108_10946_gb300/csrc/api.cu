@@ -555,7 +555,8 @@ void build_incidence(fwi_mesh* m) {
     cnt.assign(nloc + 1, 0);
     for (int q = 0; q < ns; ++q)
       for (int e = e0; e < e0 + ne; ++e) {
-        lq[q * P + e - e0] = m->lconn[(size_t)node(q) * m->Es + e];
+        const int l = m->lconn[(size_t)node(q) * m->Es + e];
+        lq[q * P + e - e0] = (uint16_t)(l < own_n ? l : l + fwi::SYM_GAP);
         cnt[place(q, e) + 1]++;
       }
     for (int l = 0; l < nloc; ++l) cnt[l + 1] += cnt[l];
@@ -565,7 +566,7 @@ void build_incidence(fwi_mesh* m) {
     // (the second entry's bit 16, any undamped DoF, follows once the damping profile is known)
     const int d[8] = {e0, ne, own, nsh, hp, hn, (int)(at / 2), (int)(size / 2)};
     std::copy(d, d + 8, &m->sdesc[(size_t)c * 8]);
-    m->T_max = std::max(m->T_max, own_n + hn);
+    m->T_max = std::max(m->T_max, own_n + fwi::SYM_GAP + hn);
     m->SH_max = std::max(m->SH_max, nloc);
   }
 }
@@ -1032,6 +1033,18 @@ int fwi_mesh_host_arrays(const fwi_mesh* m, int32_t* conn, double* mass, double*
   if (mass) std::memcpy(mass, m->M.data(), m->M.size() * sizeof(double));
   if (bmass) std::memcpy(bmass, m->Mb.data(), m->Mb.size() * sizeof(double));
   if (sigma) std::memcpy(sigma, m->sigma.data(), m->sigma.size() * sizeof(double));
+  return 0;
+}
+
+int fwi_mesh_chunk_tables(const fwi_mesh* m, int64_t* sizes, int32_t* desc, uint16_t* tables) {
+  if (!m || !sizes) return fail(FWI_EINVAL, "null argument");
+  if (m->layout != 0) return fail(FWI_EINVAL, "the plain layout has no chunks");
+  sizes[0] = m->nch();
+  sizes[1] = m->nch0;
+  sizes[2] = fwi::sym_pe(m->dim, m->nn);
+  sizes[3] = (int64_t)m->smeta.size();
+  if (desc) std::memcpy(desc, m->sdesc.data(), m->sdesc.size() * sizeof(int32_t));
+  if (tables) std::memcpy(tables, m->smeta.data(), m->smeta.size() * sizeof(uint16_t));
   return 0;
 }
 

@@ -77,8 +77,9 @@ __device__ __forceinline__ void sym_bulk(void* dst, const void* src, uint32_t by
 }
 
 // A contiguous run of floats as a bulk copy: from the 16-byte boundary at or below its start, so
-// it lands `shift` floats past the place it is copied to; whole 16-byte groups (arrays that are
-// copied this way are allocated with four floats to spare).
+// it lands `shift` floats past the place it is copied to; whole 16-byte groups, so up to three floats
+// past the run come along: arrays that are copied this way are allocated with four floats to spare,
+// and in the tables nothing else is written behind a run (SYM_GAP).
 struct SymRun {
   const float* src;
   int shift;
@@ -118,8 +119,8 @@ struct SymStep {
   uint32_t parity;
 };
 
-// Dynamic shared memory of one chunk (offsets in floats). T: largest chunk table, SH: most shared
-// DoFs (owned and halo), H: longest halo list of a chunk.
+// Dynamic shared memory of one chunk (offsets in floats). T: largest chunk table (with the gap), SH:
+// most shared DoFs (owned and halo), H: longest halo list of a chunk.
 struct SymSmem {
   int u, f, c2, ps, om, ys, yb, p1, gs, gb, ws, wb, ss, sb, ids, meta, total;
 };
@@ -145,7 +146,7 @@ __host__ __device__ inline SymSmem sym_smem(int T, int SH, int H) {
   constexpr bool APART = GRAD && D == 2;
   constexpr int SUMS = (NE + NB) * (L3 && MODE != 0 ? 2 : 1);  // y, and the omega row's (3D adjoint)
   m.ys = o, m.yb = o + NE, m.ws = o + NE + NB, m.wb = m.ws + NE, m.p1 = o + (APART ? SUMS : 0);
-  o += !LAYER ? SUMS : APART ? SUMS + up(D * SH * SG) : most(SUMS, up(D * SH * SG));
+  o += !LAYER ? SUMS : APART ? SUMS + up(D * (SH + SYM_GAP) * SG) : most(SUMS, up(D * (SH + SYM_GAP) * SG));
   m.gs = o, o += GRAD ? NE : 0;
   m.gb = o, o += GRAD ? NB : 0;
   // 3D: the second field (the forward field; omega in forward steps) lies where the layer sums go
@@ -177,8 +178,9 @@ __device__ __forceinline__ SymDesc sym_desc(const StepArgs& a, int c) {
   return d;
 }
 
-// Phase 1 of one chunk. The table: owned shared DoFs [0, nsh), bubbles, halo DoFs. The runs' shifts
-// follow from their addresses (sym_shift).
+// Phase 1 of one chunk. The table: owned shared DoFs [0, nsh), bubbles, SYM_GAP places, halo DoFs (P of
+// the shared DoFs: owned, SYM_GAP places, halo). The runs' shifts follow from their addresses
+// (sym_shift).
 // RUN (several steps in one launch): what other CTAs wrote in an earlier step comes from L2 (copies
 // of four and eight bytes would go through L1).
 template <int BYTES, bool RUN>
@@ -276,7 +278,7 @@ __device__ __forceinline__ void sym_load(const StepArgs& a, const SymStep& x, co
     }
   }
   for (int h = tid; h < cd.hn; h += NT) {
-    const int id = __ldg(a.halo + cd.hp + h), l = on + h;
+    const int id = __ldg(a.halo + cd.hp + h), l = on + SYM_GAP + h;
     reinterpret_cast<int*>(sm + L.ids)[h] = id;
     sym_cp_live<4 * SG, RUN>(us + l * SG, x.u + (size_t)id * S + s0);
     if (GRAD && (D == 3 || cd.keep)) sym_cp<4 * SG>(fs + l * SG, x.ring_u + (size_t)id * S + s0);
@@ -284,7 +286,7 @@ __device__ __forceinline__ void sym_load(const StepArgs& a, const SymStep& x, co
     if (LAYER) {
       const size_t pi = (size_t)(id - a.p_halo);
 #pragma unroll
-      for (int k = 0; k < D; ++k) sym_cp_live<4 * SG, RUN>(p1 + ((cd.nsh + h) * D + k) * SG, a.P + (pi * D + k) * S + s0);
+      for (int k = 0; k < D; ++k) sym_cp_live<4 * SG, RUN>(p1 + ((cd.nsh + SYM_GAP + h) * D + k) * SG, a.P + (pi * D + k) * S + s0);
       if (PSI) sym_cp<4 * (PSI ? PSI : 1)>(ps + l * PSI, a.lpsi + pi * PSI);
       if (OM) sym_cp_live<4 * SG, RUN>(om + l * SG, a.Y + pi * S + s0);
     }
@@ -830,7 +832,7 @@ __device__ __forceinline__ bool sym_tet_body(const StepArgs& a, const SymStep& x
       V f[3] = {mul2(wc, h0), mul2(wc, h1), mul2(wc, h2)};
       if constexpr (LAYER) {
         const int on = cd.nsh + nb;
-        const float4 sg = __ldg(sig + (l < on ? (int)pi0 + l : ids[l - on] - a.p_halo));
+        const float4 sg = __ldg(sig + (l < on ? (int)pi0 + l : ids[l - on - SYM_GAP] - a.p_halo));
         const float s1 = sg.x, s2 = sg.y, s3 = sg.z, tr = s1 + s2 + s3;
         const float psi2[3] = {c2 * (2.f * s1 - tr), c2 * (2.f * s2 - tr), c2 * (2.f * s3 - tr)};
         const float psi3[3] = {c2 * s2 * s3, c2 * s1 * s3, c2 * s1 * s2};

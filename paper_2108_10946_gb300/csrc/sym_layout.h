@@ -168,6 +168,11 @@ FWI_HD constexpr int tet_at(int o, int d, int z, int y, int i) {
          TetSym<NN>::turn_mode(i, y, d);
 }
 
+// Places between a chunk's owned DoFs and its halo DoFs in every table of the chunk kernels. The owned
+// range arrives in whole 16-byte groups, whose last may end up to three floats past it; the halo DoFs
+// are copied by other threads meanwhile, in no order to that, so they start where no group ends.
+constexpr int SYM_GAP = 3;
+
 // Order of an element's nodes in the chunk tables (local node at slot j): the local order, but a
 // triangle's vertices backwards, like its other T orbits; at KMV3 tetrahedra orbit by orbit (slot
 // 4 o + h; the interior orbit last). So a loop over like orbits need not be unrolled.

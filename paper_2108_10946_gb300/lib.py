@@ -57,6 +57,7 @@ def load():
         "fwi_num_dofs": (ctypes.c_int, [_P, ctypes.POINTER(_I64)]),
         "fwi_dof_coords": (ctypes.c_int, [_P, _P]),
         "fwi_element": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int), _P, _P, _P]),
+        "fwi_mesh_chunk_tables": (ctypes.c_int, [_P, _P, _P, _P]),
         "fwi_set_velocity": (ctypes.c_int, [_P, _P]),
         "fwi_locate": (ctypes.c_int, [_P, _P, ctypes.c_int, _P, _P]),
         "fwi_reference_element": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_int),
@@ -228,6 +229,16 @@ class Mesh:
         sig = np.zeros((self.N, self.dim))
         _check(_lib.fwi_mesh_host_arrays(self._h, _ptr(conn), _ptr(M), _ptr(Mb), _ptr(sig)))
         return conn, M, Mb, sig
+
+    def chunk_tables(self):
+        """(first layer chunk, PE, desc [chunks][8], tables) of the chunked layout; see
+        fwi_mesh_chunk_tables."""
+        n = np.zeros(4, dtype=np.int64)
+        _check(_lib.fwi_mesh_chunk_tables(self._h, _ptr(n), None, None))
+        desc = np.zeros((int(n[0]), 8), dtype=np.int32)
+        tab = np.zeros(int(n[3]), dtype=np.uint16)
+        _check(_lib.fwi_mesh_chunk_tables(self._h, _ptr(n), _ptr(desc), _ptr(tab)))
+        return int(n[1]), int(n[2]), desc, tab
 
     def locate(self, pts):
         """(element index in the library's order [npts], reference coordinates [npts][dim])
