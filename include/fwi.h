@@ -301,12 +301,14 @@ int fwi_profile_read(fwi_batch* b, double* ms, int64_t* steps);
  * device), misfit_out may be NULL. Clears the accumulators. */
 int fwi_gradient_raw(fwi_batch* b, double* dJdc_out, double* misfit_out, void* stream);
 
-/* Testing aid (no counterpart in the paper): the number of polls each bounded mbarrier wait
- * of the tensor-core kernel makes before it gives up (default 2^22; < 0 restores it; 0 gives
- * up at once). A wait that gives up stops its kernel early, waits (with the default limit)
- * for its MMAs in flight, frees its tensor memory and sets a status bit; the call then
- * returns FWI_ETIMEDOUT and the context stays usable. The batch's results of that call are
- * meaningless. */
+/* Testing aid (no counterpart in the paper): the number of polls each bounded wait inside a
+ * kernel makes before it gives up (default 2^22; < 0 restores it; 0 gives up at once): the chunk
+ * kernels' waits for their copies, the meetings of a launch of several steps, the tensor-core
+ * kernel's waits for its MMAs. A wait that gives up stops its kernel early, waits (with the
+ * default limit) for its copies or MMAs in flight, frees its tensor memory and sets a status bit;
+ * the call then returns FWI_ETIMEDOUT and the context stays usable. The batch's results of that
+ * call, its forward state and what its gradient accumulators hold are meaningless: clear the
+ * accumulators with fwi_gradient* and start from a new forward solve. */
 int fwi_batch_set_wait_limit(fwi_batch* b, int polls);
 
 int fwi_batch_free(fwi_batch* b);

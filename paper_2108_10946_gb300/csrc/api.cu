@@ -210,7 +210,7 @@ struct fwi_batch {
   double* stage_grad = nullptr;
   bool forward_done = false;
   int launch_error = 0;  // first kernel configuration error of a call (cudaError_t)
-  int tc_wait_limit = 1 << 22;  // polls of each bounded wait of the tensor-core kernel
+  int wait_limit = fwi::WAIT_POLLS;  // polls of each bounded wait of the chunk kernels
   int grad_lanes = 0;           // 1: the next adjoint keeps each shot's gradient apart
   int acc_lanes = -1;           // what the accumulators hold: -1 nothing, 0 summed, 1 per shot
   // optional per-kernel timing with CUDA events (fwi_profile)
@@ -1351,7 +1351,7 @@ StepArgs base_args(fwi_batch* b) {
   a.gseg = b->gseg;
   a.grad_lanes = b->grad_lanes;
   a.status = b->status;
-  a.tc_wait_limit = b->tc_wait_limit;
+  a.wait_limit = b->wait_limit;
   return a;
 }
 
@@ -1491,8 +1491,20 @@ int check_status(fwi_batch* b, cudaStream_t st) {
   CUDA_TRY(cudaGetLastError());
   if (b->prof) collect_profile(b);
   if (h) {
-    cudaMemsetAsync(b->status, 0, 64 * sizeof(int), st);
+    CUDA_TRY(cudaMemsetAsync(b->status, 0, 64 * sizeof(int), st));
     b->meet = 0;
+    if (h & 2) {
+      // a launch of several steps may have stopped before the halo DoFs took (and cleared) their sums
+      const fwi_mesh* m = b->m;
+      const size_t NS_ = (size_t)m->N * b->S * sizeof(float), YS = (size_t)m->Nl * b->S * sizeof(float);
+      CUDA_TRY(cudaMemsetAsync(b->r, 0, NS_, st));
+      CUDA_TRY(cudaMemsetAsync(b->gseg, 0, NS_, st));
+      if (YS) {
+        CUDA_TRY(cudaMemsetAsync(b->Pacc, 0, YS * m->dim, st));
+        CUDA_TRY(cudaMemsetAsync(b->Yacc, 0, YS, st));
+      }
+    }
+    CUDA_TRY(cudaStreamSynchronize(st));  // the next call may come on another stream
     if (h & 2) return fail(FWI_ETIMEDOUT, "a bounded wait inside a kernel gave up (the kernel returned early)");
     return fail(FWI_ERANGE, "non-finite value in the wavefield (time step above the stability limit?)");
   }
@@ -1947,7 +1959,7 @@ int fwi_batch_set_gradient_lanes(fwi_batch* b, int per_shot) {
 
 int fwi_batch_set_wait_limit(fwi_batch* b, int polls) {
   if (!b) return fail(FWI_EINVAL, "null batch");
-  b->tc_wait_limit = polls < 0 ? (1 << 22) : polls;
+  b->wait_limit = polls < 0 ? fwi::WAIT_POLLS : polls;
   return 0;
 }
 

@@ -55,10 +55,10 @@ __device__ __forceinline__ void sym_bar_init(uint64_t* bar) {
 __device__ __forceinline__ void sym_bar_expect(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
 }
-// Waits for a phase of the barrier; false if it gave up (bounded: 2^22 polls, each of which the
-// hardware may suspend for a while).
-__device__ __forceinline__ bool sym_bar_wait(uint64_t* bar, uint32_t parity) {
-  for (int i = 0; i < (1 << 22); ++i) {
+// Waits for a phase of the barrier; false if it gave up (after `polls`, each of which the hardware may
+// suspend for a while).
+__device__ __forceinline__ bool sym_bar_wait(uint64_t* bar, uint32_t parity, int polls) {
+  for (int i = 0; i < polls; ++i) {
     uint32_t done;
     asm volatile(
         "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
@@ -544,9 +544,9 @@ __device__ __forceinline__ bool sym_tri_body(const StepArgs& a, const SymStep& x
 #pragma unroll
     for (int c = 0; c < 4; ++c) A0[c >> 1][c & 1] = __ldg(a.lgeo + (size_t)c * (a.E - a.E0) + (e - a.E0));
   sym_cp_wait();
-  const bool ok = sym_bar_wait(bar, x.parity);
+  const bool ok = sym_bar_wait(bar, x.parity, a.wait_limit);
   if (__syncthreads_or(!ok)) {  // a copy did not arrive: report it and leave the fields alone
-    sym_bar_wait(bar, x.parity);
+    sym_bar_wait(bar, x.parity, WAIT_POLLS);  // (no CTA ends before its copies)
     if (tid == 0) atomicOr(a.status, 2);
     return false;
   }
@@ -772,9 +772,9 @@ __device__ __forceinline__ bool sym_tet_body(const StepArgs& a, const SymStep& x
 #pragma unroll
     for (int c = 0; c < 9; ++c) A[c / 3][c % 3] = __ldg(a.lgeo + (size_t)c * (a.E - a.E0) + (e - a.E0));
   sym_cp_wait();
-  const bool ok = sym_bar_wait(bar, x.parity);
+  const bool ok = sym_bar_wait(bar, x.parity, a.wait_limit);
   if (__syncthreads_or(!ok)) {  // a copy did not arrive: report it and leave the fields alone
-    sym_bar_wait(bar, x.parity);
+    sym_bar_wait(bar, x.parity, WAIT_POLLS);  // (no CTA ends before its copies)
     if (tid == 0) atomicOr(a.status, 2);
     return false;
   }

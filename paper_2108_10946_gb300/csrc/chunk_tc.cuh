@@ -240,7 +240,7 @@ __device__ __forceinline__ void chunk_tc_body(const StepArgs& a, float* smem, co
       tc::mma_commit(&bar);
     }
     {
-      const bool ok = tc::mbar_wait(&bar, parity, a.tc_wait_limit);
+      const bool ok = tc::mbar_wait(&bar, parity, a.wait_limit);
       if (__syncthreads_or(!ok)) {
         failed = true;
         break;
@@ -327,7 +327,7 @@ __device__ __forceinline__ void chunk_tc_body(const StepArgs& a, float* smem, co
       tc::mma_commit(&bar);
     }
     {
-      const bool ok = tc::mbar_wait(&bar, parity, a.tc_wait_limit);
+      const bool ok = tc::mbar_wait(&bar, parity, a.wait_limit);
       if (__syncthreads_or(!ok)) {
         failed = true;
         break;

@@ -9,6 +9,9 @@ namespace fwi {
 // many DoFs per chunk for every degree.
 constexpr int sym_pe(int dim, int nn) { return dim == 2 ? (nn == 7 ? 128 : nn == 12 ? 64 : nn == 18 ? 64 : 32) : nn == 15 ? 64 : 32; }
 
+// Polls after which a wait inside a kernel gives up (seconds).
+constexpr int WAIT_POLLS = 1 << 22;
+
 // Element-kernel arguments (one step of the forward, recompute or adjoint recurrence).
 // Layouts (S = shots of the batch, stored shot-interleaved so that the lanes of one
 // element read one contiguous run of S floats):
@@ -49,7 +52,7 @@ struct StepArgs {
   int T_max, SH_max;   // largest chunk table and most shared DoFs of a chunk
   int p_own, p_halo;   // layer index of an owned / halo DoF of a layer chunk: dof - shift
   int tc;              // chunked layout, 2D: element contraction on the tensor cores
-  int tc_wait_limit;   // polls of each bounded mbarrier wait of the tensor-core kernel
+  int wait_limit;      // polls of each bounded wait of the chunk kernels
   int mode;            // 0 forward, 1 adjoint (with gradient when ring != null)
   int n;               // time index (forward: step n -> n+1; adjoint: step m)
   int nt;

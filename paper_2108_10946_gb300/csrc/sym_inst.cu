@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(NT, 65536 / (registers<MODE, true>() * NT)) k_
 // every CTA takes its chunks, all CTAs meet, every thread finishes its halo DoFs, all meet again.
 // A chunk and a halo DoF stay with their CTA, so only what crosses CTAs has to come from L2. Both
 // kinds of chunks are one kernel here.
-__device__ __forceinline__ bool run_meet(unsigned* count, unsigned target) {
+__device__ __forceinline__ bool run_meet(unsigned* count, unsigned target, int polls) {
   asm volatile("fence.proxy.async;" ::: "memory");  // (the fields are written as usual, read by bulk copies)
   __syncthreads();
   bool ok = true;
@@ -86,7 +86,7 @@ __device__ __forceinline__ bool run_meet(unsigned* count, unsigned target) {
     __threadfence();
     atomicAdd(count, 1u);
     ok = false;
-    for (int i = 0; i < (1 << 22); ++i) {  // bounded: a CTA that gave up never arrives
+    for (int i = 0; i < polls; ++i) {  // bounded: a CTA that gave up never arrives
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
       if ((int)(v - target) >= 0) {
@@ -112,7 +112,8 @@ __global__ void __launch_bounds__(NT_RUN, 65536 / (registers<MODE, true>() * NT_
   extern __shared__ __align__(16) float smem_sym[];
   const int ngrp = a.S / SG, nwork = a.nch * ngrp, tid = threadIdx.x;
   if (tid == 0) sym_bar_init(reinterpret_cast<uint64_t*>(smem_sym));
-  __syncthreads();
+  // (an earlier launch of the call gave up: its CTAs never met, this one's would poll to the limit)
+  if (__syncthreads_or(tid == 0 && (__ldcg(a.status) & 2))) return;
   unsigned target = r.base;
   SymStep x{nullptr, nullptr, nullptr, 0, 0};
   for (int k = 0; k < r.steps; ++k) {
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(NT_RUN, 65536 / (registers<MODE, true>() * NT_
       asm volatile("fence.proxy.async;" ::: "memory");  // the next chunk's copies come after these reads
       __syncthreads();
     }
-    if (!run_meet(r.count, target += gridDim.x)) {
+    if (!run_meet(r.count, target += gridDim.x, a.wait_limit)) {
       if (tid == 0) atomicOr(a.status, 2);
       return;
     }
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(NT_RUN, 65536 / (registers<MODE, true>() * NT_
       const int dof = a.h0 + (int)(t / ngrp);
       halo_dof<D, SG, MODE == 0 ? 0 : 1>(a, x.u, x.u_out, dof, (int)(t % ngrp) * SG, dof >= a.halo_layer);
     }
-    if (!run_meet(r.count, target += gridDim.x)) {
+    if (!run_meet(r.count, target += gridDim.x, a.wait_limit)) {
       if (tid == 0) atomicOr(a.status, 2);
       return;
     }
