@@ -1126,6 +1126,14 @@ int fwi_set_velocity(fwi_mesh* m, const double* c) {
   const size_t Nl = (size_t)m->Nl;
   const bool lcf = m->layout == 1 || m->use_tc;  // the layer records of the plain and tensor-core steps
   int rc = 0;
+  auto have = [&](auto** p, const auto& v) {  // a host-only mesh has uploaded none of its arrays
+    if (!rc && !*p) rc = upload(p, v);
+  };
+  have(&m->d_M, m->M);
+  have(&m->d_Mb, m->Mb);
+  have(&m->d_sigma, m->sigma);
+  have(&m->d_pidx, m->pidx);
+  if (m->layout == 0) have(&m->d_sdesc, m->sdesc);
   auto room = [&](auto** p, size_t count) {  // allocated by the first call
     if (!rc && !*p) rc = dalloc(p, count);
   };
