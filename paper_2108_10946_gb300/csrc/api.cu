@@ -1207,6 +1207,7 @@ int fwi_batch_create(fwi_mesh* m, int nshots, const double* src, int nrec, const
     return fail(FWI_EINVAL, "fwi_batch_create: nshots must be a power of two <= 32, points non-null");
   if (!m->have_velocity) return fail(FWI_EINVAL, "call fwi_set_velocity before creating a batch");
   if (int rc = check_device(m)) return rc;
+  if (!m->d_geo) return fail(FWI_EINVAL, "a mesh prepared on the host only has no geometry on the device");
   *out = nullptr;
   std::unique_ptr<fwi_batch, int (*)(fwi_batch*)> b(new fwi_batch(), fwi_batch_free);
   b->m = m;

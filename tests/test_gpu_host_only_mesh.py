@@ -1,5 +1,6 @@
 """A host-only mesh (fwi_mesh_prepare_host) on a machine with a GPU: setting its velocity gives the
-time step that an uploaded mesh gives, in every form of the tables."""
+time step that an uploaded mesh gives, in every form of the tables; a batch on it, whose kernels
+would read geometry that was never uploaded, is refused."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -23,3 +24,19 @@ def test_velocity_of_a_host_only_mesh(dim, layout, tc):
             dt.append(m.dt)
         m.close()
     assert dt[:2] == dt[2:] and dt[0] > dt[1] > 0
+
+
+def test_batch_on_a_host_only_mesh_is_refused():
+    import numpy as np
+
+    import paper_2108_10946_gb300 as pkg
+    from paper_2108_10946_gb300.lib import FWI_EINVAL, FwiError
+    from synth import meshes, models
+    pkg.build()
+    V, C = meshes.structured_tri(9, 8)
+    m = pkg.Mesh(V, C, 2, 10, cfl_factor=0.8, host_only=True)
+    m.set_velocity(models.smooth2d(m.dof_coords()))
+    with pytest.raises(FwiError, match="host only") as ei:
+        pkg.Batch(m, np.array([[0.5, 0.5]]), np.array([[0.4, 0.4]]))
+    assert ei.value.code == FWI_EINVAL
+    m.close()
