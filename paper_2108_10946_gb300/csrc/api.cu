@@ -1152,6 +1152,7 @@ int fwi_set_velocity(fwi_mesh* m, const double* c) {
   CUDA_TRY(cudaMemcpy(m->d_c64, c, (size_t)N * sizeof(double), cudaMemcpyHostToDevice));
   fwi::VelocityArgs v{};
   v.N = N;
+  v.N_own = m->N_own;
   v.dim = d;
   v.nch = m->layout == 0 ? m->nch() : 0;
   v.dt = m->dt;

@@ -144,7 +144,7 @@ const KernelSet* kernel_set(int dim, int k);
 // The coefficients that follow from the velocity (fwi_set_velocity): inputs in FP64, outputs
 // rounded once. Null outputs are not formed.
 struct VelocityArgs {
-  int N, dim, nch;
+  int N, N_own, dim, nch;  // N_own: DoFs of the chunks' owned ranges (nch > 0)
   double dt, water;
   const double *c, *M, *Mb, *sigma;
   const int *pidx, *sdesc;

@@ -110,8 +110,7 @@ __global__ void __launch_bounds__(256) velocity_kernel(const VelocityArgs v) {
 __global__ void __launch_bounds__(256) splain_kernel(const VelocityArgs v) {
   const int c = (blockIdx.x * 256 + threadIdx.x) / 32, lane = threadIdx.x & 31;
   if (c >= v.nch) return;
-  const int lo = v.sdesc[8 * c + 2], hi = c + 1 < v.nch ? v.sdesc[8 * (c + 1) + 2] : v.N;
-  // (the last chunk's range runs into the halo here: it is plain only if that is, too)
+  const int lo = v.sdesc[8 * c + 2], hi = c + 1 < v.nch ? v.sdesc[8 * (c + 1) + 2] : v.N_own;
   bool plain = true;
   for (int i = lo + lane; i < hi && plain; i += 32) plain = v.cf[i] == 1.f && v.cf[2 * (size_t)v.N + i] == 0.f;
   plain = __all_sync(0xffffffffu, plain);
