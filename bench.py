@@ -372,7 +372,7 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
-def parity_sample(pkg, pool, info, k, S, T_par, workload="marine2d", gstore=False):
+def parity_sample(pkg, pool, info, k, S, T_par, workload="marine2d"):
     """The GPU library against the FP64 oracle on the workload's small marine window (same
     mesher, model, water, layer and absorbing boundary; S shots, T_par seconds): records
     rel-L2 (worst shot) and gradient rel-L2, as the tests measure them. The oracle shots run
@@ -393,7 +393,6 @@ def parity_sample(pkg, pool, info, k, S, T_par, workload="marine2d", gstore=Fals
     xg = mesh.dof_coords()
     mesh.set_velocity(small["model"](xg))
     b = pkg.Batch(mesh, srcs, small["recs"])
-    b.set_gradient_store(gstore)  # the bench's own gradient path
     rec = torch.zeros((S, nt + 1, len(small["recs"])), device="cuda")
     b.forward(torch.from_numpy(np.stack([wav] * S)).cuda(), rec)
     rec = rec.cpu().numpy()
@@ -413,26 +412,24 @@ def parity_sample(pkg, pool, info, k, S, T_par, workload="marine2d", gstore=Fals
                       f", N={info['N']}, {T_par} s, layer, absorbing boundary, residual 0.03 d"}
 
 
-# DRAM bytes (read + write) of one forward time step from an ncu capture of its launches, keyed by
-# (workload, k, S, N) so that it is reported only for the mesh, degree and shot count it was
-# measured on (none for the present kernels on this mesh; profiles/chunk_kernels.md has a graded
-# mesh of its size).
-FORWARD_TRAFFIC = {}
-
 NODES = {2: (7, 6), 3: (12, 9), 4: (18, 12), 5: (30, 15)}  # KMVktri: nodes, shared nodes
 NODES3 = {2: (15, 14), 3: (32, 28)}                           # KMVktet
+# multiply-adds of one derivative contraction (all directions) in the symmetry-adapted form
+BLOCKS, BLOCKS3 = {2: 26, 3: 80, 4: 180, 5: 500}, {2: 162, 3: 768}
 
 
 def step_roofline(prof, k, E, N, S, fp32_tflops, sm_count, peaks, src, dim=2):
     """Roofline entries of the forward time step (element kernels + shared-DoF kernel) and of
     the adjoint step with the gradient integrand, from per-step CUDA-event times.
-    Algorithmic work per step (stated in DESIGN):
+    Algorithmic work per step:
       forward flops = E S 4 d n^2 (two n x n contractions per direction per element and shot)
       adjoint flops = E S 6 d n^2 (plus the contraction of the forward field)
       forward bytes = N (16 S + 8) + E (4 n_s + 4 n_g): u, v read and written per shot, c^2
                       and M^-1 per DoF, shared-node connectivity and Ghat (n_g = 3 in 2D, 6 in
                       3D) per element
-      adjoint bytes = forward bytes + 4 N S (forward field) + 8 N (gradient segment)"""
+      adjoint bytes = forward bytes + 4 N S (forward field) + 8 N (gradient segment)
+    These flops are the dense contractions'. The kernels do fewer (the symmetry-adapted form's
+    blocks): flops_done_per_step and alu_frac_done, their share of the FP32 peak."""
     nn, ns = (NODES if dim == 2 else NODES3)[k]
     d = dim
     ng = 3 if dim == 2 else 6  # Ghat entries per element
@@ -441,7 +438,9 @@ def step_roofline(prof, k, E, N, S, fp32_tflops, sm_count, peaks, src, dim=2):
     adj_ms = (prof["adj_elem_ms"] + prof["adj_node_ms"]) / as_
     hbm = peaks["hbm_gbs"]
 
-    def entry(flops, nbytes, ms, label):
+    def entry(contractions, nbytes, ms, label):
+        flops = E * S * 2 * contractions * d * nn * nn
+        done = E * S * 2 * contractions * (BLOCKS if dim == 2 else BLOCKS3)[k]
         tf = flops / (ms * 1e-3) / 1e12
         gb = nbytes / (ms * 1e-3) / 1e9
         alu_src = f"measured FP32 FMA probe (fwi_fp32_peak), {sm_count} SMs"
@@ -454,15 +453,16 @@ def step_roofline(prof, k, E, N, S, fp32_tflops, sm_count, peaks, src, dim=2):
                  "peak_source": f"{src} MEASURED_PEAKS.json hbm_gbs", "alu_achieved_tflops": tf,
                  "alu_frac": tf / fp32_tflops}
         e.update({"traffic": None, "kernel": f"{label}, {ms * 1e3:.1f} us/step",
-                  "flops_per_step": flops, "bytes_per_step": nbytes})
+                  "flops_per_step": flops, "bytes_per_step": nbytes, "flops_done_per_step": done,
+                  "alu_frac_done": done / (ms * 1e-3) / 1e12 / fp32_tflops})
         return e
 
     fwd_bytes = N * (16 * S + 8) + E * (4 * ns + 4 * ng)
-    roof = entry(E * S * 4 * d * nn * nn, fwd_bytes, fwd_ms,
+    roof = entry(2, fwd_bytes, fwd_ms,
                  "forward time step (element kernels + shared-DoF kernel)")
     roof["element_kernel_us"] = prof["fwd_elem_ms"] / fs * 1e3
     roof["node_kernel_us"] = prof["fwd_node_ms"] / fs * 1e3
-    roof["adjoint"] = entry(E * S * 6 * d * nn * nn, fwd_bytes + 4 * N * S + 8 * N, adj_ms,
+    roof["adjoint"] = entry(3, fwd_bytes + 4 * N * S + 8 * N, adj_ms,
                             "adjoint step with the gradient integrand")
     roof["adjoint"]["element_kernel_us"] = prof["adj_elem_ms"] / as_ * 1e3
     roof["adjoint"]["node_kernel_us"] = prof["adj_node_ms"] / as_ * 1e3
@@ -487,7 +487,6 @@ def degree_line(pkg, k, args, S, fp32_tflops, sm_count, peaks, src):
     mesh = pkg.Mesh(wl["V"], wl["cells"], k, nt, dt=dt, **kw)
     mesh.set_velocity(c)
     b = pkg.Batch(mesh, wl["srcs"][:S], wl["recs"])
-    b.set_gradient_store(not args.no_gradient_store)
     R = len(wl["recs"])
     wav = torch.from_numpy(np.stack([signals.ricker_samples(5.0, dt, nt)] * S)).float().cuda()
     rec = torch.zeros((S, nt + 1, R), device="cuda")
@@ -567,8 +566,6 @@ def run_ours(args):
     S = args.shots
     shots = wl["srcs"][shots_for_rank(len(wl["srcs"]), S, rank, world)]
     batch = pkg.Batch(mesh, shots, wl["recs"])
-    # (fwi_batch_set_gradient_store: accepted, without effect)
-    batch.set_gradient_store(not args.no_gradient_store)
     R = len(wl["recs"])
     wav = np.stack([signals.ricker_samples(wl["f"], dt, nt)] * S)
     wav_d = torch.from_numpy(wav).cuda()
@@ -649,11 +646,6 @@ def run_ours(args):
     clk_sum = clk.summary(local)
     roof = step_roofline(prof, wl["k"], E, N, S, fp32_tflops, sm_count, peaks, src,
                          dim=3 if three_d else 2)
-    traffic = FORWARD_TRAFFIC.get((args.workload, wl["k"], S, N))
-    if traffic is not None:
-        roof["traffic"] = traffic
-        roof["traffic_source"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the "
-                                  "three launches of one forward step on this mesh")
 
     extra_k = []
     # the side measurements (other degrees, plain form, serving) belong to the one-GPU line;
@@ -705,8 +697,7 @@ def run_ours(args):
             # long enough for the sea-floor reflection (near 0.55 s) to reach the receivers,
             # so that the gradient below the masked water is more than rounding noise
             T_par = 0.6 if three_d else {2: 1.5, 3: 1.5, 4: 0.8, 5: 0.6}[wl["k"]]
-            parity = parity_sample(pkg, pool, info, wl["k"], S, T_par, args.workload,
-                                   gstore=not args.no_gradient_store)
+            parity = parity_sample(pkg, pool, info, wl["k"], S, T_par, args.workload)
             ob = oracle_rate(pool, wl["k"], info["dt"], cores, args.ref_steps, args.workload)
         finally:
             pool.close()
@@ -730,7 +721,6 @@ def run_ours(args):
                        "receivers": R, "ckpt_stride": args.ckpt, "C": wl["C"],
                        "l2": "inputs larger than L2 (wavefields of N*S floats, records)",
                        "parallelism": f"shots across {world} GPU(s), replicas of the mesh",
-                       "gradient_store": not args.no_gradient_store and not three_d,
                        "setup_s": setup_s},
             "e2e": {"value": e2e_val, "unit": "DoF-steps/s",
                     "h2d_bytes_per_step": int(wav.nbytes + obs_h.numel() * 4 + (N * 8 if world > 1 else 0)),
@@ -773,8 +763,7 @@ def main():
                     help="where the nvidia-smi clock samples of the timed region are written")
     ap.add_argument("--no-serving", action="store_true", help="skip the serving-stream latency run")
     ap.add_argument("--no-gradient-store", action="store_true",
-                    help="recompute the forward field's gradients in the gradient steps instead "
-                         "of storing them during the recompute (less device memory)")
+                    help="accepted, without effect: no gradient step reads stored gradients")
     ap.add_argument("--serving-scale", type=float, default=1.0,
                     help="element-count factor of the serving pool (1 = 50k-2M triangles)")
     ap.add_argument("--extra-k", default="3,4",
