@@ -131,6 +131,12 @@ int fwi_mesh_host_arrays(const fwi_mesh* m, int32_t* conn, double* mass, double*
  * from 0 on, then those of the halo list. desc and tables may be NULL. */
 int fwi_mesh_chunk_tables(const fwi_mesh* m, int64_t* sizes, int32_t* desc, uint16_t* tables);
 
+/* The damping layer's nodal coefficients as the chunked layout's kernels read them (for inspection
+ * and tests; FWI_EINVAL for the plain layout or before fwi_set_velocity). sizes[2]: layer DoFs Nl,
+ * floats per DoF. dofs[Nl]: the DoF of each row. coefs: in 2D Psi2_xx c^2 (Psi2_zz is its opposite);
+ * in 3D Psi2_kk c^2 of the three directions, then Psi3_kk c^2. dofs and coefs may be NULL. */
+int fwi_mesh_layer_coefs(const fwi_mesh* m, int64_t* sizes, int32_t* dofs, float* coefs);
+
 /* Number of global DoFs N (vertex, edge, face and interior KMV nodes). */
 int fwi_num_dofs(const fwi_mesh* m, int64_t* n);
 

@@ -166,6 +166,7 @@ struct fwi_mesh {
   int* d_sdesc = nullptr;
   unsigned short* d_smeta = nullptr;
   float* d_lpsi = nullptr;            // nodal layer coefficients, [Nl] (2D) or [Nl][4]
+  float* d_lpsi3 = nullptr;           // the others, [Nl][2] (3D)
   float* d_lcs = nullptr;             // the update's layer coefficients, [Nl][8 or 12]
   unsigned char* d_splain = nullptr;  // [nch] set with the velocity
   int nch() const { return (int)ch_e0.size() - 1; }
@@ -1047,6 +1048,24 @@ int fwi_mesh_chunk_tables(const fwi_mesh* m, int64_t* sizes, int32_t* desc, uint
   if (tables) std::memcpy(tables, m->smeta.data(), m->smeta.size() * sizeof(uint16_t));
   return 0;
 }
+int fwi_mesh_layer_coefs(const fwi_mesh* m, int64_t* sizes, int32_t* dofs, float* coefs) {
+  if (!m || !sizes) return fail(FWI_EINVAL, "null argument");
+  if (m->layout != 0) return fail(FWI_EINVAL, "the plain layout keeps other records");
+  if (!m->have_velocity) return fail(FWI_EINVAL, "set the velocity first");
+  const int count = m->dim == 2 ? 1 : 6;
+  sizes[0] = m->Nl;
+  sizes[1] = count;
+  if (dofs)
+    for (int i = 0; i < m->N; ++i)
+      if (m->pidx[i] >= 0) dofs[m->pidx[i]] = i;
+  if (coefs && m->Nl > 0) {
+    const size_t Nl = (size_t)m->Nl, row = count * sizeof(float), w = m->dim == 2 ? 4 : 16;
+    CUDA_TRY(cudaMemcpy2D(coefs, row, m->d_lpsi, w, w, Nl, cudaMemcpyDeviceToHost));
+    if (m->dim == 3) CUDA_TRY(cudaMemcpy2D(coefs + 4, row, m->d_lpsi3, 8, 8, Nl, cudaMemcpyDeviceToHost));
+  }
+  return 0;
+}
+
 
 int fwi_num_dofs(const fwi_mesh* m, int64_t* n) {
   if (!m || !n) return fail(FWI_EINVAL, "null argument");
@@ -1144,6 +1163,7 @@ int fwi_set_velocity(fwi_mesh* m, const double* c) {
   room(&m->d_mask, (size_t)N);
   if (lcf) room(&m->d_lcf, Nl * fwi::layer_coef_count(d));
   if (m->layout == 0) {
+    if (d == 3) room(&m->d_lpsi3, Nl * 2);
     room(&m->d_lpsi, Nl * (d == 2 ? 1 : 4));
     room(&m->d_lcs, Nl * (d == 2 ? 8 : 12));
     room(&m->d_splain, (size_t)m->nch());
@@ -1167,6 +1187,7 @@ int fwi_set_velocity(fwi_mesh* m, const double* c) {
   v.cvel = m->d_c;
   v.cf = m->d_cf;
   v.lcf = lcf ? m->d_lcf : nullptr;
+  v.lpsi3 = m->d_lpsi3;
   v.lpsi = m->d_lpsi;
   v.lcs = m->d_lcs;
   v.mask = m->d_mask;
@@ -1321,6 +1342,7 @@ StepArgs base_args(fwi_batch* b) {
     a.lconn = m->d_lconn;
     a.sdesc = m->d_sdesc;
     a.smeta = m->d_smeta;
+    a.lpsi3 = m->d_lpsi3;
     a.splain = m->d_splain;
     a.lpsi = m->d_lpsi;
     a.lcs = m->d_lcs;
@@ -1995,7 +2017,7 @@ int fwi_mesh_free(fwi_mesh* m) {
   if (!m) return 0;
   void* ptrs[] = {m->d_conn, m->d_geo, m->d_lgeo, m->d_pidx, m->d_c2, m->d_c, m->d_cf,
                   m->d_lcf, m->d_M, m->d_Mb, m->d_sigma, m->d_c64, m->d_mask, m->d_bub, m->d_chunks, m->d_halo, m->d_lconn,
-                  m->d_sdesc, m->d_smeta, m->d_splain, m->d_lpsi, m->d_lcs};
+                  m->d_sdesc, m->d_smeta, m->d_splain, m->d_lpsi, m->d_lpsi3, m->d_lcs};
   for (void* p : ptrs) dfree(p);
   delete m;
   return 0;

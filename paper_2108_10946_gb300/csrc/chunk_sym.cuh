@@ -124,8 +124,8 @@ struct SymStep {
 struct SymSmem {
   int u, f, c2, ps, om, ys, yb, p1, gs, gb, ws, wb, ss, sb, ids, meta, total;
 };
-// Floats per DoF of the layer's nodal coefficients in the table: Psi2 c^2 (2D adjoint; the three
-// sigma of a 3D DoF are read where they are used, the table would take the second CTA's room).
+// Floats per DoF of the layer's nodal coefficients in the table: Psi2 c^2 (2D adjoint; the six
+// of a 3D DoF are read where they are used, the table would take the second CTA's room).
 template <int D, int MODE>
 __host__ __device__ constexpr int sym_psi() { return D == 2 && MODE != 0 ? 1 : 0; }
 
@@ -236,7 +236,10 @@ __device__ __forceinline__ void sym_load(const StepArgs& a, const SymStep& x, co
       sym_prefetch(a.cf + 2 * (size_t)a.N + cd.own, on);
     }
     if (LAYER) sym_prefetch(a.lcs + pi0 * SYM_LCS<D>, on * SYM_LCS<D>);
-    if (LAYER && D == 3) sym_prefetch(a.lpsi + pi0 * 4, on * 4);
+    if (LAYER && D == 3) {
+      sym_prefetch(a.lpsi + pi0 * 4, on * 4);
+      sym_prefetch(a.lpsi3 + pi0 * 2, on * 2);
+    }
     if (LAYER && D == 3 && S == SG) sym_prefetch(a.Y + pi0 * SG, on * SG);
     // and the ranges of the chunk a wave of CTAs further on
     const int nc = chunk + a.wave;
@@ -652,9 +655,9 @@ __device__ __forceinline__ bool sym_tri_body(const StepArgs& a, const SymStep& x
 // The walk over the orbits of a tetrahedron: derivatives of N fields, node(q, g) for each node with
 // g[field][axis], then the divergence of the fluxes that node leaves in g[0] to Y (and of g[1] to
 // Y2, if DIV2).
-template <class V, int NN, int N, bool DIV2, int O, class F>
+template <class V, int NN, int N, bool DIV2, int O, class F, class G>
 __device__ __forceinline__ void sym_tet_orbits(const TetCoef<V, NN>* const (&U)[N], TetCoef<V, NN>& Y,
-                                               TetCoef<V, NN>& Y2, F node) {
+                                               TetCoef<V, NN>& Y2, F node, G coefs) {
   if constexpr (O < TetSym<NN>::NO) {
     V g[N > 1 || !DIV2 ? N : 2][3][4];
 #pragma unroll
@@ -670,7 +673,7 @@ __device__ __forceinline__ void sym_tet_orbits(const TetCoef<V, NN>* const (&U)[
       for (int f = 0; f < N; ++f)
 #pragma unroll
         for (int d = 0; d < 3; ++d) x[f][d] = g[f][d][h];
-      node(TetSym<NN>::node(O, h), x);
+      node(TetSym<NN>::node(O, h), x, [&] { return coefs(TetSym<NN>::node(O, h)); });
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         g[0][d][h] = x[0][d];
@@ -685,19 +688,30 @@ __device__ __forceinline__ void sym_tet_orbits(const TetCoef<V, NN>* const (&U)[
       tet_div<V, NN, O, 1>(g[1][1], Y2);
       tet_div<V, NN, O, 2>(g[1][2], Y2);
     }
-    sym_tet_orbits<V, NN, N, DIV2, O + 1>(U, Y, Y2, node);
+    sym_tet_orbits<V, NN, N, DIV2, O + 1>(U, Y, Y2, node, coefs);
   }
 }
 
-// The same walk rolled (KMV3: all orbits are alike; node slots 4 o + h). The unrolled code of the
-// layer kernels, some 7,000 instructions, does not fit the instruction caches.
-template <class V, int N, bool DIV2, class F>
+// A layer DoF's nodal coefficients: Psi2 c^2 of the three directions, Psi3 c^2.
+struct LayerPsi {
+  float4 a;  // Psi2, then the first of Psi3
+  float2 b;
+};
+
+// The same walk rolled (KMV3: all orbits are alike; node slots 4 o + h). coefs(q): the layer's
+// coefficients of a node, with EARLY those of an orbit before its derivatives. The unrolled code of
+// the layer kernels, some 7,000 instructions, does not fit the instruction caches.
+template <class V, int N, bool DIV2, bool EARLY, class F, class G>
 __device__ __forceinline__ void sym_tet_roll(const TetCoef<V, 32>* const (&U)[N], TetCoef<V, 32>& Y, TetCoef<V, 32>& Y2,
-                                             F node) {
+                                             F node, G coefs) {
   constexpr int NG = N > 1 || !DIV2 ? N : 2;
 #pragma unroll 1
   for (int o = 0; o < 8; ++o) {
     const float* t = c_sym + o * 96;  // [axis][output][mode] of this orbit
+    LayerPsi ps[4];
+    if constexpr (EARLY)
+#pragma unroll
+      for (int h = 0; h < 4; ++h) ps[h] = coefs(4 * o + h);
     V g[NG][3][4];
 #pragma unroll
     for (int f = 0; f < N; ++f)
@@ -719,7 +733,8 @@ __device__ __forceinline__ void sym_tet_roll(const TetCoef<V, 32>* const (&U)[N]
       for (int f = 0; f < N; ++f)
 #pragma unroll
         for (int d = 0; d < 3; ++d) x[f][d] = g[f][d][h];
-      node(4 * o + h, x);
+      if constexpr (EARLY) node(4 * o + h, x, [&] { return ps[h]; });
+      else node(4 * o + h, x, [&] { return coefs(4 * o + h); });
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         g[0][d][h] = x[0][d];
@@ -784,7 +799,7 @@ __device__ __forceinline__ bool sym_tet_body(const StepArgs& a, const SymStep& x
   const float* cs = sm + L.c2 + sym_shift(a.c2 + cd.own);
   const int ps = el * SG + ln, pb = el * NI * SG + ln;  // a thread's own places (see sym_tri_body)
   // q: a node's slot (sym_slot_node: the local node, at KMV3 orbit by orbit)
-  constexpr bool ROLL = NN == 32;
+  constexpr bool ROLL = NN == 32, EARLY = LAYER;
   auto bi = [](int q) { return ROLL ? NN - 1 - q : q - NS; };  // a bubble's place in its element
   auto at = [&](int q) { return q < NS ? (int)lq[q * PE] : bub + bi(q); };
   auto ld = [&](const float* p) { return *reinterpret_cast<const V*>(p); };
@@ -813,13 +828,19 @@ __device__ __forceinline__ bool sym_tet_body(const StepArgs& a, const SymStep& x
     const float* p1 = sm + L.p1 + (LAYER ? sym_shift(a.P + (pi0 * S + s0) * 3) : 0) + ln;
     float* p2 = sm + L.sb + (LAYER ? sym_shift(a.P + ((pi0 + cd.nsh) * S + s0) * 3) : 0) + el * NI * 3 * SG + ln;
     const int* ids = reinterpret_cast<const int*>(sm + L.ids);
-    const float4* sig = reinterpret_cast<const float4*>(a.lpsi);
+    const float4* psi = reinterpret_cast<const float4*>(a.lpsi);
+    const float2* psi3 = reinterpret_cast<const float2*>(a.lpsi3);
     tet_analyse<V, NN>(U, [&](int q) { return ld(us + at(slot_of(q)) * SG); });
     tet_zero(Y);
     if constexpr (W) tet_zero(Y2);
     // one node: x[0] in are the field's derivatives, out the flux (x[1]: the other field's; out, in
     // the layer's adjoint, the omega row's flux)
-    auto node = [&](int q, auto& g) {
+    auto coefs = [&](int q) {
+      const int l = at(q), on = cd.nsh + nb;
+      const int pi = l < on ? (int)pi0 + l : ids[l - on - SYM_GAP] - a.p_halo;
+      return LayerPsi{__ldg(psi + pi), __ldg(psi3 + pi)};
+    };
+    auto node = [&](int q, auto& g, auto layer_psi) {
       const float w = c_w[q];
       const int l = at(q);
       const float c2 = cs[l];
@@ -831,32 +852,29 @@ __device__ __forceinline__ bool sym_tet_body(const StepArgs& a, const SymStep& x
         st(own(L.gs, L.gb, q), mul2(dup<V>(w), fma2(h0, g[1][0], fma2(h1, g[1][1], mul2(h2, g[1][2])))));
       V f[3] = {mul2(wc, h0), mul2(wc, h1), mul2(wc, h2)};
       if constexpr (LAYER) {
-        const int on = cd.nsh + nb;
-        const float4 sg = __ldg(sig + (l < on ? (int)pi0 + l : ids[l - on - SYM_GAP] - a.p_halo));
-        const float s1 = sg.x, s2 = sg.y, s3 = sg.z, tr = s1 + s2 + s3;
-        const float psi2[3] = {c2 * (2.f * s1 - tr), c2 * (2.f * s2 - tr), c2 * (2.f * s3 - tr)};
-        const float psi3[3] = {c2 * s2 * s3, c2 * s1 * s3, c2 * s1 * s2};
+        // (formed in FP64 and rounded once: Psi2 cancels where two directions are damped)
+        const LayerPsi lp = layer_psi();
+        const float psi2[3] = {lp.a.x, lp.a.y, lp.a.z}, psi3k[3] = {lp.a.w, lp.b.x, lp.b.y};
         float* p = q < NS ? const_cast<float*>(p1) + (l - (l >= cd.nsh ? nb : 0)) * 3 * SG : p2 + bi(q) * 3 * SG;
-        V P[3], Q[3], s[3];
+        V P[3], Q[3], R[3], s[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
           P[k] = ld(p + k * SG);
           s[k] = fma2(dup<V>(A[0][k]), g0, fma2(dup<V>(A[1][k]), g1, mul2(dup<V>(A[2][k]), g2)));
           if constexpr (OM) {  // both gradients, each with its Psi c^2
             const V y = fma2(dup<V>(A[0][k]), g[1][0], fma2(dup<V>(A[1][k]), g[1][1], mul2(dup<V>(A[2][k]), g[1][2])));
-            s[k] = fma2(dup<V>(-psi3[k]), y, mul2(dup<V>(psi2[k]), s[k]));
+            s[k] = fma2(dup<V>(-psi3k[k]), y, mul2(dup<V>(psi2[k]), s[k]));
           }
           s[k] = mul2(dup<V>(w), s[k]);
           Q[k] = ADJ ? mul2(dup<V>(w * psi2[k]), P[k]) : mul2(dup<V>(w), P[k]);
+          if constexpr (W) R[k] = mul2(dup<V>(w * psi3k[k]), P[k]);
           if (q < NS) st(sm + L.ss + ps + (k * NS + q) * PE * SG, s[k]);
           else st(p + k * SG, s[k]);  // a bubble's P gives way to its layer sums
         }
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
           f[d] = fma2(dup<V>(A[d][0]), Q[0], fma2(dup<V>(A[d][1]), Q[1], fma2(dup<V>(A[d][2]), Q[2], f[d])));
-          if constexpr (W)
-            g[1][d] = fma2(dup<V>(w * psi3[0] * A[d][0]), P[0],
-                           fma2(dup<V>(w * psi3[1] * A[d][1]), P[1], mul2(dup<V>(w * psi3[2] * A[d][2]), P[2])));
+          if constexpr (W) g[1][d] = fma2(dup<V>(A[d][0]), R[0], fma2(dup<V>(A[d][1]), R[1], mul2(dup<V>(A[d][2]), R[2])));
         }
       }
 #pragma unroll
@@ -864,12 +882,12 @@ __device__ __forceinline__ bool sym_tet_body(const StepArgs& a, const SymStep& x
     };
     if constexpr (NF == 2) {
       const TetCoef<V, NN>* const fields[2] = {&U, &F};
-      if constexpr (ROLL) sym_tet_roll<V, 2, W>(fields, Y, Y2, node);
-      else sym_tet_orbits<V, NN, 2, W, 0>(fields, Y, Y2, node);
+      if constexpr (ROLL) sym_tet_roll<V, 2, W, EARLY>(fields, Y, Y2, node, coefs);
+      else sym_tet_orbits<V, NN, 2, W, 0>(fields, Y, Y2, node, coefs);
     } else {
       const TetCoef<V, NN>* const fields[1] = {&U};
-      if constexpr (ROLL) sym_tet_roll<V, 1, W>(fields, Y, Y2, node);
-      else sym_tet_orbits<V, NN, 1, W, 0>(fields, Y, Y2, node);
+      if constexpr (ROLL) sym_tet_roll<V, 1, W, EARLY>(fields, Y, Y2, node, coefs);
+      else sym_tet_orbits<V, NN, 1, W, 0>(fields, Y, Y2, node, coefs);
     }
   }
   if (LAYER) __syncthreads();  // every P of a shared DoF has been read

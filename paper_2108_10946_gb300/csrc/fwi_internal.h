@@ -65,7 +65,8 @@ struct StepArgs {
   const float* cf;     // [3][N]: c1, c2, c3 of the increment update
   const int* pidx;     // [N]
   const float* lcf;    // [Nl][LCF] layer coefficients (see layer_coef_layout)
-  const float* lpsi;   // of the layer DoFs: 2D [Nl] Psi2_xx c^2 = -Psi2_zz c^2; 3D [Nl][4] sigma
+  const float* lpsi;   // of the layer DoFs: 2D [Nl] Psi2_xx c^2 = -Psi2_zz c^2; 3D [Nl][4] Psi2_kk c^2, Psi3_xx c^2
+  const float* lpsi3;  // 3D [Nl][2] Psi3_yy c^2, Psi3_zz c^2
   const float* lcs;    // [Nl][8 or 12] the update's layer coefficients (chunk_sym.cuh)
   float* u;
   float* u_out;        // where u^{n+1} goes (symmetry-adapted kernels; u itself elsewhere)
@@ -148,7 +149,7 @@ struct VelocityArgs {
   double dt, water;
   const double *c, *M, *Mb, *sigma;
   const int *pidx, *sdesc;
-  float *c2, *cvel, *cf, *lcf, *lpsi, *lcs;
+  float *c2, *cvel, *cf, *lcf, *lpsi, *lpsi3, *lcs;
   unsigned char *mask, *splain;
 };
 

@@ -101,7 +101,9 @@ __global__ void __launch_bounds__(256) velocity_kernel(const VelocityArgs v) {
 #pragma unroll
     for (int k = 0; k < 12; ++k) v.lcs[(size_t)pi * 12 + k] = o[k];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v.lpsi[(size_t)pi * 4 + k] = k < 3 ? (float)s[k] : 0.f;
+    for (int k = 0; k < 4; ++k) v.lpsi[(size_t)pi * 4 + k] = k < 3 ? q[L::PSI2 + k] : q[L::PSI3];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) v.lpsi3[(size_t)pi * 2 + k] = q[L::PSI3 + 1 + k];
   }
 }
 

@@ -58,6 +58,7 @@ def load():
         "fwi_dof_coords": (ctypes.c_int, [_P, _P]),
         "fwi_element": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int), _P, _P, _P]),
         "fwi_mesh_chunk_tables": (ctypes.c_int, [_P, _P, _P, _P]),
+        "fwi_mesh_layer_coefs": (ctypes.c_int, [_P, _P, _P, _P]),
         "fwi_set_velocity": (ctypes.c_int, [_P, _P]),
         "fwi_locate": (ctypes.c_int, [_P, _P, ctypes.c_int, _P, _P]),
         "fwi_reference_element": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_int),
@@ -239,6 +240,15 @@ class Mesh:
         tab = np.zeros(int(n[3]), dtype=np.uint16)
         _check(_lib.fwi_mesh_chunk_tables(self._h, _ptr(n), _ptr(desc), _ptr(tab)))
         return int(n[1]), int(n[2]), desc, tab
+
+    def layer_coefs(self):
+        """(DoFs [Nl], coefficients [Nl][1 or 6]) of the damping layer; see fwi_mesh_layer_coefs."""
+        n = np.zeros(2, dtype=np.int64)
+        _check(_lib.fwi_mesh_layer_coefs(self._h, _ptr(n), None, None))
+        dofs = np.zeros(int(n[0]), dtype=np.int32)
+        coefs = np.zeros((int(n[0]), int(n[1])), dtype=np.float32)
+        _check(_lib.fwi_mesh_layer_coefs(self._h, _ptr(n), _ptr(dofs), _ptr(coefs)))
+        return dofs, coefs
 
     def locate(self, pts):
         """(element index in the library's order [npts], reference coordinates [npts][dim])
