@@ -124,7 +124,7 @@ struct fwi_mesh {
   int N_own = 0;      // DoFs owned by one chunk: [0, N_own); halo DoFs [N_own, N)
   int nch0 = 0;       // chunks [0, nch0) have no damping-layer element
   int L_max = 0;      // largest local DoF table of a chunk (owned + halo)
-  int O_max = 0, H_max = 0;  // largest owned range and halo list of a chunk
+  int H_max = 0;  // longest halo list of a chunk
   std::vector<int32_t> bub;                       // [E] first bubble DoF of every element
   std::vector<int32_t> ch_e0, ch_own_lo, ch_nsh;  // chunk element ranges, owned ranges
   std::vector<int32_t> ch_halo_ptr, halo_ids;     // per-chunk halo lists (global DoF ids)
@@ -794,7 +794,6 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
         }
       m->ch_halo_ptr[c + 1] = (int)m->halo_ids.size();
       m->L_max = std::max(m->L_max, own_n + (int)hmap.size());
-      m->O_max = std::max(m->O_max, own_n);
       m->H_max = std::max(m->H_max, (int)hmap.size());
     }
     build_incidence(m.get());
@@ -968,8 +967,8 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
   std::vector<int> conn_dev((size_t)m->ns * E);
   for (int e = 0; e < E; ++e)
     for (int q = 0; q < m->ns; ++q) conn_dev[(size_t)q * E + e] = m->conn[(size_t)e * n + q];
-  std::vector<int> chunks;
-  if (m->layout == 0) {
+  std::vector<int> chunks;  // of the tensor-core step, like lconn
+  if (m->use_tc) {
     for (int c = 0; c < m->nch(); ++c) {
       chunks.push_back(m->ch_e0[c]);
       chunks.push_back(m->ch_e0[c + 1] - m->ch_e0[c]);
@@ -988,10 +987,9 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
   std::vector<int> halo_dev(m->halo_ids.begin(), m->halo_ids.end());
   if (halo_dev.empty()) halo_dev.push_back(0);
   int rc;
-  if (m->layout == 0 && ((rc = upload(&m->d_chunks, chunks)) || (rc = upload(&m->d_halo, halo_dev)) ||
-
-                         (rc = upload(&m->d_lconn, m->lconn)) || (rc = upload(&m->d_sdesc, m->sdesc)) ||
-                         (rc = upload(&m->d_smeta, m->smeta)))) {
+  if ((m->use_tc && ((rc = upload(&m->d_chunks, chunks)) || (rc = upload(&m->d_lconn, m->lconn)))) ||
+      (m->layout == 0 && ((rc = upload(&m->d_halo, halo_dev)) || (rc = upload(&m->d_sdesc, m->sdesc)) ||
+                          (rc = upload(&m->d_smeta, m->smeta))))) {
     fwi_mesh_free(m.release());
     return rc;
   }
@@ -1332,7 +1330,6 @@ StepArgs base_args(fwi_batch* b) {
     a.ch0 = 0;
     a.N_own = m->N_own;
     a.L_max = m->L_max;
-    a.O_max = m->O_max;
     a.H_max = m->H_max;
     a.PE = m->P;
     a.SG = std::min(b->S, 4);

@@ -9,8 +9,8 @@
 // and sends the halo DoFs' contributions to the global accumulators.
 //
 // Layer chunks of steps without the gradient add a third group (chunk_load_layer, issued
-// once the layer indices are in the table): the damping-layer auxiliaries P (and in the 3D
-// forward Y) of every local layer DoF. Gradient steps, whose table is the largest, read P
+// once the layer indices are in the table): the damping-layer auxiliaries P of every local layer
+// DoF. Gradient steps, whose table is the largest, read P
 // from global memory (prefetched into L2 at the start of the element phase), so that two CTAs
 // still fit on an SM: with P in the table they ran at one CTA per SM and slower (542 against
 // 393 us per step on the KMV5 marine mesh).
@@ -22,7 +22,7 @@
 // in different banks): u, y [SG][Lm]; c2 [Lm]; pi [Lm] (int); v [SG][Lm] and cf [3][Lm]
 // (not in layer chunks); gradient
 // steps: F [SG][Lm], g [SG][Lm], cv [Lm]; layer chunks: s [D][SG][Lm], P [D][SG][Lm] (not in
-// gradient steps) (and in 3D sY [D][SG][Lm], yw [SG][Lm], Yv [SG][Lm]).
+// gradient steps).
 #pragma once
 #include "update.cuh"
 
@@ -48,12 +48,12 @@ __host__ __device__ inline size_t chunk_tab_floats(int L, int SG, int D, bool gr
   const size_t Lm = (size_t)chunk_stride(L);
   size_t f = Lm * (2 * (size_t)SG + 2) + (layer ? 0 : Lm * ((size_t)SG + 3));
   if (grad) f += Lm * (2 * (size_t)SG + 1);
-  if (layer) f += (grad ? 1 : 2) * Lm * D * SG + (D == 3 ? Lm * D * SG + 2 * Lm * SG : 0);
+  if (layer) f += (grad ? 1 : 2) * Lm * D * SG;
   return f;
 }
 
 struct ChunkTab {
-  float *u, *y, *v, *c2, *cf, *F, *g, *cv, *s, *P, *sY, *yw, *Yv;
+  float *u, *y, *v, *c2, *cf, *F, *g, *cv, *s, *P;
   int* pi;
 };
 
@@ -75,9 +75,6 @@ __device__ __forceinline__ ChunkTab chunk_tab(float* base, int Lm, int SG, int D
   p = t.cv + (grad ? Lm : 0);
   t.s = p;
   t.P = t.s + (layer ? (size_t)D * R : 0);
-  t.sY = t.P + (layer && !grad ? (size_t)D * R : 0);
-  t.yw = t.sY + (layer && D == 3 ? (size_t)D * R : 0);
-  t.Yv = t.yw + (layer && D == 3 ? R : 0);
   return t;
 }
 
@@ -148,23 +145,17 @@ __device__ __forceinline__ void chunk_load(const StepArgs& a, const ChunkDesc& c
       t.g[q * Lm + l] = 0.f;
     }
   if (LAYER) {
-    for (int i = tid; i < Lm * D * SG; i += nth) {
-      t.s[i] = 0.f;
-      if constexpr (D == 3) t.sY[i] = 0.f;
-    }
-    if constexpr (D == 3)
-      for (int i = tid; i < Lm * SG; i += nth) t.yw[i] = 0.f;
+    for (int i = tid; i < Lm * D * SG; i += nth) t.s[i] = 0.f;
   }
 }
 
 // Layer chunks, after group 0 has landed and a barrier: the layer auxiliaries of every
-// local layer DoF as a third copy group (P; Y in the 3D forward), zeros elsewhere.
+// local layer DoF as a third copy group, zeros elsewhere.
 template <int D>
 __device__ __forceinline__ void chunk_load_layer(const StepArgs& a, const ChunkDesc& cd,
                                                  const ChunkTab& t, int Lm, int SG, int lg, int s0,
                                                  int tid, int nth) {
   const int S = a.S;
-  const bool fwd3 = D == 3 && a.mode == 0;
   for (int i = tid; i < cd.L * SG; i += nth) {
     const int l = i >> lg, q = i & (SG - 1);
     const int pi = t.pi[l];
@@ -172,11 +163,9 @@ __device__ __forceinline__ void chunk_load_layer(const StepArgs& a, const ChunkD
 #pragma unroll
       for (int k = 0; k < D; ++k)
         cp_async4(t.P + (size_t)(k * SG + q) * Lm + l, a.P + ((size_t)pi * D + k) * S + s0 + q);
-      if (fwd3) cp_async4(t.Yv + (size_t)q * Lm + l, a.Y + (size_t)pi * S + s0 + q);
     } else {
 #pragma unroll
       for (int k = 0; k < D; ++k) t.P[(size_t)(k * SG + q) * Lm + l] = 0.f;
-      if (fwd3) t.Yv[(size_t)q * Lm + l] = 0.f;
     }
   }
   cp_async_commit();
@@ -198,14 +187,7 @@ __device__ __forceinline__ void chunk_prefetch_update(const StepArgs& a, const C
       for (int r = 0; r < 3; ++r) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.cf + (size_t)r * a.N + dof));
     }
     const int pi = t.pi[l];
-    if (pi >= 0) {
-      const float* lc = a.lcf + (size_t)pi * LC::COUNT;
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(lc));
-      if constexpr (D == 3) {  // 88-byte records may straddle two lines; the omega state Y
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(lc + LC::COUNT - 1));
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(a.Y + (size_t)pi * a.S + s0));
-      }
-    }
+    if (pi >= 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.lcf + (size_t)pi * LC::COUNT));
   }
   if (a.ring_u != nullptr) {  // gradient steps read P of every local layer DoF from global memory
     for (int l = tid; l < cd.L; l += nth) {
@@ -225,7 +207,6 @@ template <int D, bool GRAD, bool LAYER>
 __device__ __forceinline__ void chunk_store(const StepArgs& a, const ChunkDesc& cd, const ChunkTab& t,
                                             int Lm, int SG, int lg, int s0, int tid, int nth) {
   const int S = a.S;
-  const bool adj = a.mode != 0;
   if (LAYER) {
     // layer chunks read v and c1..c3 from global memory: four items per round, their reads
     // issued before any write
@@ -248,28 +229,24 @@ __device__ __forceinline__ void chunk_store(const StepArgs& a, const ChunkDesc& 
         const int i = i0 + k * nth;
         if (i >= cd.own_n * SG) break;
         const int l = i >> lg, q = i & (SG - 1), s = s0 + q;
-        float sU[D], sY[D], po[D];
-        float ywv = 0.f;
+        float sU[D], po[D];
 #pragma unroll
         for (int d = 0; d < D; ++d) {
           sU[d] = t.s[(size_t)(d * SG + q) * Lm + l];
-          sY[d] = 0.f;
-          if constexpr (D == 3) sY[d] = t.sY[(size_t)(d * SG + q) * Lm + l];
           po[d] = GRAD ? 0.f : t.P[(size_t)(d * SG + q) * Lm + l];
         }
-        if constexpr (D == 3) ywv = t.yw[(size_t)q * Lm + l];
         dof_update_pre<D>(a, cd.own_lo + l, s, t.y[q * Lm + l], t.u[q * Lm + l], vo[k], c1[k], c2[k],
-                          c3[k], t.pi[l], sU, sY, ywv, GRAD ? nullptr : po);
+                          c3[k], t.pi[l], sU, nullptr, 0.f, GRAD ? nullptr : po);
       }
     }
   } else {
     for (int i = tid; i < cd.own_n * SG; i += nth) {
       const int l = i >> lg, q = i & (SG - 1), s = s0 + q;
-      float sU[D], sY[D];
+      float sU[D];
 #pragma unroll
-      for (int d = 0; d < D; ++d) sU[d] = sY[d] = 0.f;
+      for (int d = 0; d < D; ++d) sU[d] = 0.f;
       dof_update_pre<D>(a, cd.own_lo + l, s, t.y[q * Lm + l], t.u[q * Lm + l], t.v[q * Lm + l],
-                        t.cf[l], t.cf[Lm + l], t.cf[2 * (size_t)Lm + l], -1, sU, sY, 0.f);
+                        t.cf[l], t.cf[Lm + l], t.cf[2 * (size_t)Lm + l], -1, sU, nullptr, 0.f);
     }
   }
   for (int i = tid; i < cd.hn * SG; i += nth) {
@@ -281,15 +258,8 @@ __device__ __forceinline__ void chunk_store(const StepArgs& a, const ChunkDesc& 
       const int pi = t.pi[l];
       if (pi >= 0) {
 #pragma unroll
-        for (int k = 0; k < D; ++k) {
+        for (int k = 0; k < D; ++k)
           atomicAdd(a.Pacc + ((size_t)pi * D + k) * S + s, t.s[(size_t)(k * SG + q) * Lm + l]);
-          if constexpr (D == 3) {
-            if (!adj) atomicAdd(a.PaccY + ((size_t)pi * D + k) * S + s, t.sY[(size_t)(k * SG + q) * Lm + l]);
-          }
-        }
-        if constexpr (D == 3) {
-          if (adj) atomicAdd(a.Yacc + (size_t)pi * S + s, t.yw[(size_t)q * Lm + l]);
-        }
       }
     }
   }

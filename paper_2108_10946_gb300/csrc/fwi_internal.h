@@ -33,13 +33,13 @@ struct StepArgs {
   int h0, hcnt;        // node kernel range: DoFs [h0, h0 + hcnt), r indexed from h0
   int halo_layer;      // chunked layout: first halo DoF of the damping layer (they are the last)
   // chunked layout (layout 0)
-  int O_max, H_max;    // largest owned-DoF range and halo list of a chunk
+  int H_max;           // longest halo list of a chunk
   int nch, nch0, ch0, N_own, L_max, PE, SG;  // chunks, owned DoFs, largest chunk table, elements per
                                   // chunk, shots per CTA
   const int* bub;            // [E] first bubble DoF of each element
-  const int* chunks;         // [nch][6]: e0, ne, own_lo, own_n, nsh, halo_ptr
+  const int* chunks;         // [nch][6]: e0, ne, own_lo, own_n, nsh, halo_ptr (tensor-core step)
   const int* halo;           // halo DoF ids, chunk by chunk
-  const unsigned short* lconn;  // [NS][Es] chunk-local index of each shared node
+  const unsigned short* lconn;  // [NS][Es] chunk-local index of each shared node (same)
   // symmetry-adapted chunk kernels (chunk_sym.cuh): chunk descriptors [nch][8] (e0, ne, first
   // owned DoF, owned shared DoFs, halo list and its length, tables and their floats); the tables,
   // chunk by chunk, 16-bit: table position [NS][PE] of every shared node, the incidence lists
