@@ -174,11 +174,12 @@ int run_t(const StepArgs& a, const RunArgs& r, cudaStream_t st) {
     if (e != cudaSuccess) return -(int)e;
     configured[dev] = bytes;
   }
+  const int sms = nsm[dev];
   lk.unlock();
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_run<MODE>, NT_RUN, bytes);
   if (e != cudaSuccess) return -(int)e;
   const int64_t nwork = (int64_t)a.nch * (a.S / SG);
-  const int64_t room = (int64_t)per * nsm[dev];
+  const int64_t room = (int64_t)per * sms;
   if (nwork > RUN_MAX || nwork > room) return 0;
   const int grid = (int)std::min(nwork, room);
   StepArgs b = a;
@@ -214,10 +215,10 @@ int launch_t(void (*kernel)(const StepArgs), int which, size_t bytes, const Step
     wave[which][dev] = per * nsm;
     configured[which][dev] = bytes;
   }
-  lk.unlock();
   StepArgs b = a;
   b.ch0 = ch0;
   b.wave = down ? -wave[which][dev] : wave[which][dev];
+  lk.unlock();
   kernel<<<dim3((unsigned)nch, (unsigned)(a.S / SG)), NT, bytes, st>>>(b);
   return 0;
 }
