@@ -597,8 +597,9 @@ int mesh_create(const double* verts, int64_t nverts, const int32_t* cells, int64
     return fail(FWI_EINVAL, "tensor_cores = 1 needs triangles and the chunked layout");
   m->use_tc = d == 2 && m->layout == 0 && params->tensor_cores > 0;
   // elements per chunk: the kernels' most where that still gives every SM two chunks
+  constexpr int64_t kTwoPerSm = 2 * 152;
   m->P = 32;
-  if (!m->use_tc && ncells >= (int64_t)304 * fwi::sym_pe(d, ks->nn)) m->P = fwi::sym_pe(d, ks->nn);
+  if (!m->use_tc && ncells >= kTwoPerSm * fwi::sym_pe(d, ks->nn)) m->P = fwi::sym_pe(d, ks->nn);
   if (!host_only) CUDA_TRY(cudaGetDevice(&m->device));
   std::string err;
   if (!kmvtab::build(d, params->k, m->el, err)) return fail(FWI_EINVAL, "KMV tabulation: " + err);
@@ -1046,6 +1047,7 @@ int fwi_mesh_chunk_tables(const fwi_mesh* m, int64_t* sizes, int32_t* desc, uint
   if (tables) std::memcpy(tables, m->smeta.data(), m->smeta.size() * sizeof(uint16_t));
   return 0;
 }
+
 int fwi_mesh_layer_coefs(const fwi_mesh* m, int64_t* sizes, int32_t* dofs, float* coefs) {
   if (!m || !sizes) return fail(FWI_EINVAL, "null argument");
   if (m->layout != 0) return fail(FWI_EINVAL, "the plain layout keeps other records");
@@ -1063,7 +1065,6 @@ int fwi_mesh_layer_coefs(const fwi_mesh* m, int64_t* sizes, int32_t* dofs, float
   }
   return 0;
 }
-
 
 int fwi_num_dofs(const fwi_mesh* m, int64_t* n) {
   if (!m || !n) return fail(FWI_EINVAL, "null argument");
@@ -1161,8 +1162,8 @@ int fwi_set_velocity(fwi_mesh* m, const double* c) {
   room(&m->d_mask, (size_t)N);
   if (lcf) room(&m->d_lcf, Nl * fwi::layer_coef_count(d));
   if (m->layout == 0) {
-    if (d == 3) room(&m->d_lpsi3, Nl * 2);
     room(&m->d_lpsi, Nl * (d == 2 ? 1 : 4));
+    if (d == 3) room(&m->d_lpsi3, Nl * 2);
     room(&m->d_lcs, Nl * (d == 2 ? 8 : 12));
     room(&m->d_splain, (size_t)m->nch());
   }
@@ -1185,8 +1186,8 @@ int fwi_set_velocity(fwi_mesh* m, const double* c) {
   v.cvel = m->d_c;
   v.cf = m->d_cf;
   v.lcf = lcf ? m->d_lcf : nullptr;
-  v.lpsi3 = m->d_lpsi3;
   v.lpsi = m->d_lpsi;
+  v.lpsi3 = m->d_lpsi3;
   v.lcs = m->d_lcs;
   v.mask = m->d_mask;
   v.splain = m->d_splain;
@@ -1339,9 +1340,9 @@ StepArgs base_args(fwi_batch* b) {
     a.lconn = m->d_lconn;
     a.sdesc = m->d_sdesc;
     a.smeta = m->d_smeta;
-    a.lpsi3 = m->d_lpsi3;
     a.splain = m->d_splain;
     a.lpsi = m->d_lpsi;
+    a.lpsi3 = m->d_lpsi3;
     a.lcs = m->d_lcs;
     a.halo_layer = m->Nl > 0 ? m->halo_layer : m->N;
     a.T_max = m->T_max;
@@ -1405,8 +1406,10 @@ void run_step(fwi_batch* b, const StepArgs& a, cudaStream_t st) {
     // the layer chunks run on a second stream, concurrently with the others (disjoint owned
     // DoFs; halo sums by atomics); the node kernel waits for both. Up to kBothMax chunks and shot
     // groups they share a launch instead: the fork and join cost more calls than such a step lasts,
-    // larger ones gain more from each kind's own shared memory (KMV3, 29k triangles, 8 shots: 31 us
-    // per step in two launches)
+    // larger ones gain more from each kind's own shared memory. Two launches against one, us per
+    // forward step at 2000, 3500, 5000, 7000 (chunk, group) pairs: KMV5, 4 shots 68/61, 101/108,
+    // 138/144, 184/196; KMV3, 8 shots 43/40, 66/59, 94/91, 125/136; KMV2 tetrahedra, 4 shots 98/92,
+    // 166/158, 215/206, 304/295 (tetrahedra gain at every size measured, 2 % at 10,000)
     const bool kinds = b->st2 && b->m->nch0 > 0 && b->m->nch() > b->m->nch0;
     const bool both = kinds && !(a.tc && a.mode != 0) && (int64_t)a.nch * (a.S / a.SG) <= kBothMax;
     const bool fork = kinds && !both;

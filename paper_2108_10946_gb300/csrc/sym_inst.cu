@@ -33,17 +33,23 @@ __constant__ float c_w[NN];
 namespace fwi {
 namespace {
 constexpr int NT = SymMap<SG, false>::NT, NT_RUN = SymMap<SG, true>::NT;
-// Registers a thread may take: enough CTAs per SM to hide the loads of one behind the arithmetic of
-// the others. KMV5 gradient steps hold more at a time and lose less to a fourth CTA less than to
-// spills (marine mesh, one gradient of 75 steps: 128.5 ms at 168, 133.1 ms at 128); every other
-// kernel is best at 128 (KMV4, S = 4, 250k triangles: 8.0 ms for 100 steps, 10.9 ms at 204; KMV3,
-// 120k: 8.9 and 9.8 ms), but KMV2's at one shot, which do little with what they load (2M triangles,
-// 50 steps: 3.54 ms at 48, 3.71 ms at 80).
-// Most CTAs of a launch of several steps. 256 of them (KMV2, 8,192 triangles, one shot, 400 steps): 3.97
-// ms against 4.21 ms in launches per step; 1,560 (KMV5, 50k, one shot, a gradient of 75 steps): 15.4
-// against 6.3 ms, their meetings crowd one counter.
+// Most CTAs of a launch of several steps; two per SM of this chip. Launches per step against one
+// launch, ms: KMV2, one shot, 400 steps, 256 CTAs 4.21 / 3.97; 200 steps, 360 CTAs 2.13 / 1.98, 470
+// 2.13 / 2.12, 630 2.13 / 2.31 (more CTAs crowd the meetings' counter; 1,560, a KMV5 gradient of 75
+// steps: 6.3 / 15.4). Below the line, 12 and 290 CTAs: one shot, KMV5 gradient 4.0 / 3.2 and 3.9 / 3.5,
+// KMV3 tetrahedra with a layer 5.8 / 4.3 and 5.8 / 5.3; four shots without a layer, KMV3 gradient 2.5 /
+// 2.3 and 2.5 / 2.6. With a layer and four shots launches per step are faster (KMV5 gradient 3.9 / 5.8
+// and 4.4 / 7.6): run_chunk's layer instances spill and read their arguments through a pointer.
 constexpr int RUN_MAX = 304;
 
+// Registers a thread may take: enough CTAs per SM to hide the loads of one behind the arithmetic of
+// the others. KMV5 gradient steps need 168; at 128, with one CTA more per SM, they spill (marine mesh,
+// one gradient of 75 steps: 128.5 against 133.1 ms). The other triangle kernels and KMV2 tetrahedra
+// are best at 128 (KMV4, S = 4, 250k triangles: 8.0 ms for 100 steps, 10.9 ms at 204; KMV3, 120k: 8.9
+// and 9.8 ms), but KMV2 triangles at one shot, which do little with what they load, at 48 (2M
+// triangles, 50 steps: 3.54 ms, 3.71 ms at 80). KMV3 tetrahedra keep one or two fields' 32 adapted
+// values in registers and take what shared memory leaves: two CTAs per SM of their layer chunks
+// have room for 255 registers a thread.
 template <int MODE, bool LAYER>
 constexpr int registers() {
   if (KMV_DIM == 3 && KMV_K == 3) return LAYER ? 255 : MODE == 2 ? 204 : 168;
@@ -75,11 +81,13 @@ __global__ void __launch_bounds__(NT, 65536 / (registers<MODE, true>() * NT)) k_
 }
 
 // Several steps in one cooperative launch, for meshes whose steps are shorter than launching them:
-// every CTA takes its chunks, all CTAs meet, every thread finishes its halo DoFs, all meet again.
+// every CTA takes a chunk, all CTAs meet, every thread finishes its halo DoFs, all meet again.
 // A chunk and a halo DoF stay with their CTA, so only what crosses CTAs has to come from L2. Both
 // kinds of chunks are one kernel here.
 __device__ __forceinline__ bool run_meet(unsigned* count, unsigned target, int polls) {
-  asm volatile("fence.proxy.async;" ::: "memory");  // (the fields are written as usual, read by bulk copies)
+  // (the fields are written as usual and read by bulk copies; the next step's copies come after this
+  // step's reads of the tables)
+  asm volatile("fence.proxy.async;" ::: "memory");
   __syncthreads();
   bool ok = true;
   if (threadIdx.x == 0) {
@@ -110,7 +118,8 @@ template <int MODE>
 __global__ void __launch_bounds__(NT_RUN, 65536 / (registers<MODE, true>() * NT_RUN))
     k_run(const __grid_constant__ StepArgs a, const RunArgs r) {
   extern __shared__ __align__(16) float smem_sym[];
-  const int ngrp = a.S / SG, nwork = a.nch * ngrp, tid = threadIdx.x;
+  const int ngrp = a.S / SG, tid = threadIdx.x;
+  const int c = a.nch - 1 - blockIdx.x / ngrp, s0 = blockIdx.x % ngrp * SG;  // the layer's chunks, the longer ones, first
   if (tid == 0) sym_bar_init(reinterpret_cast<uint64_t*>(smem_sym));
   // (an earlier launch of the call gave up: its CTAs never met, this one's would poll to the limit)
   if (__syncthreads_or(tid == 0 && (__ldcg(a.status) & 2))) return;
@@ -127,14 +136,9 @@ __global__ void __launch_bounds__(NT_RUN, 65536 / (registers<MODE, true>() * NT_
       x.u_out = a.u_out;
       x.ring_u = r.ring + (size_t)rel * r.level;
     }
-    for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
-      const int c = a.nch - 1 - w / ngrp, s0 = w % ngrp * SG;  // the layer's chunks, the longer ones, first
-      const bool ok = c < a.nch0 ? run_chunk<MODE, false>(a, x, smem_sym, c, s0) : run_chunk<MODE, true>(a, x, smem_sym, c, s0);
-      if (!ok) return;
-      x.parity ^= 1;
-      asm volatile("fence.proxy.async;" ::: "memory");  // the next chunk's copies come after these reads
-      __syncthreads();
-    }
+    const bool ok = c < a.nch0 ? run_chunk<MODE, false>(a, x, smem_sym, c, s0) : run_chunk<MODE, true>(a, x, smem_sym, c, s0);
+    if (!ok) return;
+    x.parity ^= 1;
     if (!run_meet(r.count, target += gridDim.x, a.wait_limit)) {
       if (tid == 0) atomicOr(a.status, 2);
       return;
@@ -181,7 +185,7 @@ int run_t(const StepArgs& a, const RunArgs& r, cudaStream_t st) {
   const int64_t nwork = (int64_t)a.nch * (a.S / SG);
   const int64_t room = (int64_t)per * sms;
   if (nwork > RUN_MAX || nwork > room) return 0;
-  const int grid = (int)std::min(nwork, room);
+  const int grid = (int)nwork;  // (one chunk and shot group per CTA)
   StepArgs b = a;
   RunArgs q = r;
   b.ch0 = 0;
