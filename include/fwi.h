@@ -325,9 +325,9 @@ int fwi_last_error(char* buf, int len);
 
 /* Measurement aid (no counterpart in the paper): the FP32 FMA throughput of the current
  * device in TFLOP/s, from a kernel of independent packed FP32x2 FMA chains on every SM (best
- * of five timed launches, CUDA events), and its SM count. The element kernels, at 4 d n^2
- * flops per element and shot, are bound by this rate; it is the denominator of their roofline
- * fraction. Allocates and frees a 16 KiB buffer. */
+ * of five timed launches, CUDA events), and its SM count: the denominator of the element kernels'
+ * arithmetic fraction (they carry out a quarter to a third of a dense contraction's 4 d n^2 flops per
+ * element and shot). Allocates and frees a 16 KiB buffer. */
 int fwi_fp32_peak(double* tflops, int* sm_count);
 
 /* Kernel launches the library issued on this thread since the last call (counter read and

@@ -17,9 +17,9 @@
 // Owned DoFs are read and written by this CTA only; halo DoFs are only read here.
 //
 // What bounds it: instruction issue, then latency. KMV5 triangles, 4 shots (graded grid of 348k
-// triangles, forward step): chunks without layer elements (60 %) 109 us, 3,180 instructions per warp
-// of which 1,720 on the FMA pipes, issue slots 64 % full, 279 MB of DRAM traffic (38 % of the copy
-// rate); layer chunks 184 us at 39 % (three CTAs per SM for their shared memory). The dense form
+// triangles, forward step): chunks without layer elements (60 %) 108 us, 3,200 instructions per warp
+// of which 1,720 on the FMA pipes, issue slots 65 % full, 279 MB of DRAM traffic (38 % of the copy
+// rate); layer chunks 181 us at 40 % (three CTAs per SM for their shared memory). The dense form
 // with rows of Dhat from shared memory took 384 and 225 us on a mesh of this size. KMV2, one shot,
 // 2M triangles: 71 us per step with the halo kernel's 8, 210 MB; KMV4, 4 shots, 250k: 57 us, 163 MB.
 // Chunk sizes (sym_pe): at 32 triangles the KMV2 step spent 115 us, its chunks' fixed chain of loads
